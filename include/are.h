@@ -252,13 +252,16 @@ typedef struct {
                                 terms behind their column mask, 32 bytes where the layer
                                 holds few entries per catalog event, else 64, or in FP32
                                 the dense row of up to 16 ELTs; are_layer_rows tells which;
-                                FP64 with exact trial sums), 3 (FP64) staged rows of an
+                                FP64 with exact trial sums; where few of the layer's events
+                                have an occurrence loss, only their rows, found by one bit per
+                                catalog event), 3 (FP64) staged rows of an
                                 FP32 screen with the marked entries read from the FP64
                                 table */
     int32_t rows_in_flight;  /* register rows and persistent kernel: groups of 32 events
-                                per batch, 1 or 2; staged kernel: events per lane per
-                                batch, 1 or 2; 0 (in a loaded tuning file): the
-                                kernel's default */
+                                per batch, 1 or 2 (register rows: every occurrence's row is
+                                read); staged kernel: events per lane per batch, 1 or 2; 0:
+                                the kernel's default (register rows: marked events only,
+                                where the layer calls for it) */
     int32_t trials_per_item; /* trials per work item (persistent kernel) */
     int32_t blocks_per_sm;   /* 0 = as many as fit */
     double ms;               /* measured time of one pass */
@@ -271,8 +274,10 @@ typedef struct {
  * and keep the fastest for this kind of work: precision, YET layout, widest
  * table row, mean events per trial and one layer vs several.  Later
  * are_simulate and are_simulate_portfolio calls of that kind use it.
- * Untuned work runs the register-rows kernel with one group of 32 events per
- * batch over 32-byte FP32 rows and two over wider rows and FP64 rows.
+ * Untuned work runs the register-rows kernel in its default form: over the
+ * marked events where the layer's share of them is small, else over every
+ * row, with one group of 32 events per batch over 32-byte FP32 rows and two
+ * over wider rows and FP64 rows.
  * *best (may be NULL) receives the winner.  Runs on `stream` and waits. */
 ARE_API are_status are_autotune(are_ctx *ctx, const int32_t *layers, int32_t n_layers,
                                 int32_t yet, are_precision precision, void *stream,

@@ -209,6 +209,12 @@ void free_packed(are_ctx *ctx, Packed &p)
     p = Packed{};
 }
 
+void free_marks(are_ctx *ctx, Marks &m)
+{
+    dfree(ctx, m.map.d, sizeof(uint32_t) * (size_t)m.map.words);
+    m = Marks{};
+}
+
 void free_folded(are_ctx *ctx, Folded &f)
 {
     dfree(ctx, f.d, f.bytes);
@@ -284,9 +290,6 @@ Compact &build_compact(are_ctx *ctx, Layer &L, int32_t catalog, cudaStream_t s)
     return c;
 }
 
-// The tables an analysis of layer L in `precision` reads, built if missing.
-void ensure_tables(are_ctx *ctx, Layer &L, const Yet &y, are_precision precision, cudaStream_t s,
-                   bool rebuild);
 TuneEntry tuned(are_ctx *ctx, are_precision p, const Yet &y, int jp, bool multi);
 
 // Build (or rebuild) the layer's table for `catalog` in fp32 or fp64.
@@ -334,19 +337,17 @@ void size_packed(are_ctx *ctx, Layer &L, Packed &p, int32_t catalog, int rw, siz
     }
 }
 
-int64_t layer_entries(are_ctx *ctx, const Layer &L)
+int64_t layer_entries(const Layer &L)
 {
-    int64_t entries = 0;
-    for (int32_t h : L.elts) entries += ctx->elts.at(h).n;
-    ARE_CHECK(entries < (1LL << 32), ARE_EINVAL, "a layer's ELTs hold 2^32 or more entries");
-    return entries;
+    ARE_CHECK(L.entries < (1LL << 32), ARE_EINVAL, "a layer's ELTs hold 2^32 or more entries");
+    return L.entries;
 }
 
 // Words per packed row of the layer over a catalog of `catalog` events (0:
 // the dense FP32 row), from its ELT entries per catalog event.
-int row_words(are_ctx *ctx, const Layer &L, int32_t catalog, bool fp32)
+int row_words(const Layer &L, int32_t catalog, bool fp32)
 {
-    const double tpe = catalog > 0 ? (double)layer_entries(ctx, L) / (double)catalog : 0.0;
+    const double tpe = catalog > 0 ? (double)layer_entries(L) / (double)catalog : 0.0;
     return packed_row_words((int)L.elts.size(), tpe, fp32);
 }
 
@@ -355,9 +356,9 @@ int row_words(are_ctx *ctx, const Layer &L, int32_t catalog, bool fp32)
 Packed &build_packed64(are_ctx *ctx, Layer &L, int32_t catalog, cudaStream_t s)
 {
     Packed &p = L.p64;
-    const int rw = row_words(ctx, L, catalog, false);
+    const int rw = row_words(L, catalog, false);
     size_packed(ctx, L, p, catalog, rw, rw * sizeof(unsigned long long),
-                sizeof(double) * (size_t)layer_entries(ctx, L));
+                sizeof(double) * (size_t)layer_entries(L));
     const ScatterArgs a = scatter_args(ctx, L, catalog, table_jp((int)L.elts.size(), false));
     ctx->launches += launch_pack64_direct(a, catalog, rw, static_cast<unsigned long long *>(p.rows()),
                                           static_cast<double *>(p.ovf()), p.used(), s);
@@ -370,7 +371,7 @@ Packed &build_packed32_direct(are_ctx *ctx, Layer &L, int32_t catalog, int pw, c
 {
     Packed &p = L.p32;
     const ScatterArgs a = scatter_args(ctx, L, catalog, table_jp((int)L.elts.size(), true));
-    size_packed(ctx, L, p, catalog, pw, pw * sizeof(float), sizeof(float) * (size_t)layer_entries(ctx, L));
+    size_packed(ctx, L, p, catalog, pw, pw * sizeof(float), sizeof(float) * (size_t)layer_entries(L));
     ctx->launches += launch_pack32_direct(a, catalog, pw, static_cast<uint32_t *>(p.rows()),
                                           static_cast<float *>(p.ovf()), p.used(), s);
     return p;
@@ -385,12 +386,20 @@ void ensure_aux(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, int kernel, 
     if (!fp32 && kernel == 3 && (fresh || !L.t32u.d || L.t32u.catalog != catalog)) build_screen(ctx, L, catalog, s);
 }
 
+void fill_terms(const Layer &L, TermsF32 &t32, TermsF64 &t64)
+{
+    t64.occ_r = L.terms.occ_ret;
+    t64.occ_l = L.terms.occ_lim;
+    t32.occ_r = (float)L.terms.occ_ret;
+    t32.occ_l = (float)L.terms.occ_lim;
+}
+
 // The packed rows a register-rows analysis (kernel 2) of the layer reads,
 // built if missing (or always, with rebuild); false where it reads the
 // dense FP32 table instead.
 bool ensure_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, cudaStream_t s, bool rebuild)
 {
-    const int w = row_words(ctx, L, catalog, fp32);
+    const int w = row_words(L, catalog, fp32);
     if (!w) return false;
     Packed &p = fp32 ? L.p32 : L.p64;
     if (rebuild || !p.d || p.catalog != catalog || p.rw != w) {
@@ -402,6 +411,128 @@ bool ensure_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, cudaStrea
     return true;
 }
 
+// An upper bound of the layer's occurrence losses: min(OccL, the sum over
+// its ELTs of the largest term), the largest term being the term of the
+// ELT's largest loss (a term is non-decreasing in the loss), with a margin
+// for the rounding of that sum.
+double loss_bound(are_ctx *ctx, const Layer &L)
+{
+    double g = 0.0;
+    for (int32_t h : L.elts) {
+        const Elt &e = ctx->elts.at(h);
+        if (e.n == 0) continue;
+        double x = e.terms.fx * e.max_loss - e.terms.deductible;
+        x = x > 0.0 ? x : 0.0;
+        x = x > e.terms.limit ? e.terms.limit : x;
+        g += e.terms.share * x;
+    }
+    return std::min(g, L.terms.occ_lim) * (1.0 + 1e-9);
+}
+
+// An estimate of the share of the catalog's events that have an occurrence
+// loss in the layer: an event with m terms is taken to need one above OccR /
+// m, m the mean number of terms of the events that have any (entries fall on
+// events independently).  From the ELTs' counts of losses by quarter octave.
+double marked_share(are_ctx *ctx, const Layer &L, int32_t catalog)
+{
+    if (L.marked_catalog == catalog) return L.marked;
+    const double per_event = (double)layer_entries(L) / (double)catalog;
+    const double m = per_event > 0.0 ? per_event / -std::expm1(-per_event) : 1.0;
+    double above = 0.0;
+    for (int32_t h : L.elts) {
+        const Elt &e = ctx->elts.at(h);
+        const double need = L.terms.occ_ret / m;   // of a term: share * (fx * x - D), at most share * Lim
+        if (!(e.terms.share * e.terms.limit > 0.0) || e.terms.share * e.terms.limit < need) continue;
+        const double x = (need / e.terms.share + e.terms.deductible) / e.terms.fx;   // the loss that gives it
+        uint64_t bits;
+        std::memcpy(&bits, &x, sizeof bits);
+        const double at = std::isfinite(x) ? (double)bits / (double)(1ull << 50) - e.bin0 : 1e300;
+        for (size_t i = 0; i < e.bins.size(); ++i)
+            above += e.bins[i] * std::min(1.0, std::max(0.0, (double)(i + 1) - at));
+    }
+    L.marked = -std::expm1(-above / (double)catalog);
+    L.marked_catalog = catalog;
+    return L.marked;
+}
+
+// Whether the register-rows analysis of the layer over a YET looks its
+// occurrences up in marks first (marked.cuh).  It depends on the layer, the
+// YET and the precision alone, so that every split of the trials, the
+// streamed analysis and the server form a trial's sum alike.
+//  * The marks of the catalog fit a block's shared memory.
+//  * FP32: losses far below the type's largest value (the exact sums hold no
+//    infinity).
+//  * Trials long enough for a pass: with 16 ELTs of 2% of a 1M-event catalog
+//    and Kahan sums, 40 events a trial take 0.78 of the every-row rate, 120
+//    events 1.27, 250 events 2.1 (FP64 1.0, 1.7, 2.6); the FP32 kernel with
+//    FP64 sums is slow on short trials and gains at every length (20: 1.37).
+//  * Few enough rows to read: at 1000 events a trial Kahan sums gain 1.82
+//    where 0.27 of the events are marked, break even at 0.55 and lose (0.87)
+//    at 0.7; the FP32 kernel with FP64 sums gains 2.5, 1.4 and 1.2 there,
+//    1.08 at 0.8 and loses (0.52) at 0.96; FP64 2.3, 1.8, 1.5 and 1.3, and
+//    0.87 at 0.96.
+bool uses_marks(are_ctx *ctx, const Layer &L, const Yet &y, are_precision p)
+{
+    if (y.catalog <= 0 || mark_shape(y.catalog).words == 0) return false;
+    if (p != ARE_FP64 && !(L.bound < 1e37)) return false;
+    const double mean = y.n_trials ? (double)y.n_events / (double)y.n_trials : 0.0;
+    const double share = marked_share(ctx, L, y.catalog);
+    switch (p) {
+    case ARE_FP32_KAHAN: return mean >= 80.0 && share <= 0.5;
+    case ARE_FP32_FP64AGG: return share <= 0.75;
+    default: return mean >= 50.0 && share <= 0.85;
+    }
+}
+
+// The rows of a register-rows analysis -- packed, or the dense FP32 table --
+// and, with `marked`, their marks where the layer's analysis uses them.
+void ensure_rows(are_ctx *ctx, Layer &L, const Yet &y, are_precision p, bool marked, cudaStream_t s, bool rebuild)
+{
+    const bool fp32 = p != ARE_FP64;
+    const int32_t catalog = y.catalog;
+    const bool packed = ensure_packed(ctx, L, catalog, fp32, s, rebuild);
+    if (!packed && (rebuild || !L.t32.d || L.t32.catalog != catalog)) build_table(ctx, L, catalog, fp32, s);
+    if (!marked || !uses_marks(ctx, L, y, p)) return;
+    Marks &m = fp32 ? L.m32 : L.m64;
+    if (!rebuild && m.map.d && m.catalog == catalog) return;
+    if (m.map.d && m.catalog != catalog) free_marks(ctx, m);
+    if (!m.map.d) {
+        const MarkMap shape = mark_shape(catalog);
+        uint32_t *d = (uint32_t *)dalloc(ctx, sizeof(uint32_t) * (size_t)shape.words);
+        ++L.generation;
+        m.map = shape;
+        m.map.d = d;
+        m.catalog = catalog;
+    }
+    TermsF32 t32;
+    TermsF64 t64;
+    fill_terms(L, t32, t64);
+    const ScatterArgs a = scatter_args(ctx, L, catalog, 0);
+    if (fp32)
+        ctx->launches += packed ? launch_marks32(a, m.map, L.p32.rows(), L.p32.ovf(), true, L.p32.rw, t32, s)
+                                : launch_marks32(a, m.map, L.t32.d, nullptr, false, L.t32.jp, t32, s);
+    else
+        ctx->launches += launch_marks64(a, m.map, L.p64.rows(), L.p64.ovf(), L.p64.rw, t64, s);
+}
+
+// The tables that a kernel choice reads for a layer in the direct layout,
+// built if missing (or always, with rebuild).
+void ensure_direct(are_ctx *ctx, Layer &L, const Yet &y, are_precision p, const TuneEntry &te, cudaStream_t s,
+                   bool rebuild)
+{
+    const bool fp32 = p != ARE_FP64;
+    const int32_t catalog = y.catalog;
+    if (te.kernel == 2) {   // a dense table only where the rows are dense
+        ensure_rows(ctx, L, y, p, te.cfg.rows_in_flight == 0, s, rebuild);
+        return;
+    }
+    const Table &t = fp32 ? L.t32 : L.t64;
+    const bool fresh = rebuild || !t.d || t.catalog != catalog;
+    if (fresh) build_table(ctx, L, catalog, fp32, s);
+    ensure_aux(ctx, L, catalog, fp32, te.kernel, fresh, s);
+}
+
+// The tables an analysis of layer L in `precision` reads.
 void ensure_tables(are_ctx *ctx, Layer &L, const Yet &y, are_precision precision, cudaStream_t s,
                    bool rebuild)
 {
@@ -412,13 +543,7 @@ void ensure_tables(are_ctx *ctx, Layer &L, const Yet &y, are_precision precision
         return;
     }
     const int jp = table_jp((int)L.elts.size(), fp32);
-    const int kernel = tuned(ctx, precision, y, jp, false).kernel;
-    // packed rows straight from the ELT entries; a dense table only when a kernel needs one
-    if (kernel == 2 && ensure_packed(ctx, L, catalog, fp32, s, rebuild)) return;
-    const Table &t = fp32 ? L.t32 : L.t64;
-    const bool fresh = rebuild || !t.d || t.catalog != catalog;
-    if (fresh) build_table(ctx, L, catalog, fp32, s);
-    ensure_aux(ctx, L, catalog, fp32, kernel, fresh, s);
+    ensure_direct(ctx, L, y, precision, tuned(ctx, precision, y, jp, false), s, rebuild);
 }
 
 Layer &layer_of(are_ctx *ctx, int32_t h)
@@ -438,14 +563,6 @@ void check_precision(are_precision p)
 {
     ARE_CHECK(p == ARE_FP64 || p == ARE_FP32_KAHAN || p == ARE_FP32_FP64AGG, ARE_EINVAL,
               "unknown precision " + std::to_string((int)p));
-}
-
-void fill_terms(const Layer &L, TermsF32 &t32, TermsF64 &t64)
-{
-    t64.occ_r = L.terms.occ_ret;
-    t64.occ_l = L.terms.occ_lim;
-    t32.occ_r = (float)L.terms.occ_ret;
-    t32.occ_l = (float)L.terms.occ_lim;
 }
 
 // (Re)build the layer's folded table for `catalog` from its ELTs.
@@ -501,23 +618,11 @@ ItemWork item_work(const Yet &y, int64_t trial_begin, int64_t n_trials, const It
     return w;
 }
 
-// The fixed-point scale of the FP64 register-rows kernel's exact running
-// sums: s = 125 - floor(log2(B)) for an upper bound B of every occurrence
-// loss of the layer -- min(OccL, the sum over its ELTs of the largest term),
-// the largest term being the term of the ELT's largest loss (a term is
-// non-decreasing in the loss), with a margin for the rounding of that sum.
-int fixed_scale(are_ctx *ctx, const Layer &L)
+// The fixed-point scale of the exact running sums: s = 125 - floor(log2(B))
+// for the upper bound B of the layer's occurrence losses.
+int fixed_scale(const Layer &L)
 {
-    double g = 0.0;
-    for (int32_t h : L.elts) {
-        const Elt &e = ctx->elts.at(h);
-        if (e.n == 0) continue;
-        double x = e.terms.fx * e.max_loss - e.terms.deductible;
-        x = x > 0.0 ? x : 0.0;
-        x = x > e.terms.limit ? e.terms.limit : x;
-        g += e.terms.share * x;
-    }
-    double b = std::min(g, L.terms.occ_lim) * (1.0 + 1e-9);
+    const double b = L.bound;
     if (!(b > 0.0)) return 0;
     int ex = 0;
     std::frexp(b, &ex);          // b = f * 2^ex, 0.5 <= f < 1: floor(log2 b) = ex - 1
@@ -557,11 +662,16 @@ int run_single(are_ctx *ctx, const Layer &L, const Yet &y, int64_t trial_begin, 
     TermsF64 t64;
     fill_terms(L, t32, t64);
     a.n_elts = (int32_t)L.elts.size();
+    const Marks &m = fp32 ? L.m32 : L.m64;   // built where this choice uses them (ensure_rows)
+    const bool marked = !compact && te.kernel == 2 && te.cfg.rows_in_flight == 0 && m.map.d &&
+                        m.catalog == y.catalog && uses_marks(ctx, L, y, precision);
     if (fp32 && !compact && te.kernel == 2 && L.p32.d && L.p32.catalog == y.catalog &&
-        L.p32.rw == row_words(ctx, L, y.catalog, true)) {
+        L.p32.rw == row_words(L, y.catalog, true)) {
         a.table = L.p32.rows();   // register rows over the packed FP32 rows
         a.table2 = L.p32.ovf();
         a.kernel = 5;
+        if (marked)
+            return launch_marked32(a, m.map, precision, true, L.p32.rw, t32, fixed_scale(L), ctx->num_sms, s);
         return launch_simulate(a, precision, L.p32.rw, &t32, &t64, ctx->num_sms, s);
     }
     if (compact) {   // the staged kernel, through the row index
@@ -574,7 +684,8 @@ int run_single(are_ctx *ctx, const Layer &L, const Yet &y, int64_t trial_begin, 
         if (te.kernel == 2 && L.p64.d && L.p64.catalog == y.catalog) {   // packed FP64 rows
             a.table = L.p64.rows();
             a.table2 = L.p64.ovf();
-            return launch_rows64(a, L.p64.rw, t64, fixed_scale(ctx, L), ctx->num_sms, s);
+            if (marked) return launch_marked64(a, m.map, L.p64.rw, t64, fixed_scale(L), ctx->num_sms, s);
+            return launch_rows64(a, L.p64.rw, t64, fixed_scale(L), ctx->num_sms, s);
         }
         if (te.kernel == 3 && L.t32u.d && L.t32u.catalog == y.catalog) {   // the FP32 screen
             a.table2 = L.t32u.d;
@@ -583,6 +694,7 @@ int run_single(are_ctx *ctx, const Layer &L, const Yet &y, int64_t trial_begin, 
         }
         return launch_staged64(a, t.jp, t64, ctx->num_sms, s);   // (or an aux table not built)
     }
+    if (marked) return launch_marked32(a, m.map, precision, false, t.jp, t32, fixed_scale(L), ctx->num_sms, s);
     return launch_simulate(a, precision, t.jp, &t32, &t64, ctx->num_sms, s);
 }
 
@@ -724,18 +836,12 @@ void check_multi_args(are_ctx *ctx, const int32_t *layers, int32_t n_layers, con
     }
 }
 
-// Every layer's table and the tables beside it that `kernel` reads (0: none).
-void ensure_tables(are_ctx *ctx, const int32_t *layers, int32_t n_layers, const Yet &y, bool fp32,
-                   cudaStream_t s, int kernel = 0)
+// The tables of several layers that a kernel choice reads (the direct
+// layout), built if missing.
+void ensure_tables(are_ctx *ctx, const int32_t *layers, int32_t n_layers, const Yet &y, are_precision p,
+                   cudaStream_t s, const TuneEntry &te)
 {
-    for (int32_t i = 0; i < n_layers; ++i) {
-        Layer &L = layer_of(ctx, layers[i]);
-        if (kernel == 2 && ensure_packed(ctx, L, y.catalog, fp32, s, false)) continue;   // packed rows
-        const Table &t = fp32 ? L.t32 : L.t64;
-        const bool fresh = !t.d || t.catalog != y.catalog;
-        if (fresh) build_table(ctx, L, y.catalog, fp32, s);
-        ensure_aux(ctx, L, y.catalog, fp32, kernel, fresh, s);
-    }
+    for (int32_t i = 0; i < n_layers; ++i) ensure_direct(ctx, layer_of(ctx, layers[i]), y, p, te, s, false);
 }
 
 int max_width(are_ctx *ctx, const int32_t *layers, int32_t n_layers, bool fp32)
@@ -820,6 +926,8 @@ are_status are_destroy(are_ctx *ctx)
             free_table(ctx, kv.second.t32u);
             free_packed(ctx, kv.second.p64);
             free_packed(ctx, kv.second.p32);
+            free_marks(ctx, kv.second.m32);
+            free_marks(ctx, kv.second.m64);
             free_folded(ctx, kv.second.fold);
             free_compact(ctx, kv.second.comp);
         }
@@ -987,6 +1095,17 @@ are_status are_load_elt(are_ctx *ctx, int32_t n_entries, const int32_t *event_id
         }
         ARE_CHECK(!dup, ARE_EINVAL, "duplicate event id within one ELT");
         Elt e;
+        if (n_entries > 0) {   // the losses by quarter octave
+            auto bin = [](double x) {
+                uint64_t b;
+                std::memcpy(&b, &x, sizeof b);
+                return (int32_t)(b >> 50 & 0x1fff);
+            };
+            const double least = *std::min_element(loss.begin(), loss.end());
+            e.bin0 = bin(least);
+            e.bins.assign((size_t)(bin(max_loss) - e.bin0 + 1), 0u);
+            for (double x : loss) ++e.bins[(size_t)(bin(x) - e.bin0)];
+        }
         e.n = n_entries;
         e.max_id = max_id;
         e.max_loss = max_loss;
@@ -1030,6 +1149,8 @@ are_status are_define_layer(are_ctx *ctx, const int32_t *elt_handles, int32_t n_
             L.elts.push_back(h);
         }
         L.terms = positive_zeros(t);
+        for (int32_t h : L.elts) L.entries += ctx->elts[h].n;
+        L.bound = loss_bound(ctx, L);
         for (int32_t h : L.elts) ctx->elts[h].users++;
         const int32_t h = ctx->next_handle++;
         ctx->layers[h] = L;
@@ -1072,6 +1193,8 @@ are_status are_free_layer(are_ctx *ctx, int32_t h)
         free_table(ctx, L.t32u);
         free_packed(ctx, L.p64);
         free_packed(ctx, L.p32);
+        free_marks(ctx, L.m32);
+        free_marks(ctx, L.m64);
         free_folded(ctx, L.fold);
         free_compact(ctx, L.comp);
         for (int32_t e : L.elts) ctx->elts[e].users--;
@@ -1154,13 +1277,13 @@ are_status are_layer_rows(are_ctx *ctx, int32_t layer, int32_t yet, are_precisio
         const int k = kernel >= 0 ? kernel : tuned(ctx, precision, y, table_jp(J, fp32), false).kernel;
         int rb = table_jp(J, fp32) * (fp32 ? 4 : 8), pk = 0;
         if (fp32 && L.layout != ARE_LAYOUT_COMPACT && k == 2) {
-            const int pw = row_words(ctx, L, y.catalog, true);
+            const int pw = row_words(L, y.catalog, true);
             if (pw) {
                 rb = pw * 4;
                 pk = 1;
             }
         } else if (!fp32 && k == 2) {
-            rb = row_words(ctx, L, y.catalog, false) * 8;
+            rb = row_words(L, y.catalog, false) * 8;
             pk = 1;
         } else if (!fp32 && k == 3) {
             rb = table_jp(J, true) * 4;   // the screen's rows (and the marked FP64 entries)
@@ -1532,10 +1655,10 @@ are_status are_simulate_occurrences(are_ctx *ctx, int32_t layer, int32_t yet, in
             const Packed &p = fp32 ? L.p32 : L.p64;
             a.table = p.rows();
             a.table2 = p.ovf();
-            ctx->launches += launch_rows_occ(a, fp32 ? 1 : 0, p.rw, t32, t64, fixed_scale(ctx, L), ctx->num_sms,
+            ctx->launches += launch_rows_occ(a, fp32 ? 1 : 0, p.rw, t32, t64, fixed_scale(L), ctx->num_sms,
                                              cs.s);
         } else {         // dense FP32 rows
-            ctx->launches += launch_rows_occ(a, 2, t.jp, t32, t64, fixed_scale(ctx, L), ctx->num_sms, cs.s);
+            ctx->launches += launch_rows_occ(a, 2, t.jp, t32, t64, fixed_scale(L), ctx->num_sms, cs.s);
         }
         cs.finish();
     });
@@ -1626,8 +1749,8 @@ are_status are_simulate_portfolio(are_ctx *ctx, const int32_t *layers, int32_t n
         check_multi_args(ctx, layers, n_layers, y, trial_begin, n_trials, ylts);
         CallStream cs(ctx, stream);
         const bool fp32 = precision != ARE_FP64;
-        const int k = tuned(ctx, precision, y, max_width(ctx, layers, n_layers, fp32), n_layers > 1).kernel;
-        ensure_tables(ctx, layers, n_layers, y, fp32, cs.s, k);
+        ensure_tables(ctx, layers, n_layers, y, precision, cs.s,
+                      tuned(ctx, precision, y, max_width(ctx, layers, n_layers, fp32), n_layers > 1));
         const std::vector<int32_t> lv(layers, layers + n_layers);
         const std::vector<double *> yv(ylts, ylts + n_layers);
         std::vector<uint64_t> gens;
@@ -1772,20 +1895,25 @@ are_status are_autotune(are_ctx *ctx, const int32_t *layers, int32_t n_layers, i
         check_multi_args(ctx, layers, n_layers, y, 0, y.n_trials, nullptr);
         CallStream cs(ctx, stream);
         const bool fp32 = precision != ARE_FP64;
-        ensure_tables(ctx, layers, n_layers, y, fp32, cs.s, 2);              // packed rows
-        ensure_tables(ctx, layers, n_layers, y, fp32, cs.s, 1);              // dense rows
-        if (!fp32) ensure_tables(ctx, layers, n_layers, y, fp32, cs.s, 3);  // FP64: the screen
+        for (int k : {2, 1, 3}) {   // register rows and their marks, dense rows, (FP64) the screen
+            TuneEntry e;
+            e.kernel = k;
+            e.cfg.rows_in_flight = 0;
+            if (k != 3 || !fp32) ensure_tables(ctx, layers, n_layers, y, precision, cs.s, e);
+        }
         const bool multi = n_layers > 1;
         const int jp = max_width(ctx, layers, n_layers, fp32);
         const std::string key = tune_key(precision, y, jp, multi);
         std::vector<TuneEntry> cands;
+        bool marks = false;                   // some layer's occurrences can be looked up in marks first
+        for (int32_t i = 0; i < n_layers; ++i) marks |= uses_marks(ctx, layer_of(ctx, layers[i]), y, precision);
+        for (int u : {0, 1, 2}) {   // register rows: the default, or every row read, one or two groups of 32 events
+            TuneEntry e;
+            e.kernel = 2;
+            e.cfg.rows_in_flight = u;
+            if (u || marks) cands.push_back(e);
+        }
         if (fp32) {
-            for (int u : {1, 2}) {            // register rows, one or two groups of 32 events
-                TuneEntry e;
-                e.kernel = 2;
-                e.cfg.rows_in_flight = u;
-                cands.push_back(e);
-            }
             for (int epl : {1, 2}) {          // staged rows, one or two events per lane
                 TuneEntry e;
                 e.kernel = 1;
@@ -1801,12 +1929,6 @@ are_status are_autotune(are_ctx *ctx, const int32_t *layers, int32_t n_layers, i
                     cands.push_back(e);
                 }
         } else {
-            for (int u : {1, 2}) {      // register rows over the packed FP64 rows
-                TuneEntry e;
-                e.kernel = 2;
-                e.cfg.rows_in_flight = u;
-                cands.push_back(e);
-            }
             for (int k : {1, 3}) {      // staged FP64 rows, staged screen rows
                 TuneEntry e;
                 e.kernel = k;

@@ -67,6 +67,8 @@ struct Elt {
     int32_t n = 0;
     int32_t max_id = -1;
     double max_loss = 0.0;         // largest loss of the ELT
+    int32_t bin0 = 0;              // its losses counted by quarter octaves: bins[i] of those whose
+    std::vector<uint32_t> bins;    // bit pattern >> 50 is bin0 + i
     int32_t *d_ids = nullptr;
     double *d_loss = nullptr;
     are_fin_terms terms{};
@@ -144,6 +146,33 @@ struct Packed {
     void *ovf() const { return static_cast<char *>(d) + rows_bytes + 256; }
 };
 
+// The marks of one layer's register rows: one bit per catalog event, set
+// where the event's occurrence loss is not 0 (marked.cuh).  A catalog of more
+// than kMaxMarkWords * 32 events folds: event e >= bits has the bit of e - bits.
+constexpr int32_t kMaxMarkWords = 41600;   // what a block's shared memory holds beside its lists (marked.cuh)
+struct MarkMap {
+    uint32_t *d = nullptr;
+    int32_t words = 0;       // a multiple of 4
+    uint32_t bits = 0;       // 32 x words
+    bool fold = false;
+};
+struct Marks {
+    int32_t catalog = -1;
+    MarkMap map;
+};
+// The shape of a catalog's marks; words 0 where more than two events would
+// share a bit.
+inline MarkMap mark_shape(int32_t catalog)
+{
+    MarkMap m;
+    const int64_t words = ((int64_t)catalog + 127) / 128 * 4;
+    if (words > 2 * (int64_t)kMaxMarkWords) return m;
+    m.fold = words > kMaxMarkWords;
+    m.words = m.fold ? kMaxMarkWords : (int32_t)words;
+    m.bits = (uint32_t)m.words * 32u;
+    return m;
+}
+
 struct Layer {
     std::vector<int32_t> elts;
     are_layer_terms terms{};
@@ -151,9 +180,14 @@ struct Layer {
     Table t32u;              // FP32 screen of t64: its values rounded up
     Packed p64;              // packed FP64 rows of t64
     Packed p32;              // packed FP32 rows of t32 (layers of more than 8 ELTs)
+    Marks m32, m64;          // marks of the FP32 and FP64 register rows
     Folded fold;
     int layout = 0;          // ARE_LAYOUT_DIRECT or ARE_LAYOUT_COMPACT (FP32 analysis)
     Compact comp;
+    int64_t entries = 0;       // entries of its ELTs
+    double bound = 0.0;        // upper bound of its occurrence losses
+    mutable int32_t marked_catalog = -1;     // the catalog of the estimate below
+    mutable double marked = 0.0;             // estimated share of the catalog's events with an occurrence loss
     uint64_t generation = 0;   // bumped whenever a table is (re)allocated or freed
 };
 
@@ -361,6 +395,18 @@ int launch_rows_occ(const SimArgs &a, int form, int row_words, const TermsF32 &t
                     int num_sms, cudaStream_t s);
 int launch_rows64(const SimArgs &a, int row_words, const TermsF64 &t, int scale, int num_sms,
                   cudaStream_t s);
+
+// marked32.cu, marked64.cu: the trial pass over marked events (a.table and
+// a.table2 the rows and their overflow; scale as for launch_rows64), and the
+// marks of a layer's rows.
+int launch_marked32(const SimArgs &a, const MarkMap &m, are_precision prec, bool packed, int row_words,
+                    const TermsF32 &t, int scale, int num_sms, cudaStream_t s);
+int launch_marks32(const ScatterArgs &a, const MarkMap &m, const void *table, const void *ovf, bool packed,
+                   int row_words, const TermsF32 &t, cudaStream_t s);
+int launch_marked64(const SimArgs &a, const MarkMap &m, int row_words, const TermsF64 &t, int scale, int num_sms,
+                    cudaStream_t s);
+int launch_marks64(const ScatterArgs &a, const MarkMap &m, const void *table, const void *ovf, int row_words,
+                   const TermsF64 &t, cudaStream_t s);
 
 // simulate.cu
 int launch_simulate(const SimArgs &a, are_precision prec, int jp, const TermsF32 *t32,

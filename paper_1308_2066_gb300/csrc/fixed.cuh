@@ -39,15 +39,9 @@ __device__ __forceinline__ int ilog2_bits(unsigned long long b)
     return (63 - __clzll((long long)b)) - 1074;   // subnormal
 }
 
-// h * 2^s as a 128-bit integer (round half up below the last bit).  With
-// s = 125 - floor(log2(hmax)) and h <= hmax the result is below 2^126.
-__device__ __forceinline__ void to_fixed(double h, int s, unsigned long long &lo, unsigned long long &hi)
+// m * 2^sh as a 128-bit integer (round half up below the last bit).
+__device__ __forceinline__ void shifted(unsigned long long m, int sh, unsigned long long &lo, unsigned long long &hi)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(h);
-    const int be = (int)((b >> 52) & 0x7ff);
-    unsigned long long m = b & ((1ull << 52) - 1);
-    if (be) m |= 1ull << 52;
-    const int sh = (be ? be : 1) - 1075 + s;    // value = m * 2^sh
     lo = 0;
     hi = 0;
     if (sh >= 64) {
@@ -61,6 +55,17 @@ __device__ __forceinline__ void to_fixed(double h, int s, unsigned long long &lo
         const int n = -sh;
         lo = (m >> n) + ((m >> (n - 1)) & 1ull);
     }
+}
+
+// h * 2^s as a 128-bit integer (round half up below the last bit).  With
+// s = 125 - floor(log2(hmax)) and h <= hmax the result is below 2^126.
+__device__ __forceinline__ void to_fixed(double h, int s, unsigned long long &lo, unsigned long long &hi)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(h);
+    const int be = (int)((b >> 52) & 0x7ff);
+    unsigned long long m = b & ((1ull << 52) - 1);
+    if (be) m |= 1ull << 52;
+    shifted(m, (be ? be : 1) - 1075 + s, lo, hi);    // value = m * 2^(e + s)
 }
 
 // (top:hi:lo) * 2^-s rounded once to the nearest double.
