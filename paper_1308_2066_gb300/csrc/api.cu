@@ -157,6 +157,52 @@ void dfree(are_ctx *ctx, void *p, size_t bytes)
     ctx->cached += it->second;
 }
 
+// The context's pinned host scratch for the length of a call (under the
+// context's lock), kept between calls up to kHostScratchKept.
+constexpr size_t kHostScratchKept = 64u << 20;
+constexpr size_t kIdsSeenKept = (8u << 20) / sizeof(uint64_t);
+class HostScratch {
+  public:
+    explicit HostScratch(are_ctx *c) : ctx(c) {}
+    ~HostScratch()
+    {
+        if (ctx->h_scratch_bytes > kHostScratchKept) release();
+    }
+    HostScratch(const HostScratch &) = delete;
+    HostScratch &operator=(const HostScratch &) = delete;
+    void *get(size_t bytes)
+    {
+        if (bytes > ctx->h_scratch_bytes) {
+            const size_t size = std::max(bytes, std::min(2 * ctx->h_scratch_bytes, kHostScratchKept));
+            release();
+            ARE_CUDA_TRY(cudaMallocHost(&ctx->h_scratch, size));
+            ctx->h_scratch_bytes = size;
+        }
+        return ctx->h_scratch;
+    }
+
+  private:
+    void release()
+    {
+        cudaFreeHost(ctx->h_scratch);
+        ctx->h_scratch = nullptr;
+        ctx->h_scratch_bytes = 0;
+    }
+    are_ctx *ctx;
+};
+
+// Whether a kernel of the context may read an array of `align`-byte elements
+// at p as it is: device memory of this GPU, aligned.
+bool readable_here(const are_ctx *ctx, const void *p, size_t align)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == ctx->device && reinterpret_cast<uintptr_t>(p) % align == 0;
+}
+
 // Copy n bytes from src (host or device) into device memory dst.
 void copy_in(void *dst, const void *src, size_t n, cudaStream_t s)
 {
@@ -232,13 +278,7 @@ ScatterArgs scatter_args(are_ctx *ctx, const Layer &L, int32_t catalog, int jp)
         ARE_CHECK(e.max_id < catalog, ARE_EINVAL,
                   "ELT " + std::to_string(L.elts[j]) + " holds event id " + std::to_string(e.max_id) +
                       " outside the YET's catalog of " + std::to_string(catalog));
-        a.ids[j] = e.d_ids;
-        a.loss[j] = e.d_loss;
-        a.n[j] = e.n;
-        a.fx[j] = e.terms.fx;
-        a.ded[j] = e.terms.deductible;
-        a.lim[j] = e.terms.limit;
-        a.share[j] = e.terms.share;
+        set_elt(a, (int)j, e);
     }
     return a;
 }
@@ -292,13 +332,46 @@ Compact &build_compact(are_ctx *ctx, Layer &L, int32_t catalog, cudaStream_t s)
 
 TuneEntry tuned(are_ctx *ctx, are_precision p, const Yet &y, int jp, bool multi);
 
-// Build (or rebuild) the layer's table for `catalog` in fp32 or fp64.
-Table &build_table(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, cudaStream_t s)
+void fill_terms(const Layer &L, TermsF32 &t32, TermsF64 &t64)
+{
+    t64.occ_r = L.terms.occ_ret;
+    t64.occ_l = L.terms.occ_lim;
+    t32.occ_r = (float)L.terms.occ_ret;
+    t32.occ_l = (float)L.terms.occ_lim;
+}
+
+// The layer's marks beside its FP32 or FP64 rows, sized for `catalog`.
+MarkMap &size_marks(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32)
+{
+    Marks &m = fp32 ? L.m32 : L.m64;
+    if (m.map.d && m.catalog != catalog) free_marks(ctx, m);
+    if (!m.map.d) {
+        const MarkMap shape = mark_shape(catalog);
+        uint32_t *d = (uint32_t *)dalloc(ctx, sizeof(uint32_t) * (size_t)shape.words);
+        ++L.generation;
+        m.map = shape;
+        m.map.d = d;
+        m.catalog = catalog;
+    }
+    return m.map;
+}
+
+// Build (or rebuild) the layer's table for `catalog` in fp32 or fp64; with
+// `marked` (fp32) its marks too.
+Table &build_table(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, cudaStream_t s, bool marked = false)
 {
     Table &t = fp32 ? L.t32 : L.t64;
     const int jp = table_jp((int)L.elts.size(), fp32);
     const ScatterArgs a = scatter_args(ctx, L, catalog, jp);
     size_table(ctx, L, t, catalog, jp, fp32 ? 4 : 8);
+    TermsF32 t32;
+    TermsF64 t64;
+    fill_terms(L, t32, t64);
+    const MarkMap m = marked ? size_marks(ctx, L, catalog, true) : MarkMap{};
+    if (fp32 && elts_bucketed(a)) {
+        ctx->launches += launch_tile_rows(a, catalog, true, false, jp, t.d, nullptr, m, t32, t64, s);
+        return t;
+    }
     ARE_CUDA_TRY(cudaMemsetAsync(t.d, 0, t.bytes, s));
     ctx->launches += launch_scatter_table(t.d, fp32, a, s);
     return t;
@@ -351,63 +424,51 @@ int row_words(const Layer &L, int32_t catalog, bool fp32)
     return packed_row_words((int)L.elts.size(), tpe, fp32);
 }
 
-// The packed FP64 rows of the layer, built straight from its ELT entries (no
-// dense table), read by the FP64 register-rows kernel.
-Packed &build_packed64(are_ctx *ctx, Layer &L, int32_t catalog, cudaStream_t s)
+// The packed rows of the layer (and, with `marked`, their marks), built from
+// its ELT entries with no dense table: what the register-rows kernels read.
+void build_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, int words, bool marked, cudaStream_t s)
 {
-    Packed &p = L.p64;
-    const int rw = row_words(L, catalog, false);
-    size_packed(ctx, L, p, catalog, rw, rw * sizeof(unsigned long long),
-                sizeof(double) * (size_t)layer_entries(L));
-    const ScatterArgs a = scatter_args(ctx, L, catalog, table_jp((int)L.elts.size(), false));
-    ctx->launches += launch_pack64_direct(a, catalog, rw, static_cast<unsigned long long *>(p.rows()),
-                                          static_cast<double *>(p.ovf()), p.used(), s);
-    return p;
-}
-
-// The packed FP32 rows (pw words each) built straight from the layer's ELT
-// entries, with no dense table: what the FP32 register-rows kernel reads.
-Packed &build_packed32_direct(are_ctx *ctx, Layer &L, int32_t catalog, int pw, cudaStream_t s)
-{
-    Packed &p = L.p32;
-    const ScatterArgs a = scatter_args(ctx, L, catalog, table_jp((int)L.elts.size(), true));
-    size_packed(ctx, L, p, catalog, pw, pw * sizeof(float), sizeof(float) * (size_t)layer_entries(L));
-    ctx->launches += launch_pack32_direct(a, catalog, pw, static_cast<uint32_t *>(p.rows()),
-                                          static_cast<float *>(p.ovf()), p.used(), s);
-    return p;
+    Packed &p = fp32 ? L.p32 : L.p64;
+    const size_t elem = fp32 ? sizeof(float) : sizeof(double);
+    const ScatterArgs a = scatter_args(ctx, L, catalog, table_jp((int)L.elts.size(), fp32));
+    size_packed(ctx, L, p, catalog, words, words * elem, elem * (size_t)layer_entries(L));
+    TermsF32 t32;
+    TermsF64 t64;
+    fill_terms(L, t32, t64);
+    const MarkMap m = marked ? size_marks(ctx, L, catalog, fp32) : MarkMap{};
+    if (elts_bucketed(a)) {
+        ctx->launches += launch_tile_rows(a, catalog, fp32, true, words, p.rows(), p.ovf(), m, t32, t64, s);
+        return;
+    }
+    // ids past the buckets' range (and past any marks)
+    if (fp32)
+        ctx->launches += launch_pack32_direct(a, catalog, words, static_cast<uint32_t *>(p.rows()),
+                                              static_cast<float *>(p.ovf()), p.used(), s);
+    else
+        ctx->launches += launch_pack64_direct(a, catalog, words, static_cast<unsigned long long *>(p.rows()),
+                                              static_cast<double *>(p.ovf()), p.used(), s);
 }
 
 // The table beside a layer's dense FP64 table that a kernel choice reads:
 // the FP32 screen (kernel 3).  `fresh`: the layer's table was just rebuilt.
 // (The packed rows of the register-rows kernels are built from the ELT
-// entries: build_packed32_direct, build_packed64.)
+// entries: build_packed.)
 void ensure_aux(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, int kernel, bool fresh, cudaStream_t s)
 {
     if (!fp32 && kernel == 3 && (fresh || !L.t32u.d || L.t32u.catalog != catalog)) build_screen(ctx, L, catalog, s);
 }
 
-void fill_terms(const Layer &L, TermsF32 &t32, TermsF64 &t64)
-{
-    t64.occ_r = L.terms.occ_ret;
-    t64.occ_l = L.terms.occ_lim;
-    t32.occ_r = (float)L.terms.occ_ret;
-    t32.occ_l = (float)L.terms.occ_lim;
-}
-
 // The packed rows a register-rows analysis (kernel 2) of the layer reads,
-// built if missing (or always, with rebuild); false where it reads the
-// dense FP32 table instead.
-bool ensure_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, cudaStream_t s, bool rebuild)
+// built if missing (or always, with rebuild, or where `marked` asks for marks
+// that are missing); false where it reads the dense FP32 table instead.
+bool ensure_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, bool marked, cudaStream_t s, bool rebuild)
 {
     const int w = row_words(L, catalog, fp32);
     if (!w) return false;
-    Packed &p = fp32 ? L.p32 : L.p64;
-    if (rebuild || !p.d || p.catalog != catalog || p.rw != w) {
-        if (fp32)
-            build_packed32_direct(ctx, L, catalog, w, s);
-        else
-            build_packed64(ctx, L, catalog, s);
-    }
+    const Packed &p = fp32 ? L.p32 : L.p64;
+    const Marks &m = fp32 ? L.m32 : L.m64;
+    if (rebuild || !p.d || p.catalog != catalog || p.rw != w || (marked && (!m.map.d || m.catalog != catalog)))
+        build_packed(ctx, L, catalog, fp32, w, marked, s);
     return true;
 }
 
@@ -448,7 +509,7 @@ double marked_share(are_ctx *ctx, const Layer &L, int32_t catalog)
         std::memcpy(&bits, &x, sizeof bits);
         const double at = std::isfinite(x) ? (double)bits / (double)(1ull << 50) - e.bin0 : 1e300;
         for (size_t i = 0; i < e.bins.size(); ++i)
-            above += e.bins[i] * std::min(1.0, std::max(0.0, (double)(i + 1) - at));
+            above += e.bin_weight * e.bins[i] * std::min(1.0, std::max(0.0, (double)(i + 1) - at));
     }
     L.marked = -std::expm1(-above / (double)catalog);
     L.marked_catalog = catalog;
@@ -490,29 +551,11 @@ void ensure_rows(are_ctx *ctx, Layer &L, const Yet &y, are_precision p, bool mar
 {
     const bool fp32 = p != ARE_FP64;
     const int32_t catalog = y.catalog;
-    const bool packed = ensure_packed(ctx, L, catalog, fp32, s, rebuild);
-    if (!packed && (rebuild || !L.t32.d || L.t32.catalog != catalog)) build_table(ctx, L, catalog, fp32, s);
-    if (!marked || !uses_marks(ctx, L, y, p)) return;
-    Marks &m = fp32 ? L.m32 : L.m64;
-    if (!rebuild && m.map.d && m.catalog == catalog) return;
-    if (m.map.d && m.catalog != catalog) free_marks(ctx, m);
-    if (!m.map.d) {
-        const MarkMap shape = mark_shape(catalog);
-        uint32_t *d = (uint32_t *)dalloc(ctx, sizeof(uint32_t) * (size_t)shape.words);
-        ++L.generation;
-        m.map = shape;
-        m.map.d = d;
-        m.catalog = catalog;
-    }
-    TermsF32 t32;
-    TermsF64 t64;
-    fill_terms(L, t32, t64);
-    const ScatterArgs a = scatter_args(ctx, L, catalog, 0);
-    if (fp32)
-        ctx->launches += packed ? launch_marks32(a, m.map, L.p32.rows(), L.p32.ovf(), true, L.p32.rw, t32, s)
-                                : launch_marks32(a, m.map, L.t32.d, nullptr, false, L.t32.jp, t32, s);
-    else
-        ctx->launches += launch_marks64(a, m.map, L.p64.rows(), L.p64.ovf(), L.p64.rw, t64, s);
+    marked = marked && uses_marks(ctx, L, y, p);
+    if (ensure_packed(ctx, L, catalog, fp32, marked, s, rebuild)) return;
+    if (rebuild || !L.t32.d || L.t32.catalog != catalog ||
+        (marked && (!L.m32.map.d || L.m32.catalog != catalog)))
+        build_table(ctx, L, catalog, true, s, marked);
 }
 
 // The tables that a kernel choice reads for a layer in the direct layout,
@@ -948,6 +991,7 @@ are_status are_destroy(are_ctx *ctx)
         if (ctx->d_flag) cudaFree(ctx->d_flag);
         if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
         if (ctx->h_result) cudaFreeHost(ctx->h_result);
+        if (ctx->h_scratch) cudaFreeHost(ctx->h_scratch);
         release_cache(ctx);
         if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
         if (ctx->stream) cudaStreamDestroy(ctx->stream);
@@ -1067,63 +1111,105 @@ are_status are_load_elt(are_ctx *ctx, int32_t n_entries, const int32_t *event_id
                   "share must lie in [0, 1]");
         fence_device_inputs({event_ids, losses});
         cudaStream_t s = ctx->stream;
-        std::vector<int32_t> ids = to_host(event_ids, (size_t)n_entries, s);
-        std::vector<double> loss = to_host(losses, (size_t)n_entries, s);
-        int32_t max_id = -1;
-        double max_loss = 0.0;
-        for (int32_t i = 0; i < n_entries; ++i) {
-            ARE_CHECK(ids[i] >= 0, ARE_EINVAL, "negative event id in ELT");
-            ARE_CHECK(nonneg_finite(loss[i]), ARE_EINVAL, "ELT losses must be finite and >= 0");
-            ARE_CHECK(std::isfinite(f.fx * loss[i]), ARE_EINVAL, "fx * loss overflows");
-            max_id = std::max(max_id, ids[i]);
-            max_loss = std::max(max_loss, loss[i]);
+        const size_t n = (size_t)n_entries;
+        HostScratch hs(ctx);
+        const int32_t *ids = event_ids;   // on the host
+        const double *loss = losses;
+        if (n && (is_device_ptr(event_ids) || is_device_ptr(losses))) {
+            double *in_loss = static_cast<double *>(hs.get(n * (sizeof(double) + sizeof(int32_t))));
+            int32_t *in_ids = reinterpret_cast<int32_t *>(in_loss + n);
+            ARE_CUDA_TRY(cudaMemcpyAsync(in_loss, losses, n * sizeof(double), cudaMemcpyDefault, s));
+            ARE_CUDA_TRY(cudaMemcpyAsync(in_ids, event_ids, n * sizeof(int32_t), cudaMemcpyDefault, s));
+            ARE_CUDA_TRY(cudaStreamSynchronize(s));
+            ids = in_ids;
+            loss = in_loss;
         }
+        constexpr uint64_t kSign = 1ull << 63, kInf = 0x7ffull << 52;
+        int32_t max_id = -1;
+        uint64_t most = 0, least = ~0ull;   // of the losses' bit patterns (-0.0 as 0)
+        bool bad_id = false, bad_loss = false;
+        auto bits_of = [&](size_t i) {
+            uint64_t x;
+            std::memcpy(&x, loss + i, sizeof x);
+            return x == kSign ? 0 : x;
+        };
+        for (size_t i = 0; i < n; ++i) {
+            bad_id |= ids[i] < 0;
+            max_id = std::max(max_id, ids[i]);
+        }
+        for (size_t i = 0; i < n; ++i) {
+            const uint64_t x = bits_of(i);
+            bad_loss |= x >= kInf;          // negative, infinite or NaN
+            most = std::max(most, x);
+            least = std::min(least, x);
+        }
+        ARE_CHECK(!bad_id, ARE_EINVAL, "negative event id in ELT");
+        ARE_CHECK(!bad_loss, ARE_EINVAL, "ELT losses must be finite and >= 0");
+        Elt e;
+        std::memcpy(&e.max_loss, &most, sizeof most);
+        ARE_CHECK(std::isfinite(f.fx * e.max_loss), ARE_EINVAL, "fx * loss overflows");
         bool dup = false;
-        if (n_entries == 0) {
+        if (n == 0) {
         } else if (max_id < (1 << 28)) {   // bitmap of the ids seen
-            std::vector<uint64_t> seen((size_t)max_id / 64 + 1, 0);
-            for (int32_t i = 0; i < n_entries && !dup; ++i) {
+            std::vector<uint64_t> &seen = ctx->ids_seen;
+            seen.assign((size_t)max_id / 64 + 1, 0);
+            for (size_t i = 0; i < n; ++i) {
                 uint64_t &w = seen[(size_t)ids[i] >> 6];
                 const uint64_t b = 1ull << (ids[i] & 63);
-                dup = (w & b) != 0;
+                dup |= (w & b) != 0;
                 w |= b;
             }
+            if (seen.size() > kIdsSeenKept) std::vector<uint64_t>().swap(seen);
         } else {
-            std::vector<int32_t> sorted(ids);
+            std::vector<int32_t> sorted(ids, ids + n);
             std::sort(sorted.begin(), sorted.end());
             dup = std::adjacent_find(sorted.begin(), sorted.end()) != sorted.end();
         }
         ARE_CHECK(!dup, ARE_EINVAL, "duplicate event id within one ELT");
-        Elt e;
-        if (n_entries > 0) {   // the losses by quarter octave
-            auto bin = [](double x) {
-                uint64_t b;
-                std::memcpy(&b, &x, sizeof b);
-                return (int32_t)(b >> 50 & 0x1fff);
-            };
-            const double least = *std::min_element(loss.begin(), loss.end());
-            e.bin0 = bin(least);
-            e.bins.assign((size_t)(bin(max_loss) - e.bin0 + 1), 0u);
-            for (double x : loss) ++e.bins[(size_t)(bin(x) - e.bin0)];
-        }
         e.n = n_entries;
         e.max_id = max_id;
-        e.max_loss = max_loss;
         e.terms = f;
+        if (n) {   // the losses by quarter octave, of up to about 4096 of them
+            e.bin0 = (int32_t)(least >> 50);
+            e.bins.assign((size_t)((int32_t)(most >> 50) - e.bin0 + 1), 0u);
+            const size_t step = n / 4096 + 1;
+            for (size_t i = 0; i < n; i += step) ++e.bins[(size_t)((int32_t)(bits_of(i) >> 50) - e.bin0)];
+            e.bin_weight = (double)n / (double)((n + step - 1) / step);
+        }
+        if (n && max_id < kMaxBucketedId) e.tiles = max_id / kEltTile + 1;
+        e.ids_bytes = sizeof(int32_t) * (n + (e.tiles ? 2 * ((size_t)e.tiles + 1) : 0));   // ids, offsets, scratch
+        char *tmp = nullptr;
+        const size_t tmp_bytes = n * (sizeof(double) + sizeof(int32_t));
         try {
-            e.d_ids = (int32_t *)dalloc(ctx, sizeof(int32_t) * n_entries);
-            e.d_loss = (double *)dalloc(ctx, sizeof(double) * n_entries);
-            copy_in(e.d_ids, ids.data(), sizeof(int32_t) * n_entries, s);
-            copy_in(e.d_loss, loss.data(), sizeof(double) * n_entries, s);
+            e.d_ids = (int32_t *)dalloc(ctx, e.ids_bytes);
+            e.d_loss = (double *)dalloc(ctx, sizeof(double) * n);
+            if (!e.tiles) {
+                copy_in(e.d_ids, event_ids, sizeof(int32_t) * n, s);
+                copy_in(e.d_loss, losses, sizeof(double) * n, s);
+            } else {   // bucketed on the device, from where the entries are if they can be read there
+                e.d_off = e.d_ids + n;
+                const int32_t *src_ids = event_ids;
+                const double *src_loss = losses;
+                if (!readable_here(ctx, event_ids, sizeof(int32_t)) || !readable_here(ctx, losses, sizeof(double))) {
+                    tmp = (char *)dalloc(ctx, tmp_bytes);
+                    copy_in(tmp, losses, sizeof(double) * n, s);
+                    copy_in(tmp + sizeof(double) * n, event_ids, sizeof(int32_t) * n, s);
+                    src_loss = reinterpret_cast<const double *>(tmp);
+                    src_ids = reinterpret_cast<const int32_t *>(src_loss + n);
+                }
+                ctx->launches += launch_bucket(src_ids, src_loss, n_entries, e.tiles, e.d_ids, e.d_loss, e.d_off,
+                                               e.d_off + e.tiles + 1, s);
+            }
             ARE_CUDA_TRY(cudaStreamSynchronize(s));
         } catch (...) {
-            dfree(ctx, e.d_ids, sizeof(int32_t) * n_entries);
-            dfree(ctx, e.d_loss, sizeof(double) * n_entries);
+            dfree(ctx, tmp, tmp_bytes);
+            dfree(ctx, e.d_ids, e.ids_bytes);
+            dfree(ctx, e.d_loss, sizeof(double) * n);
             throw;
         }
-        e.bytes = (sizeof(int32_t) + sizeof(double)) * n_entries;
+        dfree(ctx, tmp, tmp_bytes);
         const int32_t h = ctx->next_handle++;
-        ctx->elts[h] = e;
+        ctx->elts[h] = std::move(e);
         *elt_handle = h;
     });
 }
@@ -1177,7 +1263,7 @@ are_status are_free_elt(are_ctx *ctx, int32_t h)
         ARE_CHECK(it != ctx->elts.end(), ARE_ENOTFOUND, "unknown ELT handle " + std::to_string(h));
         ARE_CHECK(it->second.users == 0, ARE_EINVAL, "ELT is used by a layer");
         ARE_CHECK(!ctx->server, ARE_EBUSY, "a pricing server is running on this context");
-        dfree(ctx, it->second.d_ids, sizeof(int32_t) * it->second.n);
+        dfree(ctx, it->second.d_ids, it->second.ids_bytes);
         dfree(ctx, it->second.d_loss, sizeof(double) * it->second.n);
         ctx->elts.erase(it);
     });
@@ -1627,7 +1713,7 @@ are_status are_simulate_occurrences(are_ctx *ctx, int32_t layer, int32_t yet, in
         Table &t = fp32 ? L.t32 : L.t64;
         // the rows of the register-rows form (the direct layout, whatever the
         // layer's analysis layout): packed where the layer's row size calls for them
-        const bool packed = ensure_packed(ctx, L, y.catalog, fp32, cs.s, false);
+        const bool packed = ensure_packed(ctx, L, y.catalog, fp32, false, cs.s, false);
         if (!packed && (!t.d || t.catalog != y.catalog)) build_table(ctx, L, y.catalog, fp32, cs.s);
         SimArgs a{};
         a.ids = y.d_ids;

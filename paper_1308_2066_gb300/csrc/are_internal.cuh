@@ -63,16 +63,25 @@ struct Yet {
 };
 constexpr int64_t kIdPad = 64;     // zero ids after the last event (vector over-read)
 
+// An ELT's entries lie in buckets, one per tile of kEltTile catalog events in
+// event order (within a bucket in any order), with the buckets' offsets,
+// where the ids stay below kMaxBucketedId (a block's shared memory counts the
+// buckets); else in the order given.
+constexpr int32_t kEltTile = 256;
+constexpr int32_t kMaxBucketedId = 48 * 1024 * kEltTile;
 struct Elt {
     int32_t n = 0;
     int32_t max_id = -1;
+    int32_t tiles = 0;             // buckets: tiles up to the last id's
+    int32_t *d_off = nullptr;      // tiles + 1 offsets (in d_ids' allocation), or nullptr
     double max_loss = 0.0;         // largest loss of the ELT
-    int32_t bin0 = 0;              // its losses counted by quarter octaves: bins[i] of those whose
-    std::vector<uint32_t> bins;    // bit pattern >> 50 is bin0 + i
+    int32_t bin0 = 0;              // its losses (or an even sample of them, bin_weight losses each) counted by
+    std::vector<uint32_t> bins;    // quarter octaves: bins[i] of those whose bit pattern >> 50 is bin0 + i
+    double bin_weight = 1.0;
     int32_t *d_ids = nullptr;
     double *d_loss = nullptr;
     are_fin_terms terms{};
-    size_t bytes = 0;
+    size_t ids_bytes = 0;          // of d_ids' allocation
     int users = 0;                 // layers referring to it
 };
 
@@ -162,6 +171,7 @@ struct Marks {
 };
 // The shape of a catalog's marks; words 0 where more than two events would
 // share a bit.
+static_assert(2LL * 32 * kMaxMarkWords <= kMaxBucketedId, "a marked catalog's ELTs lie in buckets");
 inline MarkMap mark_shape(int32_t catalog)
 {
     MarkMap m;
@@ -244,6 +254,8 @@ struct FoldArgs {
 
 // The layer's ELTs and their financial terms, as the table builders read them.
 struct ScatterArgs {
+    const int32_t *off[kMaxElts];  // bucket offsets, or nullptr
+    int32_t tiles[kMaxElts];
     const int32_t *ids[kMaxElts];
     const double *loss[kMaxElts];
     int32_t n[kMaxElts];
@@ -330,6 +342,31 @@ struct Plan {
 // repack.cu
 int launch_scatter_table(void *table, bool fp32, const ScatterArgs &a, cudaStream_t s,
                          bool round_up = false);
+// Entry j of the table builders' arguments.
+inline void set_elt(ScatterArgs &a, int j, const Elt &e)
+{
+    a.off[j] = e.d_off;
+    a.tiles[j] = e.tiles;
+    a.ids[j] = e.d_ids;
+    a.loss[j] = e.d_loss;
+    a.n[j] = e.n;
+    a.fx[j] = e.terms.fx;
+    a.ded[j] = e.terms.deductible;
+    a.lim[j] = e.terms.limit;
+    a.share[j] = e.terms.share;
+}
+// Whether every ELT's entries lie in buckets.
+inline bool elts_bucketed(const ScatterArgs &a)
+{
+    for (int j = 0; j < a.n_elts; ++j)
+        if (a.n[j] > 0 && !a.off[j]) return false;
+    return true;
+}
+// tile_rows.cu
+int launch_bucket(const int32_t *ids, const double *loss, int32_t n, int32_t tiles, int32_t *out_ids, double *out_loss,
+                  int32_t *off, int32_t *next, cudaStream_t s);
+int launch_tile_rows(const ScatterArgs &elts, int32_t catalog, bool fp32, bool packed, int words, void *rows, void *ovf,
+                     const MarkMap &marks, const TermsF32 &o32, const TermsF64 &o64, cudaStream_t s);
 int launch_screen64(const SimArgs &a, int jp32, const TermsF64 &t, int num_sms, cudaStream_t s);
 int64_t compact_scan_blocks(int32_t catalog);
 int launch_build_compact(int32_t *row_of, int32_t *counts, float *rows, size_t rows_bytes,
@@ -397,16 +434,11 @@ int launch_rows64(const SimArgs &a, int row_words, const TermsF64 &t, int scale,
                   cudaStream_t s);
 
 // marked32.cu, marked64.cu: the trial pass over marked events (a.table and
-// a.table2 the rows and their overflow; scale as for launch_rows64), and the
-// marks of a layer's rows.
+// a.table2 the rows and their overflow; scale as for launch_rows64).
 int launch_marked32(const SimArgs &a, const MarkMap &m, are_precision prec, bool packed, int row_words,
                     const TermsF32 &t, int scale, int num_sms, cudaStream_t s);
-int launch_marks32(const ScatterArgs &a, const MarkMap &m, const void *table, const void *ovf, bool packed,
-                   int row_words, const TermsF32 &t, cudaStream_t s);
 int launch_marked64(const SimArgs &a, const MarkMap &m, int row_words, const TermsF64 &t, int scale, int num_sms,
                     cudaStream_t s);
-int launch_marks64(const ScatterArgs &a, const MarkMap &m, const void *table, const void *ovf, int row_words,
-                   const TermsF64 &t, cudaStream_t s);
 
 // simulate.cu
 int launch_simulate(const SimArgs &a, are_precision prec, int jp, const TermsF32 *t32,
@@ -466,6 +498,9 @@ struct are_ctx {
     int *h_flag = nullptr;   // pinned mirror
     are::SelectScratch sel;
     double *h_result = nullptr;  // pinned, 2 * kMaxTargets
+    void *h_scratch = nullptr;   // pinned: ELTs being loaded
+    size_t h_scratch_bytes = 0;
+    std::vector<uint64_t> ids_seen;   // bitmap of an ELT being loaded
     uint64_t launches = 0;       // kernels launched by this context
     cudaStream_t capture = nullptr;           // stream used to capture plans
     std::map<std::string, are::TuneEntry> tune;

@@ -7,7 +7,8 @@
 // loss.  Reading a row for each of them is bound by the L1 unit (one line
 // lookup per occurrence, about one per SM clock whatever the row's size).
 // So the table build marks the events whose occurrence loss is not 0, one
-// bit per catalog event (k_mark), and the trial pass looks each occurrence up
+// bit per catalog event (tile_rows.cu; event e's is bit 31 - e % 32 of word
+// e / 32, so a rotation by e brings it to the top), and the trial pass looks each occurrence up
 // in the marks first, held in shared memory; an unmarked event's loss is 0
 // in the same arithmetic, so leaving it out of the sum changes nothing.
 //
@@ -184,14 +185,6 @@ __device__ __forceinline__ void to_fixed(float x, int s, unsigned long long &lo,
     const uint32_t m = be ? (u & 0x7fffffu) | 0x800000u : u;
     fixed::shifted(m, (be ? be : 1) - 150 + s, lo, hi);   // x * 2^s = m * 2^(e + s)
 }
-
-// ---------------------------------------------------------------------------
-// the marks
-// ---------------------------------------------------------------------------
-
-// Event e's bit is bit 31 - e % 32 of word e / 32, so a rotation by e brings
-// it to the top.
-__device__ __forceinline__ uint32_t mark_bit(uint32_t e) { return 0x80000000u >> (e & 31); }
 
 // ---------------------------------------------------------------------------
 // the trial pass
@@ -539,21 +532,6 @@ __global__ void __launch_bounds__(32 * pass_warps(ACC == ARE_FP32_KAHAN, FIXED),
     }
 }
 
-// Marks the events whose occurrence loss is not 0: every ELT entry (grid.y =
-// ELT) forms its event's loss from the event's row.
-template <typename Rows>
-__global__ void k_mark(const ScatterArgs a, const Rows rows_, uint32_t *__restrict__ marks, uint32_t bits)
-{
-    const int j = blockIdx.y;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n[j]; i += gridDim.x * blockDim.x) {
-        uint32_t e = (uint32_t)a.ids[j][i];
-        if (rows_.loss(rows_.load(e), e) != 0) {
-            e = min(e, e - bits);
-            atomicOr(marks + (e >> 5), mark_bit(e));
-        }
-    }
-}
-
 template <typename Rows, int ACC, bool FIXED, bool FOLD>
 void launch_pass_t(const PassArgs &a, const Rows &rows_, int num_sms, cudaStream_t s)
 {
@@ -588,20 +566,6 @@ void launch_pass(const SimArgs &a, const MarkMap &m, const Rows &rows_, int scal
     else
         m.fold ? launch_pass_t<Rows, ACC, true, true>(p, rows_, num_sms, s)
                : launch_pass_t<Rows, ACC, true, false>(p, rows_, num_sms, s);
-}
-
-template <typename Rows>
-int launch_marks(const ScatterArgs &a, const MarkMap &m, const Rows &rows_, cudaStream_t s)
-{
-    ARE_CUDA_TRY(cudaMemsetAsync(m.d, 0, sizeof(uint32_t) * (size_t)m.words, s));
-    int32_t nmax = 0;
-    for (int j = 0; j < a.n_elts; ++j) nmax = a.n[j] > nmax ? a.n[j] : nmax;
-    if (nmax == 0) return 0;
-    dim3 grid((unsigned)((nmax + 255) / 256), (unsigned)a.n_elts);
-    if (grid.x > 4096) grid.x = 4096;
-    k_mark<Rows><<<grid, 256, 0, s>>>(a, rows_, m.d, m.bits);
-    ARE_CUDA_TRY(cudaGetLastError());
-    return 1;
 }
 
 }  // namespace marked

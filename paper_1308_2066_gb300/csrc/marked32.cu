@@ -1,5 +1,5 @@
 // marked32.cu -- the trial pass over marked events (marked.cuh) with FP32
-// rows, packed or dense, and the marks of a layer's FP32 rows.
+// rows, packed or dense.
 #include <cuda_runtime.h>
 
 #include <string>
@@ -42,12 +42,6 @@ int launch_marked32(const SimArgs &a, const MarkMap &m, are_precision prec, bool
         return 0;
     });
     return 1;
-}
-
-int launch_marks32(const ScatterArgs &a, const MarkMap &m, const void *table, const void *ovf, bool packed,
-                   int row_words, const TermsF32 &t, cudaStream_t s)
-{
-    return with_rows(table, ovf, packed, row_words, t, [&](auto r) { return marked::launch_marks(a, m, r, s); });
 }
 
 }  // namespace are

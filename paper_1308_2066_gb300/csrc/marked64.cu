@@ -1,5 +1,5 @@
 // marked64.cu -- the trial pass over marked events (marked.cuh) with packed
-// FP64 rows, and the marks of a layer's FP64 rows.
+// FP64 rows.
 #include <cuda_runtime.h>
 
 #include <string>
@@ -36,12 +36,6 @@ int launch_marked64(const SimArgs &a, const MarkMap &m, int row_words, const Ter
         return 0;
     });
     return 1;
-}
-
-int launch_marks64(const ScatterArgs &a, const MarkMap &m, const void *table, const void *ovf, int row_words,
-                   const TermsF64 &t, cudaStream_t s)
-{
-    return with_rows(table, ovf, row_words, t, [&](auto r) { return marked::launch_marks(a, m, r, s); });
 }
 
 }  // namespace are

@@ -230,14 +230,7 @@ void build_request_table(Server &S, Slot &sl)
         a.n_elts = (int32_t)sl.req.elts.size();
         a.jp = sl.jp;
         for (size_t j = 0; j < sl.req.elts.size(); ++j) {
-            const Elt &e = S.ctx->elts.at(sl.req.elts[j]);
-            a.ids[j] = e.d_ids;
-            a.loss[j] = e.d_loss;
-            a.n[j] = e.n;
-            a.fx[j] = e.terms.fx;
-            a.ded[j] = e.terms.deductible;
-            a.lim[j] = e.terms.limit;
-            a.share[j] = e.terms.share;
+            set_elt(a, (int)j, S.ctx->elts.at(sl.req.elts[j]));
         }
     }
     if (S.cfg.folded) {
@@ -245,6 +238,14 @@ void build_request_table(Server &S, Slot &sl)
         add_launches(S, launch_fold(a, sl.req.terms.occ_ret, sl.req.terms.occ_lim, S.y->catalog,
                                     folded_F(b, S.y->catalog), folded_bits(b), folded_hmax(b),
                                     S.ctx->num_sms, S.stream));
+        return;
+    }
+    if (elts_bucketed(a)) {
+        const bool packed = sl.pw != 0;
+        add_launches(S, launch_tile_rows(a, S.y->catalog, true, packed, packed ? sl.pw : sl.jp,
+                                         packed ? (void *)packed_rows(S, sl) : (void *)(S.d_arena + sl.tab_off),
+                                         packed ? packed_ovf(S, sl) : nullptr, MarkMap{}, TermsF32{}, TermsF64{},
+                                         S.stream));
         return;
     }
     if (sl.pw) {   // packed rows straight from the ELT entries

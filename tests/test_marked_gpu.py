@@ -123,3 +123,43 @@ def test_the_share_of_marked_events_decides(are):
             are.are_free_yet(ctx, y)
     finally:
         are.are_destroy(ctx)
+
+
+@pytest.mark.parametrize("J,C,nnz", [(3, 255, 100), (5, 256, 200), (9, 257, 100), (16, 513, 60), (16, 1000, 700),
+                                     (32, 70_000, 700), (32, 300, 300), (10, 48 * 65536 * 4 + 300, 500)])
+def test_rows_built_tile_by_tile(are, orc, J, C, nnz):
+    """One-event trials give every event's loss from the rows as built: tiles
+    of 256 events around their edges, more entries in a tile than it keeps
+    between its passes, every ELT holding an event (overflows), ELTs whose
+    last tile comes before the catalog's, an ELT without entries, and ids past
+    the buckets.  FP64 equals the oracle's bit for bit; FP32 terms are rounded
+    once and up to 32 of them added."""
+    import torch
+    g = np.random.Generator(np.random.PCG64(J + C))
+    top = C if C < 1 << 20 else C - 1
+    near = np.arange(top - 300, top) if C >= 1 << 20 else np.arange(C)
+    elts = []
+    for j in range(J):
+        pool = near if j % 2 else near[: max(1, near.size - 40 * j % near.size)]
+        ids = g.permutation(pool)[: min(nnz, pool.size)].astype(np.int32)
+        elts.append(W.percentile_terms(W.ELT(ids, g.lognormal(11, 1.5, ids.size))))
+    elts[J // 2] = W.ELT(np.zeros(0, np.int32), np.zeros(0))
+    events = g.permutation(near)[:2000].astype(np.int32)
+    yet = W.YET(catalog=C, n_trials=events.size, ids=events, k=1)
+    wl = W.Workload("t", yet, elts, [W.Layer(list(range(J)), 2e4, 1e6, 0.0, INF)])
+    ref = orc.simulate_layer(wl).ylt
+    ctx = are.are_create(0)
+    try:
+        y = are.are_load_yet(ctx, C, events.size, None, 1, events)
+        hs = [are.are_load_elt(ctx, e.ids, e.losses, e.fx, e.ded, e.lim, e.share) for e in elts]
+        layer = are.are_define_layer(ctx, hs, 2e4, 1e6, 0.0, INF)
+        for p in (0, 1, 2):
+            out = torch.full((events.size,), -1.0, dtype=torch.float64, device="cuda")
+            are.are_simulate(ctx, layer, y, 0, events.size, p, out)
+            if p == 0:
+                np.testing.assert_array_equal(out.cpu().numpy(), ref)
+            else:    # 34 roundings at the scale of the event loss, at most 32 limits
+                bound = 34 * 2.0 ** -24 * sum(e.lim for e in elts if np.isfinite(e.lim))
+                np.testing.assert_allclose(out.cpu().numpy(), ref, rtol=1e-5, atol=bound)
+    finally:
+        are.are_destroy(ctx)
