@@ -945,7 +945,7 @@ are_status are_create(are_ctx **out, int device, size_t mem_budget_bytes)
         ARE_CUDA_TRY(cudaMalloc(&ctx->d_flag, sizeof(int)));
         ARE_CUDA_TRY(cudaMallocHost(&ctx->h_flag, sizeof(int)));
         ARE_CUDA_TRY(cudaMallocHost(&ctx->h_result, sizeof(double) * 2 * kMaxTargets));
-        select_alloc(ctx->sel, ctx->num_sms);
+        select_alloc(ctx->sel, 1);
     });
     if (st != ARE_OK) {
         are_destroy(ctx);
@@ -988,6 +988,7 @@ are_status are_destroy(are_ctx *ctx)
         if (ctx->h_multi) cudaFreeHost(ctx->h_multi);
         if (ctx->capture) cudaStreamDestroy(ctx->capture);
         select_free(ctx->sel);
+        select_free(ctx->sel_multi);
         if (ctx->d_flag) cudaFree(ctx->d_flag);
         if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
         if (ctx->h_result) cudaFreeHost(ctx->h_result);
@@ -1776,19 +1777,25 @@ are_status are_risk_measures(are_ctx *ctx, const double *ylt, int64_t n,
             CallStream cs(ctx, stream);
             cudaStream_t s = cs.s;
             const int32_t nr = (int32_t)ranks.size();
+            // written by the selection itself where it can, else copied
+            const bool direct = (n_rp == 0 || readable_here(ctx, pml_out, sizeof(double))) &&
+                                (n_tv == 0 || readable_here(ctx, tvar_out, sizeof(double)));
             for (int32_t b = 0; b < nr; b += kMaxTargets) {
                 const int nt = std::min<int32_t>(kMaxTargets, nr - b);
-                ctx->launches += launch_select(ylt, n, ranks.data() + b, nt, ctx->sel, ctx->num_sms, s);
-                // result: (m-th largest, mean of the m largest) per target
-                const int p_end = std::min(b + nt, n_rp);
-                if (p_end > b)
+                // targets up to n_rp are values, the others means
+                const int values = std::min(std::max(n_rp - b, 0), nt);
+                double *out[kMaxTargets] = {};
+                for (int t = 0; t < nt; ++t) out[t] = t < values ? pml_out + b + t : tvar_out + (b + t - n_rp);
+                ctx->launches += launch_select(ylt, n, ranks.data() + b, nt, values, direct ? out : nullptr, ctx->sel,
+                                               ctx->num_sms, s);
+                if (direct) continue;
+                if (values)
                     ARE_CUDA_TRY(cudaMemcpy2DAsync(pml_out + b, sizeof(double), ctx->sel.result, 2 * sizeof(double),
-                                                   sizeof(double), p_end - b, cudaMemcpyDeviceToDevice, s));
-                const int t_begin = std::max(b, n_rp);
-                if (b + nt > t_begin)
-                    ARE_CUDA_TRY(cudaMemcpy2DAsync(tvar_out + (t_begin - n_rp), sizeof(double),
-                                                   ctx->sel.result + 2 * (t_begin - b) + 1, 2 * sizeof(double),
-                                                   sizeof(double), b + nt - t_begin, cudaMemcpyDeviceToDevice, s));
+                                                   sizeof(double), values, cudaMemcpyDeviceToDevice, s));
+                if (nt > values)
+                    ARE_CUDA_TRY(cudaMemcpy2DAsync(tvar_out + (b + values - n_rp), sizeof(double),
+                                                   ctx->sel.result + 2 * values + 1, 2 * sizeof(double),
+                                                   sizeof(double), nt - values, cudaMemcpyDeviceToDevice, s));
             }
             cs.finish();
             return;
@@ -1807,7 +1814,8 @@ are_status are_risk_measures(are_ctx *ctx, const double *ylt, int64_t n,
             if (tmp) copy_in(tmp, ylt, sizeof(double) * n, s);
             for (size_t b = 0; b < ranks.size(); b += kMaxTargets) {
                 const int nt = (int)std::min<size_t>(kMaxTargets, ranks.size() - b);
-                ctx->launches += launch_select(d_y, n, ranks.data() + b, nt, ctx->sel, ctx->num_sms, s);
+                const int values = std::min(std::max(n_rp - (int32_t)b, 0), nt);
+                ctx->launches += launch_select(d_y, n, ranks.data() + b, nt, values, nullptr, ctx->sel, ctx->num_sms, s);
                 ARE_CUDA_TRY(cudaMemcpyAsync(ctx->h_result, ctx->sel.result, sizeof(double) * 2 * nt,
                                              cudaMemcpyDeviceToHost, s));
                 ARE_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1930,7 +1938,8 @@ are_status are_risk_measures_batch(are_ctx *ctx, const double *const *ylts, int3
         if (ranks.empty()) return;
         CallStream cs(ctx, stream);
         const size_t ptr_bytes = (sizeof(double *) * n_ylt + 255) / 256 * 256;
-        const size_t need = ptr_bytes + select_multi_bytes(n_ylt, n, ctx->num_sms);
+        if (!ctx->sel_multi.coop) select_alloc(ctx->sel_multi, kMultiGroups);
+        const size_t need = ptr_bytes + sizeof(double) * 2 * kMaxTargets * (size_t)n_ylt;
         if (ctx->multi_bytes < need) {
             ARE_CUDA_TRY(cudaStreamSynchronize(cs.s));
             dfree(ctx, ctx->d_multi, ctx->multi_bytes);
@@ -1950,12 +1959,12 @@ are_status are_risk_measures_batch(are_ctx *ctx, const double *const *ylts, int3
         const double *const *d_ptrs = static_cast<const double *const *>(ctx->d_multi);
         ARE_CUDA_TRY(cudaMemcpyAsync(ctx->d_multi, ylts, sizeof(double *) * n_ylt,
                                      cudaMemcpyHostToDevice, cs.s));
-        void *scratch = static_cast<unsigned char *>(ctx->d_multi) + ptr_bytes;
+        double *d_res = reinterpret_cast<double *>(static_cast<unsigned char *>(ctx->d_multi) + ptr_bytes);
         for (size_t b = 0; b < ranks.size(); b += kMaxTargets) {
             const int nt = (int)std::min<size_t>(kMaxTargets, ranks.size() - b);
-            double *d_res = nullptr;
-            ctx->launches += launch_select_multi(d_ptrs, n_ylt, n, ranks.data() + b, nt, scratch,
-                                                 ctx->num_sms, cs.s, &d_res);
+            const int values = std::min(std::max(n_rp - (int32_t)b, 0), nt);
+            ctx->launches += launch_select_multi(d_ptrs, n_ylt, n, ranks.data() + b, nt, values, d_res,
+                                                 ctx->sel_multi, ctx->num_sms, cs.s);
             ARE_CUDA_TRY(cudaMemcpyAsync(ctx->h_multi, d_res, sizeof(double) * count,
                                          cudaMemcpyDeviceToHost, cs.s));
             ARE_CUDA_TRY(cudaStreamSynchronize(cs.s));

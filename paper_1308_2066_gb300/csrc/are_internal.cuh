@@ -446,16 +446,12 @@ int launch_simulate(const SimArgs &a, are_precision prec, int jp, const TermsF32
 
 // select.cu
 struct SelectScratch {
-    uint32_t *hist = nullptr;       // 3 * kMaxTargets * 256
-    unsigned long long *state = nullptr;  // per target: prefix, remaining rank
-    unsigned int *ctrl = nullptr;   // 4 words: blocks arrived, top word of the largest |value|
-    unsigned long long *acc = nullptr;    // per target: integer tail sums and count (7 words)
-    double *result = nullptr;       // per target: value, tail mean
-    unsigned long long *app = nullptr;    // single-YLT selection, per target: keys kept
-    unsigned long long *cand = nullptr;   // per target: the kept keys of its bucket
-    int max_blocks = 0;
+    void *coop = nullptr;           // per group of blocks, left ready for the next selection
+    int groups = 0;                 // YLTs selected at a time
+    double *result = nullptr;       // single YLT, per target: value, tail mean
 };
-void select_alloc(SelectScratch &s, int num_sms);
+void select_alloc(SelectScratch &s, int groups);
+constexpr int kMultiGroups = 16;    // of the batched selection (3.5 MB)
 // Ranks of the risk measures (definitions in include/are.h); -1 when the
 // return period or level is out of range.
 int64_t rank_for_return_period(int64_t n, double rp);
@@ -463,19 +459,16 @@ int64_t rank_for_level(int64_t n, double a);
 // Message of the calling thread's last failed are_risk_measures_static call.
 const char *static_last_error();
 void select_free(SelectScratch &s);
-constexpr int kSelectLaunches = 1 + 8 + 1;    // the multi-YLT and allocation-free selections
-inline int select_max_blocks(int num_sms) { return num_sms * 4; }
-// ranks[t] (1-based, descending order) for n_targets <= kMaxTargets; writes
-// result[2*t] = m-th largest value, result[2*t+1] = mean of the m largest.
-cudaError_t select_enqueue(const double *ylt, int64_t n, const int64_t *ranks, int nt,
-                           const SelectScratch &s, cudaStream_t st);
-// The same for n_ylt YLTs of n losses each (device array of pointers); the
-// scratch must be sized by select_multi_bytes.  Results: result[(y*8+t)*2].
-size_t select_multi_bytes(int n_ylt, int64_t n, int num_sms);
-int launch_select_multi(const double *const *ylts, int n_ylt, int64_t n, const int64_t *ranks,
-                        int nt, void *scratch, int num_sms, cudaStream_t st, double **result);
-int launch_select(const double *ylt, int64_t n, const int64_t *ranks, int n_targets,
-                   SelectScratch &s, int num_sms, cudaStream_t st);
+// ranks[t] (1-based, descending order) for nt <= kMaxTargets: s.result[2*t]
+// receives the ranks[t]-th largest value and, from target n_values on,
+// s.result[2*t+1] the mean of the ranks[t] largest; out[t] (out or it may be
+// null) receives the value, or from target n_values on the mean.
+int launch_select(const double *ylt, int64_t n, const int64_t *ranks, int nt, int n_values, double *const *out,
+                  SelectScratch &s, int num_sms, cudaStream_t st);
+// The same for n_ylt YLTs of n losses each (device array of pointers):
+// results[(y * kMaxTargets + t) * 2].
+int launch_select_multi(const double *const *ylts, int n_ylt, int64_t n, const int64_t *ranks, int nt, int n_values,
+                        double *results, SelectScratch &s, int num_sms, cudaStream_t st);
 
 }  // namespace are
 
@@ -496,7 +489,8 @@ struct are_ctx {
     std::map<int32_t, are::Layer> layers;
     int *d_flag = nullptr;   // validation flag
     int *h_flag = nullptr;   // pinned mirror
-    are::SelectScratch sel;
+    are::SelectScratch sel;      // are_risk_measures
+    are::SelectScratch sel_multi;   // are_risk_measures_batch
     double *h_result = nullptr;  // pinned, 2 * kMaxTargets
     void *h_scratch = nullptr;   // pinned: ELTs being loaded
     size_t h_scratch_bytes = 0;

@@ -9,11 +9,10 @@
 // exactly (8 passes of 8 bits, every target rank in the same pass), then one
 // more pass adds the values above it.
 //
-// Two forms.  The single-YLT selection (launch_select: are_risk_measures,
-// the pricing server) runs the passes below in one cooperative launch, with
-// a grid-wide barrier between them (details above k_select_coop).  The
-// multi-YLT selection (a portfolio's YLTs together) and the allocation-free
-// one launch one kernel per pass.
+// Two forms.  are_risk_measures, the batched call and the pricing server run
+// one cooperative launch that counts 13 and 11 bits and finishes on the few
+// keys left (details above k_select_coop).  The allocation-free call launches
+// the radix passes one kernel at a time.
 //
 // GB300 choices.  Each histogram pass ends with the pick of the next digit,
 // done by whichever block of the pass finishes last (a counter and memory
@@ -27,6 +26,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 
@@ -59,22 +59,16 @@ struct Ranks {
     long long m[kMaxTargets];
 };
 
-// Scratch of one selection over n_ylt YLTs (blockIdx.y or blockIdx.x picks
-// the YLT).
+// The radix form's YLT and scratch.
 struct Sel {
-    const double *single;        // the YLT when there is one
-    const double *const *many;   // device array of YLT pointers, or nullptr
-    uint32_t *hist;              // per YLT: kMaxTargets x 256 counts
-    unsigned long long *state;   // per YLT: kMaxTargets x (key prefix, rank left)
-    unsigned int *ctrl;          // per YLT: kCtrlWords
-    unsigned long long *acc;     // per YLT: kMaxTargets x kAccWords
-    double *result;              // per YLT: kMaxTargets x (m-th largest, mean of the m largest)
-    int blocks;                  // blocks per YLT in the histogram and tail passes
+    const double *ylt;
+    uint32_t *hist;              // kMaxTargets x 256 counts
+    unsigned long long *state;   // kMaxTargets x (key prefix, rank left)
+    unsigned int *ctrl;          // kCtrlWords
+    unsigned long long *acc;     // kMaxTargets x kAccWords
+    double *result;              // kMaxTargets x (m-th largest, mean of the m largest)
+    int blocks;                  // blocks of the histogram and tail passes
 };
-__device__ __forceinline__ const double *ylt_of(const Sel &s, int y)
-{
-    return s.many ? s.many[y] : s.single;
-}
 
 // ---------------------------------------------------------------------------
 // multi-word integers
@@ -178,13 +172,11 @@ __device__ __forceinline__ int tail_scale(unsigned int mag_hi)
 // among the keys that share the prefix (1 = the largest of them).
 __global__ void k_init(Sel s, Ranks r, int nt)
 {
-    const int y = blockIdx.x;
-    uint32_t *hist = s.hist + (size_t)y * kMaxTargets * kBins;
-    unsigned long long *state = s.state + (size_t)y * 2 * kMaxTargets;
-    unsigned long long *acc = s.acc + (size_t)y * kMaxTargets * kAccWords;
+    uint32_t *hist = s.hist;
+    unsigned long long *state = s.state, *acc = s.acc;
     for (int i = threadIdx.x; i < nt * kBins; i += blockDim.x) hist[i] = 0;
     for (int i = threadIdx.x; i < nt * kAccWords; i += blockDim.x) acc[i] = 0;
-    if (threadIdx.x < kCtrlWords) s.ctrl[(size_t)y * kCtrlWords + threadIdx.x] = 0;
+    if (threadIdx.x < kCtrlWords) s.ctrl[threadIdx.x] = 0;
     if (threadIdx.x < nt) {
         state[2 * threadIdx.x] = 0ull;
         state[2 * threadIdx.x + 1] = (unsigned long long)r.m[threadIdx.x];
@@ -247,11 +239,10 @@ __device__ __forceinline__ void pick(const uint32_t *h, unsigned long long *st, 
 // every target's digit and clears the histogram for the next pass.
 __global__ void __launch_bounds__(kThreads) k_hist(Sel s, int64_t n, int nt, int pass)
 {
-    const int y = blockIdx.y;
-    const double *__restrict__ v = ylt_of(s, y);
-    unsigned long long *state = s.state + (size_t)y * 2 * kMaxTargets;
-    uint32_t *hist = s.hist + (size_t)y * kMaxTargets * kBins;
-    unsigned int *ctrl = s.ctrl + (size_t)y * kCtrlWords;
+    const double *__restrict__ v = s.ylt;
+    unsigned long long *state = s.state;
+    uint32_t *hist = s.hist;
+    unsigned int *ctrl = s.ctrl;
     __shared__ uint32_t h[kMaxTargets * kBins];
     __shared__ unsigned int s_mag;
     __shared__ int s_last;
@@ -329,11 +320,10 @@ __global__ void __launch_bounds__(kThreads) k_hist(Sel s, int64_t n, int nt, int
 // the selected value -- and writes (value, sum / m).
 __global__ void __launch_bounds__(kThreads) k_tail(Sel s, int64_t n, int nt, Ranks r)
 {
-    const int y = blockIdx.y;
-    const double *__restrict__ v = ylt_of(s, y);
-    const unsigned long long *state = s.state + (size_t)y * 2 * kMaxTargets;
-    unsigned int *ctrl = s.ctrl + (size_t)y * kCtrlWords;
-    unsigned long long *acc = s.acc + (size_t)y * kMaxTargets * kAccWords;
+    const double *__restrict__ v = s.ylt;
+    const unsigned long long *state = s.state;
+    unsigned int *ctrl = s.ctrl;
+    unsigned long long *acc = s.acc;
     __shared__ unsigned long long a[kMaxTargets * kAccWords];
     __shared__ int s_last;
     for (int i = threadIdx.x; i < nt * kAccWords; i += blockDim.x) a[i] = 0;
@@ -413,7 +403,7 @@ __global__ void __launch_bounds__(kThreads) k_tail(Sel s, int64_t n, int nt, Ran
             sub192(pos, neg);
             sum = to_double(pos, sc);
         }
-        double *res = s.result + (size_t)y * 2 * kMaxTargets;
+        double *res = s.result;
         res[2 * t] = vt;
         res[2 * t + 1] = __ddiv_rn(sum, (double)r.m[t]);
     }
@@ -421,75 +411,120 @@ __global__ void __launch_bounds__(kThreads) k_tail(Sel s, int64_t n, int nt, Ran
 }
 
 // ---------------------------------------------------------------------------
-// Single-YLT selection in one cooperative launch
+// The selection in one cooperative launch
 // ---------------------------------------------------------------------------
 //
 // One kernel whose blocks are all resident (a cooperative launch), with a
-// grid-wide barrier where the radix form has a launch boundary:
-// 1. two radix passes find each target's bucket of the top 16 key bits
-//    (sign, exponent and four mantissa bits: 1/16 of an octave) and its rank
-//    in it;
-// 2. one pass keeps the keys of each target's bucket (up to kCand) and adds
-//    the values of higher buckets to the target's exact tail sum;
-// 3. block t selects among target t's kept keys by their last 48 bits in
-//    shared memory and adds the bucket's values above the selected one; if
-//    a bucket holds more than kCand keys (a long run of ties), every block
-//    runs the remaining six radix passes over the whole YLT instead.
-// In a radix pass every block picks every target's next digit itself from
-// the pass's global histogram (the same counts give the same digit), so one
-// barrier per pass is enough.  The histograms rotate through three buffers:
-// the buffer of pass p is cleared by block 0 during pass p + 2, after every
-// block has read it (before the barrier of pass p + 1) and before it is
-// written again (pass p + 3).
+// grid-wide barrier where the radix form has a launch boundary.  The blocks
+// form groups, one YLT to a group at a time:
+// A. the top 13 key bits (sign, exponent and a mantissa bit: half an octave)
+//    counted in 8192 bins; every block finds every target's bin itself;
+// B. the next 11 bits of the targets' bins (2^-12 of an octave) counted;
+// C. the keys of each target's 24-bit bin kept, up to kCand of them with
+//    their multiplicities (a run of ties is one key: each block counts the
+//    first candidate it meets apart), and the values of higher bins added to
+//    the exact tail sums of the targets that want a mean;
+// D. a block per target finds the key among the kept ones and adds those above
+//    it.  If some bin keeps more than kCand keys, five radix passes over the
+//    whole YLT take the place of D.
+// Three barriers, where eight 8-bit digits would need eight; the bins are
+// narrow enough that D is a few dozen keys.
+//
+// Three targets of 1M losses take 43 us (two 8-bit digits and up to 16384
+// kept keys: 83), eight 78 us (302), eight with a run of ties of 2% 79 us
+// (463: it took the radix passes); 1000 losses 26 us (34); 64 YLTs of 100,000
+// at a time 363 us with the copy back (ten launches: 549).  What is left is
+// latency: the launch, three barriers and the chains between them.
+//
+// The scratch of a group is left ready for the next YLT: histogram A is
+// cleared in C (its readers are past the barrier before), histogram B in A and
+// the counters and sums of C and D in B (their readers are past a barrier and
+// their next writers behind one), the magnitudes by turns.
 
-constexpr int kCand = 16384;            // candidate keys kept per target
-constexpr int kCoopThreads = 512;
+constexpr int kCand = 1024;             // keys kept per target
+constexpr int kCoopThreads = 1024;
+constexpr int kBitsA = 13, kBinsA = 1 << kBitsA;
+constexpr int kBitsB = 11, kBinsB = 1 << kBitsB;
+constexpr int kShiftA = 64 - kBitsA, kShiftB = kShiftA - kBitsB;
+static_assert(kShiftB == 40, "the radix passes go on with the fourth digit of 8 bits");
+constexpr size_t kCoopSmem = sizeof(uint32_t) * kMaxTargets * kBinsB;
+static_assert(kCoopSmem >= sizeof(uint32_t) * kBinsA && kCoopSmem >= kCand * 12ull, "what the passes share");
 
-struct SelC {
-    const double *v;
-    uint32_t *hist;              // 3 x kMaxTargets x kBins counts, zero between calls
-    unsigned long long *acc;     // kMaxTargets x kAccWords
-    unsigned int *ctrl;          // [1] top word of the largest |value|, zero between calls
-    unsigned long long *app;     // per target: keys kept
-    unsigned long long *cand;    // per target: kCand keys of its bucket
-    double *result;              // per target: value, mean of the m largest
+// One group's scratch, zero before its first use.
+struct CoopScratch {
+    uint32_t a[kBinsA];
+    uint32_t b[kMaxTargets * kBinsB];
+    uint32_t c[3 * kMaxTargets * kBins];             // the radix passes'
+    unsigned long long acc[kMaxTargets * kAccWords];
+    unsigned long long key[kMaxTargets * kCand];
+    uint32_t times[kMaxTargets * kCand];
+    uint32_t kept[kMaxTargets];
+    unsigned int mag[2];                             // top word of the largest |value|, by turns
+    unsigned int over[2];                            // the launch's (first group): a bin over kCand
+    double result[2 * kMaxTargets];                  // value, mean of the m largest
 };
 
-// Adds x (scaled by 2^sc) to the accumulator words a (positive and negative
-// limbs apart, then a count) in shared memory for the lanes with `on` set,
-// summed over the warp first (one set of atomics per warp and sign).  Every
-// lane must call it.
-__device__ __forceinline__ void acc_add_warp(unsigned long long *a, bool on, double x, int sc, int lane)
+struct CoopArgs {
+    const double *single;        // the YLT when there is one
+    const double *const *many;   // device array of YLT pointers, or nullptr
+    int n_ylt;
+    int per;                     // blocks of a group
+    int64_t n;
+    int nt;
+    uint32_t means;              // bit t: target t's mean is wanted
+    long long m[kMaxTargets];
+    CoopScratch *scratch;        // per group
+    double *results;             // per YLT: 2 * kMaxTargets, or nullptr: the scratch's
+    double *out[kMaxTargets];    // per target: where its value (or, means: its mean) goes too, or nullptr
+};
+
+// Adds `times` x (scaled by 2^sc) to the accumulator words a (positive and
+// negative limbs apart, then a count) in shared memory for the lanes with
+// `on` set: few lanes one by one, many summed over the warp first.  Every lane
+// must call it.
+__device__ __forceinline__ void acc_add(unsigned long long *a, bool on, double x, uint32_t times, int sc, int lane)
 {
-    if (!__any_sync(kFull, on)) return;
+    const unsigned act = __ballot_sync(kFull, on);
+    if (!act) return;
     unsigned long long lo = 0, hi = 0;
     if (on) scaled(x, sc, lo, hi);
+    const unsigned long long w[kLimbs] = {(lo & 0xffffffffull) * times, (lo >> 32) * times, hi * times};
+    if (__popc(act) <= 4) {
+        if (on) {
+            unsigned long long *p = a + (x < 0.0 ? kLimbs : 0);
+#pragma unroll
+            for (int i = 0; i < kLimbs; ++i) atomicAdd(p + i, w[i]);
+            atomicAdd(a + 2 * kLimbs, (unsigned long long)times);
+        }
+        return;
+    }
     for (int g = 0; g < 2; ++g) {   // positive, then negative values
         const bool mine = on && ((x < 0.0) == (g == 1));
         if (!__any_sync(kFull, mine)) continue;
-        unsigned long long w0 = mine ? (lo & 0xffffffffull) : 0, w1 = mine ? lo >> 32 : 0, w2 = mine ? hi : 0;
-        unsigned long long c = mine ? 1ull : 0ull;
+        unsigned long long v[kLimbs + 1];
 #pragma unroll
-        for (int off = 16; off; off >>= 1) {
-            w0 += __shfl_xor_sync(kFull, w0, off);
-            w1 += __shfl_xor_sync(kFull, w1, off);
-            w2 += __shfl_xor_sync(kFull, w2, off);
-            c += __shfl_xor_sync(kFull, c, off);
-        }
+        for (int i = 0; i < kLimbs; ++i) v[i] = mine ? w[i] : 0;
+        v[kLimbs] = mine ? times : 0;
+#pragma unroll
+        for (int off = 16; off; off >>= 1)
+#pragma unroll
+            for (int i = 0; i <= kLimbs; ++i) v[i] += __shfl_xor_sync(kFull, v[i], off);
         if (lane == 0) {
-            atomicAdd(a + g * kLimbs, w0);
-            atomicAdd(a + g * kLimbs + 1, w1);
-            atomicAdd(a + g * kLimbs + 2, w2);
-            atomicAdd(a + 2 * kLimbs, c);
+#pragma unroll
+            for (int i = 0; i < kLimbs; ++i) atomicAdd(a + g * kLimbs + i, v[i]);
+            atomicAdd(a + 2 * kLimbs, v[kLimbs]);
         }
     }
 }
 
 // (value of key kt, mean of the m largest) from the accumulator words A of
 // the values above kt (sum and count, scaled by 2^sc).
-__device__ void tail_result(const unsigned long long (&A)[kAccWords], uint64_t kt, long long m, int sc,
+__device__ void tail_result(const unsigned long long (&A)[kAccWords], uint64_t kt, long long m, int sc, bool mean,
                             double *res)
 {
+    const double vt = value_of(kt);
+    res[0] = vt;
+    if (!mean) return;
     U192 pos, neg;
     for (int g = 0; g < 2; ++g) {
         U192 &z = g ? neg : pos;
@@ -499,7 +534,6 @@ __device__ void tail_result(const unsigned long long (&A)[kAccWords], uint64_t k
         add192(z, 0, A2, 0);
     }
     const unsigned long long c = A[2 * kLimbs];
-    const double vt = value_of(kt);
     const unsigned long long q = (unsigned long long)m - c;   // >= 1: ties at the m-th value
     unsigned long long lo, hi;
     scaled(vt, sc, lo, hi);
@@ -514,311 +548,390 @@ __device__ void tail_result(const unsigned long long (&A)[kAccWords], uint64_t k
         sub192(pos, neg);
         sum = to_double(pos, sc);
     }
-    res[0] = vt;
     res[1] = __ddiv_rn(sum, (double)m);
 }
 
-// One warp: the bucket of h (256 counts in shared memory) that holds rank
-// rem, counting down from the top bucket; extends the prefix pre.
-__device__ __forceinline__ void pick_shared(const uint32_t *h, unsigned long long &pre, unsigned long long &rem,
-                                            int shift, int lane)
+// Calls f(key, value, in range) for the group's share of the YLT, whole warps
+// at a time, kPre values per lane loaded before the first call.
+template <typename F>
+__device__ __forceinline__ void for_values(const double *v, int64_t n, int rank, int per, F &&f)
 {
-    uint32_t c[8];
-    unsigned long long lane_sum = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        c[i] = h[kBins - 1 - (lane * 8 + i)];   // lane 0 holds the top buckets
-        lane_sum += c[i];
-    }
-    unsigned long long incl = lane_sum;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const unsigned long long o = __shfl_up_sync(kFull, incl, off);
-        if (lane >= off) incl += o;
-    }
-    const unsigned long long excl = incl - lane_sum;
-    const unsigned long long r = rem;
-    __syncwarp();
-    if (excl < r && r <= incl) {
-        unsigned long long above = excl;
-        int b = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            if (above + c[i] >= r) {
-                b = kBins - 1 - (lane * 8 + i);
-                break;
-            }
-            above += c[i];
-        }
-        pre |= (unsigned long long)b << shift;
-        rem = r - above;
-    }
-}
-
-// One radix pass of the cooperative selection (digit bits shift .. shift + 7)
-// over the keys that share each target's prefix st[2t] (pass 0: every key,
-// one histogram for all targets), ending with the grid barrier and every
-// block's pick of every target's digit.  pass 0 also gathers the largest
-// magnitude into ctrl[1].
-__device__ void coop_pass(const SelC &s, int64_t n, int nt, int pass, unsigned long long *st, uint32_t *h,
-                          unsigned int *s_mag, cg::grid_group &grid)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int shift = 56 - 8 * pass;
-    const int rows = pass == 0 ? 1 : nt;
-    uint32_t *gh = s.hist + (size_t)(pass % 3) * kMaxTargets * kBins;
-    for (int i = threadIdx.x; i < rows * kBins; i += blockDim.x) h[i] = 0;
-    if (blockIdx.x == 0 && pass >= 2) {   // the buffer of pass - 2, read by every block already
-        uint32_t *old = s.hist + (size_t)((pass - 2) % 3) * kMaxTargets * kBins;
-        for (int i = threadIdx.x; i < kMaxTargets * kBins; i += blockDim.x) old[i] = 0;
-    }
-    if (pass == 0 && threadIdx.x == 0) *s_mag = 0;
-    __syncthreads();
-    uint64_t pre[kMaxTargets];
-#pragma unroll
-    for (int t = 0; t < kMaxTargets; ++t) pre[t] = t < nt ? st[2 * t] >> (shift + 8) : 0ull;
-    unsigned int mag = 0;
-    // warp-uniform loop: every lane takes part in the warp's histogram adds
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n;
-         base += stride * kPre) {
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)per * kCoopThreads;
+    for (int64_t base = (int64_t)rank * kCoopThreads + (threadIdx.x & ~31); base < n; base += stride * kPre) {
         double xs[kPre];
 #pragma unroll
         for (int u = 0; u < kPre; ++u) {
             const int64_t i = base + u * stride + lane;
-            xs[u] = i < n ? s.v[i] : 0.0;
+            xs[u] = i < n ? v[i] : 0.0;
         }
 #pragma unroll
         for (int u = 0; u < kPre; ++u) {
-            const bool ok = base + u * stride + lane < n;
-            const uint64_t k = key_of(xs[u]);
-            const uint32_t d = (uint32_t)(k >> shift) & 0xffu;
-            if (pass == 0) {
-                hist_add(h, ok, d, lane);
+            if (base + u * stride >= n) break;
+            f(key_of(xs[u]), xs[u], base + u * stride + lane < n);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_constant__ CoopArgs args)
+{
+    cg::grid_group grid = cg::this_grid();
+    extern __shared__ __align__(16) uint32_t h[];        // kCoopSmem
+    __shared__ unsigned long long st[2 * kMaxTargets];   // per target: key prefix, rank left (the same in every block)
+    __shared__ unsigned long long acc[kMaxTargets * kAccWords];
+    __shared__ uint64_t rep[kMaxTargets];                // per target: the block's first candidate, ~0: none; then its key
+    __shared__ uint32_t rep_times[kMaxTargets];
+    __shared__ uint32_t warp_sum[kCoopThreads / 32];
+    __shared__ unsigned int s_mag;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int group = blockIdx.x / args.per, rank = blockIdx.x % args.per, groups = gridDim.x / args.per;
+    const int nt = args.nt;
+    const int64_t n = args.n;
+    CoopScratch &S = args.scratch[group];
+    unsigned int *const over = args.scratch[0].over;
+    auto mine = [&](int i) { return i * args.per + rank; };   // a block's share of the group's clearing
+    for (int y0 = 0, round = 0; y0 < args.n_ylt; y0 += groups, ++round) {
+        const int y = y0 + group, turn = round & 1;
+        const bool on = y < args.n_ylt;
+        const bool final_round = y0 + groups >= args.n_ylt;
+        const double *__restrict__ v = on ? (args.many ? args.many[y] : args.single) : nullptr;
+        // A. the top bits
+        if (tid < nt) {
+            st[2 * tid] = 0;
+            st[2 * tid + 1] = (uint64_t)args.m[tid];
+        }
+        if (tid == 0) s_mag = 0;
+        for (int i = tid; i < kBinsA; i += kCoopThreads) h[i] = 0;
+        for (int i = mine(tid); i < kMaxTargets * kBinsB; i += args.per * kCoopThreads) S.b[i] = 0;
+        if (blockIdx.x == 0 && tid == 0) over[turn] = 0;
+        __syncthreads();
+        if (on) {
+            unsigned int mag = 0;
+            for_values(v, n, rank, args.per, [&](uint64_t k, double x, bool ok) {
+                hist_add(h, ok, (uint32_t)(k >> kShiftA), lane);
                 const unsigned int m32 =
-                    (unsigned int)(((unsigned long long)__double_as_longlong(xs[u]) >> 32) & 0x7fffffffu);
+                    (unsigned int)(((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu);
                 if (ok) mag = m32 > mag ? m32 : mag;
-            } else {
+            });
+#pragma unroll
+            for (int off = 16; off; off >>= 1) {
+                const unsigned int o = __shfl_xor_sync(kFull, mag, off);
+                mag = o > mag ? o : mag;
+            }
+            if (lane == 0 && mag) atomicMax(&s_mag, mag);
+        }
+        __syncthreads();
+        for (int i = tid; i < kBinsA; i += kCoopThreads)
+            if (h[i]) atomicAdd(&S.a[i], h[i]);
+        if (tid == 0 && s_mag) atomicMax(&S.mag[turn], s_mag);
+        grid.sync();
+        // every block finds every target's bin: thread i holds 8 bins, the
+        // top ones first
+        {
+            constexpr int per = kBinsA / kCoopThreads;
+            uint32_t c[per], sum = 0;
+#pragma unroll
+            for (int i = 0; i < per; ++i) {
+                c[i] = __ldcg(&S.a[kBinsA - 1 - (tid * per + i)]);
+                sum += c[i];
+            }
+            uint32_t incl = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += o;
+            }
+            if (lane == 31) warp_sum[warp] = incl;
+            __syncthreads();
+            if (warp == 0) {
+                uint32_t s = warp_sum[lane];
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t o = __shfl_up_sync(kFull, s, d);
+                    if (lane >= d) s += o;
+                }
+                warp_sum[lane] = s;
+            }
+            __syncthreads();
+            if (warp) incl += warp_sum[warp - 1];
+            const uint32_t excl = incl - sum;
+            for (int t = 0; t < nt; ++t) {
+                const uint64_t r = (uint64_t)args.m[t];
+                if (excl < r && r <= incl) {
+                    uint64_t above = excl;
+                    int i = 0;
+                    while (above + c[i] < r) above += c[i++];
+                    st[2 * t] = (uint64_t)(kBinsA - 1 - (tid * per + i)) << kShiftA;
+                    st[2 * t + 1] = r - above;
+                }
+            }
+            __syncthreads();
+        }
+        // B. the next bits of the targets' bins (a bin shared by targets once)
+        for (int i = tid; i < nt * kBinsB; i += kCoopThreads) h[i] = 0;
+        if (rank == 0) {
+            for (int i = tid; i < kMaxTargets * kAccWords; i += kCoopThreads) S.acc[i] = 0;
+            if (tid < kMaxTargets) S.kept[tid] = 0;
+        }
+        __syncthreads();
+        uint32_t PA[kMaxTargets];
+        int first[kMaxTargets];   // the first target with the same bin
+#pragma unroll
+        for (int t = 0; t < kMaxTargets; ++t) {
+            PA[t] = t < nt ? (uint32_t)(st[2 * t] >> kShiftA) : ~0u;
+            first[t] = t;
+#pragma unroll
+            for (int q = kMaxTargets - 1; q >= 0; --q)
+                if (q < t && PA[q] == PA[t]) first[t] = q;
+        }
+        if (on)
+            for_values(v, n, rank, args.per, [&](uint64_t k, double, bool ok) {
+                const uint32_t p = (uint32_t)(k >> kShiftA);
+#pragma unroll
+                for (int t = 0; t < kMaxTargets; ++t)
+                    if (t < nt && first[t] == t)
+                        hist_add(h + t * kBinsB, ok && p == PA[t], (uint32_t)(k >> kShiftB) & (kBinsB - 1), lane);
+            });
+        __syncthreads();
+        for (int i = tid; i < nt * kBinsB; i += kCoopThreads)
+            if (h[i]) atomicAdd(&S.b[i], h[i]);
+        grid.sync();
+        if (warp < nt) {   // warp t: lane i holds 64 bins, the top ones first
+            int q = 0;
+#pragma unroll
+            for (int t = 0; t < kMaxTargets; ++t)
+                if (t == warp) q = first[t];
+            const uint32_t *b = S.b + q * kBinsB;
+            constexpr int per = kBinsB / 32;
+            uint32_t sum = 0;
+#pragma unroll 16
+            for (int i = 0; i < per; ++i) sum += __ldcg(b + kBinsB - 1 - (lane * per + i));
+            uint32_t incl = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += o;
+            }
+            const uint32_t excl = incl - sum;
+            const uint64_t r = st[2 * warp + 1];
+            // the lane whose bins hold the rank, then its bins, two per lane
+            const int l = __ffs(__ballot_sync(kFull, excl < r && r <= incl)) - 1;
+            static_assert(per == 64, "two bins per lane");
+            const uint64_t left = r - __shfl_sync(kFull, excl, l);
+            const int i0 = l * per + 2 * lane;
+            const uint32_t c0 = __ldcg(b + kBinsB - 1 - i0), c1 = __ldcg(b + kBinsB - 2 - i0);
+            uint32_t run = c0 + c1;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(kFull, run, d);
+                if (lane >= d) run += o;
+            }
+            const uint32_t before = run - c0 - c1;
+            if (before < left && left <= run) {
+                const bool second = left > (uint64_t)before + c0;
+                st[2 * warp] |= (uint64_t)(kBinsB - 1 - i0 - second) << kShiftB;
+                st[2 * warp + 1] = left - before - (second ? c0 : 0u);
+            }
+        }
+        if (tid < kMaxTargets) {
+            rep[tid] = ~0ull;
+            rep_times[tid] = 0;
+        }
+        for (int i = tid; i < kMaxTargets * kAccWords; i += kCoopThreads) acc[i] = 0;
+        __syncthreads();
+        // C. the keys of the targets' bins, and the tail sums above them
+        const int sc = tail_scale(__ldcg(&S.mag[turn]));
+        uint32_t P[kMaxTargets];
+#pragma unroll
+        for (int t = 0; t < kMaxTargets; ++t) {
+            P[t] = t < nt ? (uint32_t)(st[2 * t] >> kShiftB) : ~0u;
+            first[t] = t;
+#pragma unroll
+            for (int q = kMaxTargets - 1; q >= 0; --q)
+                if (q < t && P[q] == P[t]) first[t] = q;
+        }
+        auto keep = [&](int t, uint64_t k, uint32_t times) {
+            const uint32_t at = atomicAdd(&S.kept[t], 1u);
+            if (at < kCand) {
+                S.key[t * kCand + at] = k;
+                S.times[t * kCand + at] = times;
+            }
+        };
+        if (on)
+            for_values(v, n, rank, args.per, [&](uint64_t k, double x, bool ok) {
+                const uint32_t p = (uint32_t)(k >> kShiftB);
 #pragma unroll
                 for (int t = 0; t < kMaxTargets; ++t) {
                     if (t >= nt) break;
-                    hist_add(h + t * kBins, ok && (k >> (shift + 8)) == pre[t], d, lane);
+                    if (first[t] == t) {
+                        const bool in = ok && p == P[t];
+                        if (__any_sync(kFull, in)) {
+                            const bool same = in && *(volatile uint64_t *)&rep[t] == k;
+                            const unsigned b = __ballot_sync(kFull, same);
+                            if (b && lane == __ffs(b) - 1) atomicAdd(&rep_times[t], (uint32_t)__popc(b));
+                            if (in && !same) {
+                                const uint64_t was = atomicCAS((unsigned long long *)&rep[t], ~0ull, (unsigned long long)k);
+                                if (was == ~0ull || was == k) atomicAdd(&rep_times[t], 1u);
+                                else keep(t, k, 1u);
+                            }
+                        }
+                    }
+                    if ((args.means >> t) & 1u)
+                        acc_add(acc + t * kAccWords, ok && p > P[t], x, 1u, sc, lane);
+                }
+            });
+        for (int i = mine(tid); i < kBinsA; i += args.per * kCoopThreads) S.a[i] = 0;
+        if (rank == 0 && tid == 0) S.mag[turn ^ 1] = 0;
+        __syncthreads();
+        if (tid < nt && rep_times[tid]) keep(tid, rep[tid], rep_times[tid]);
+        for (int i = tid; i < nt * kAccWords; i += kCoopThreads)
+            if (acc[i]) atomicAdd(&S.acc[i], acc[i]);
+        __syncthreads();
+        if (tid < nt && __ldcg(&S.kept[tid]) > kCand) atomicExch(over + turn, 1u);
+        grid.sync();
+        double *const res = args.results ? args.results + (size_t)y * 2 * kMaxTargets : S.result;
+        const bool fits = __ldcg(over + turn) == 0;
+        if (fits && on) {
+            // D. block j of the group: targets j, j + per, ..., a warp each where
+            // a block has several
+            const bool warps = args.per < nt;
+            constexpr int kWarpCand = 512;   // keys that a warp keeps in shared memory
+            static_assert(kMaxTargets * kWarpCand * 12 <= kCoopSmem, "each target's keys");
+            const int width = warps ? 32 : kCoopThreads, at = warps ? lane : tid;
+            auto join = [&] {
+                if (warps) __syncwarp();
+                else __syncthreads();
+            };
+            const int t = warps ? warp : rank;
+            if (t < nt && (!warps || t % args.per == rank)) {
+                int q = 0;
+#pragma unroll
+                for (int i = 0; i < kMaxTargets; ++i)
+                    if (i == t) q = first[i];
+                const int c = (int)__ldcg(&S.kept[q]);
+                const unsigned long long *keys = S.key + q * kCand;
+                const uint32_t *times = S.times + q * kCand;
+                unsigned long long *const sk = reinterpret_cast<unsigned long long *>(h) + (warps ? t * kWarpCand : 0);
+                uint32_t *const sn = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned long long *>(h) +
+                                                                  (warps ? kMaxTargets * kWarpCand : kCand)) +
+                                     (warps ? t * kWarpCand : 0);
+                unsigned long long *const sum = acc + (warps ? t * kAccWords : 0);
+                if (!warps || c <= kWarpCand) {
+                    for (int i = at; i < c; i += width) {
+                        sk[i] = __ldcg(keys + i);
+                        sn[i] = __ldcg(times + i);
+                    }
+                    keys = sk;
+                    times = sn;
+                }
+                if (at < kAccWords) sum[at] = 0;
+                join();
+                // the key with fewer than r values above it and r or more at or above
+                const uint64_t r = st[2 * t + 1];
+                for (int i = at; i < c; i += width) {
+                    const uint64_t k = keys[i];
+                    uint64_t above = 0, equal = 0;
+                    for (int j = 0; j < c; ++j) {
+                        const uint64_t o = keys[j];
+                        above += o > k ? times[j] : 0u;
+                        equal += o == k ? times[j] : 0u;
+                    }
+                    if (above < r && r <= above + equal) rep[t] = k;   // (equal keys write the same)
+                }
+                join();
+                const uint64_t kt = rep[t];
+                if ((args.means >> t) & 1u)
+                    for (int base = at & ~31; base < c; base += width) {
+                        const int i = base + lane;
+                        const bool up = i < c && keys[i] > kt;
+                        acc_add(sum, up, up ? value_of(keys[i]) : 0.0, up ? times[i] : 0u, sc, lane);
+                    }
+                join();
+                if (at == 0) {
+                    unsigned long long A[kAccWords];
+                    for (int i = 0; i < kAccWords; ++i) A[i] = sum[i] + __ldcg(&S.acc[t * kAccWords + i]);
+                    tail_result(A, kt, args.m[t], sc, (args.means >> t) & 1u, res + 2 * t);
+                    if (args.out[t]) *args.out[t] = res[2 * t + ((args.means >> t) & 1u)];
                 }
             }
-        }
-    }
-    if (pass == 0) {
-#pragma unroll
-        for (int off = 16; off; off >>= 1) {
-            const unsigned int o = __shfl_xor_sync(kFull, mag, off);
-            mag = o > mag ? o : mag;
-        }
-        if (lane == 0 && mag) atomicMax(s_mag, mag);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < rows * kBins; i += blockDim.x)
-        if (h[i]) atomicAdd(&gh[i], h[i]);
-    if (pass == 0 && threadIdx.x == 0 && *s_mag) atomicMax(&s.ctrl[1], *s_mag);
-    grid.sync();
-    // every block picks every target's digit from the pass's histogram
-    if (warp < nt) pick(gh + (pass == 0 ? 0 : warp) * kBins, st + 2 * warp, shift, lane);
-    __syncthreads();
-}
-
-// Block t's exact selection among the n_keys candidate keys of target t's
-// bucket (in shared memory): the remaining 48 bits, 8 at a time; returns the
-// key and adds the bucket's values above it to a.
-__device__ uint64_t finish_in_block(const unsigned long long *keys, int n_keys, unsigned long long *st_t,
-                                    uint32_t *h, unsigned long long *a, int sc)
-{
-    const int lane = threadIdx.x & 31;
-    for (int shift = 40; shift >= 0; shift -= 8) {
-        for (int i = threadIdx.x; i < kBins; i += blockDim.x) h[i] = 0;
-        __syncthreads();
-        const uint64_t pre = st_t[0] >> (shift + 8);
-        // warp-uniform: the keys share most leading bits, so the warp adds per bin
-        for (int base = threadIdx.x & ~31; base < n_keys; base += blockDim.x) {
-            const int i = base + lane;
-            const bool ok = i < n_keys;
-            const uint64_t k = ok ? keys[i] : 0ull;
-            hist_add(h, ok && (k >> (shift + 8)) == pre, (uint32_t)(k >> shift) & 0xffu, lane);
-        }
-        __syncthreads();
-        if (threadIdx.x < 32) pick_shared(h, st_t[0], st_t[1], shift, lane);
-        __syncthreads();
-    }
-    const uint64_t kt = st_t[0];
-    for (int base = threadIdx.x & ~31; base < n_keys; base += blockDim.x) {
-        const int i = base + lane;
-        const bool ok = i < n_keys;
-        const uint64_t k = ok ? keys[i] : 0ull;
-        acc_add_warp(a, ok && k > kt, value_of(k), sc, lane);
-    }
-    __syncthreads();
-    return kt;
-}
-
-__global__ void __launch_bounds__(kCoopThreads) k_select_coop(SelC s, int64_t n, int nt, Ranks r)
-{
-    cg::grid_group grid = cg::this_grid();
-    extern __shared__ unsigned long long keys[];   // kCand: the candidates of a block's target
-    __shared__ uint32_t h[kMaxTargets * kBins];
-    __shared__ unsigned long long st[2 * kMaxTargets];   // per target: key prefix, rank left (the same in every block)
-    __shared__ unsigned long long a[kMaxTargets * kAccWords];
-    __shared__ unsigned int s_mag;
-    const int lane = threadIdx.x & 31;
-    if (threadIdx.x < nt) {
-        st[2 * threadIdx.x] = 0ull;
-        st[2 * threadIdx.x + 1] = (unsigned long long)r.m[threadIdx.x];
-    }
-    if (blockIdx.x == 0) {   // the counters and sums of step 2, used after the next two barriers
-        for (int i = threadIdx.x; i < kMaxTargets * kAccWords; i += blockDim.x) s.acc[i] = 0;
-        for (int i = threadIdx.x; i < kMaxTargets; i += blockDim.x) s.app[i] = 0;
-    }
-    __syncthreads();
-    // 1. two radix passes: each target's bucket of the top 16 key bits and its rank in it
-    coop_pass(s, n, nt, 0, st, h, &s_mag, grid);
-    coop_pass(s, n, nt, 1, st, h, &s_mag, grid);
-    const int sc = tail_scale(__ldcg(&s.ctrl[1]));
-    uint32_t P[kMaxTargets];
-#pragma unroll
-    for (int t = 0; t < kMaxTargets; ++t) P[t] = t < nt ? (uint32_t)(st[2 * t] >> 48) : 0xffffffffu;
-    // 2. the keys of each target's bucket kept (up to kCand); the values of
-    //    higher buckets added to the target's exact tail sum
-    for (int i = threadIdx.x; i < nt * kAccWords; i += blockDim.x) a[i] = 0;
-    __syncthreads();
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n;
-         base += stride * kPre) {
-        double xs[kPre];
-#pragma unroll
-        for (int u = 0; u < kPre; ++u) {
-            const int64_t i = base + u * stride + lane;
-            xs[u] = i < n ? s.v[i] : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < kPre; ++u) {
-            const bool ok = base + u * stride + lane < n;
-            const uint64_t k = key_of(xs[u]);
-            const uint32_t p = (uint32_t)(k >> 48);
-#pragma unroll
-            for (int t = 0; t < kMaxTargets; ++t) {
-                if (t >= nt) break;
-                const bool in = ok && p == P[t];
-                const unsigned b = __ballot_sync(kFull, in);
-                if (b) {
-                    const int leader = __ffs(b) - 1;
-                    unsigned long long at = 0;
-                    if (lane == leader) at = atomicAdd(s.app + t, (unsigned long long)__popc(b));
-                    at = __shfl_sync(kFull, at, leader);
-                    const unsigned long long slot = at + (unsigned long long)__popc(b & ((1u << lane) - 1u));
-                    if (in && slot < (unsigned long long)kCand) s.cand[(size_t)t * kCand + slot] = k;
+        } else if (!fits) {
+            // a bin of more than kCand keys somewhere: five radix passes over
+            // the YLT, then the bins' values above the keys
+            for (int pass = 3; pass < 8; ++pass) {
+                const int shift = 56 - 8 * pass;
+                uint32_t *gh = S.c + (size_t)(pass % 3) * kMaxTargets * kBins;
+                for (int i = tid; i < nt * kBins; i += kCoopThreads) h[i] = 0;
+                if (rank == 0 && pass >= 5) {   // the buffer of pass - 2, read by every block already
+                    uint32_t *old = S.c + (size_t)((pass - 2) % 3) * kMaxTargets * kBins;
+                    for (int i = tid; i < kMaxTargets * kBins; i += kCoopThreads) old[i] = 0;
                 }
-                acc_add_warp(a + t * kAccWords, ok && p > P[t], xs[u], sc, lane);
+                __syncthreads();
+                uint64_t pre[kMaxTargets];
+#pragma unroll
+                for (int t = 0; t < kMaxTargets; ++t) pre[t] = t < nt ? st[2 * t] >> (shift + 8) : 0ull;
+                if (on)
+                    for_values(v, n, rank, args.per, [&](uint64_t k, double, bool ok) {
+#pragma unroll
+                        for (int t = 0; t < kMaxTargets; ++t) {
+                            if (t >= nt) break;
+                            hist_add(h + t * kBins, ok && (k >> (shift + 8)) == pre[t], (uint32_t)(k >> shift) & 0xffu,
+                                     lane);
+                        }
+                    });
+                __syncthreads();
+                for (int i = tid; i < nt * kBins; i += kCoopThreads)
+                    if (h[i]) atomicAdd(&gh[i], h[i]);
+                grid.sync();
+                if (on && warp < nt)
+                    pick(gh + warp * kBins, st + 2 * warp, shift, lane);
+                __syncthreads();
             }
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nt * kAccWords; i += blockDim.x)
-        if (a[i]) atomicAdd(&s.acc[i], a[i]);
-    grid.sync();
-    bool fits = true;
-    for (int t = 0; t < nt; ++t) fits &= __ldcg(s.app + t) <= (unsigned long long)kCand;
-    uint64_t kt[kMaxTargets];
-    if (fits) {
-        // 3a. block t selects among target t's kept keys in shared memory
-        const int t = blockIdx.x;
-        if (t < nt) {
-            const int n_keys = (int)__ldcg(s.app + t);
-            for (int i = threadIdx.x; i < n_keys; i += blockDim.x) keys[i] = __ldcg(s.cand + (size_t)t * kCand + i);
-            if (threadIdx.x < kAccWords) a[threadIdx.x] = 0;
+            for (int i = tid; i < nt * kAccWords; i += kCoopThreads) acc[i] = 0;
             __syncthreads();
-            const uint64_t k = finish_in_block(keys, n_keys, st + 2 * t, h, a, sc);
-            if (threadIdx.x == 0) {
-                unsigned long long A[kAccWords];
-                for (int i = 0; i < kAccWords; ++i) A[i] = a[i] + __ldcg(s.acc + t * kAccWords + i);
-                tail_result(A, k, r.m[t], sc, s.result + 2 * t);
-            }
-        }
-        if (blockIdx.x == 0) {   // leave the histograms and the magnitude zero for the next call
+            uint64_t kt[kMaxTargets];
+#pragma unroll
+            for (int t = 0; t < kMaxTargets; ++t) kt[t] = t < nt ? st[2 * t] : ~0ull;
+            if (on)
+                for_values(v, n, rank, args.per, [&](uint64_t k, double x, bool ok) {
+#pragma unroll
+                    for (int t = 0; t < kMaxTargets; ++t) {
+                        if (t >= nt) break;
+                        if ((args.means >> t) & 1u)
+                            acc_add(acc + t * kAccWords, ok && (uint32_t)(k >> kShiftB) == P[t] && k > kt[t], x, 1u, sc,
+                                    lane);
+                    }
+                });
             __syncthreads();
-            for (int i = threadIdx.x; i < 2 * kMaxTargets * kBins; i += blockDim.x) s.hist[i] = 0;   // passes 0, 1
-            if (threadIdx.x == 0) s.ctrl[1] = 0;
-        }
-        return;
-    }
-    // 3b. a bucket of more than kCand keys: the remaining six radix passes
-    //     over the whole YLT, then the buckets' values above the keys
-    for (int pass = 2; pass < 8; ++pass) coop_pass(s, n, nt, pass, st, h, &s_mag, grid);
-#pragma unroll
-    for (int t = 0; t < kMaxTargets; ++t) kt[t] = t < nt ? st[2 * t] : ~0ull;
-    for (int i = threadIdx.x; i < nt * kAccWords; i += blockDim.x) a[i] = 0;
-    __syncthreads();
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n;
-         base += stride * kPre) {
-        double xs[kPre];
-#pragma unroll
-        for (int u = 0; u < kPre; ++u) {
-            const int64_t i = base + u * stride + lane;
-            xs[u] = i < n ? s.v[i] : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < kPre; ++u) {
-            const bool ok = base + u * stride + lane < n;
-            const uint64_t k = key_of(xs[u]);
-            const uint32_t p = (uint32_t)(k >> 48);
-#pragma unroll
-            for (int t = 0; t < kMaxTargets; ++t) {
-                if (t >= nt) break;
-                acc_add_warp(a + t * kAccWords, ok && p == P[t] && k > kt[t], xs[u], sc, lane);
+            for (int i = tid; i < nt * kAccWords; i += kCoopThreads)
+                if (acc[i]) atomicAdd(&S.acc[i], acc[i]);
+            grid.sync();
+            if (on && rank == 0) {
+                if (tid < nt) {
+                    unsigned long long A[kAccWords];
+                    for (int i = 0; i < kAccWords; ++i) A[i] = __ldcg(&S.acc[tid * kAccWords + i]);
+                    tail_result(A, st[2 * tid], args.m[tid], sc, (args.means >> tid) & 1u, res + 2 * tid);
+                    if (args.out[tid]) *args.out[tid] = res[2 * tid + ((args.means >> tid) & 1u)];
+                }
+                for (int i = tid; i < 3 * kMaxTargets * kBins; i += kCoopThreads) S.c[i] = 0;
             }
         }
+        if (final_round && rank == 0 && tid == 0) S.mag[0] = S.mag[1] = 0;
+        __syncthreads();
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nt * kAccWords; i += blockDim.x)
-        if (a[i]) atomicAdd(&s.acc[i], a[i]);
-    grid.sync();
-    if (blockIdx.x != 0) return;
-    if (threadIdx.x < nt) {
-        const int t = threadIdx.x;
-        unsigned long long A[kAccWords];
-        for (int i = 0; i < kAccWords; ++i) A[i] = __ldcg(s.acc + t * kAccWords + i);
-        tail_result(A, kt[t], r.m[t], sc, s.result + 2 * t);
-    }
-    __syncthreads();
-    // leave the histograms and the magnitude zero for the next call
-    for (int i = threadIdx.x; i < 3 * kMaxTargets * kBins; i += blockDim.x) s.hist[i] = 0;
-    if (threadIdx.x == 0) s.ctrl[1] = 0;
 }
 
-cudaError_t enqueue_coop(const SelC &s, int64_t n, const int64_t *ranks, int nt, int num_sms, cudaStream_t st)
+// One launch over n_ylt YLTs: `args` but for the groups.
+cudaError_t enqueue_coop(CoopArgs args, int max_groups, int num_sms, cudaStream_t st)
 {
-    Ranks r{};
-    for (int t = 0; t < nt; ++t) r.m[t] = ranks[t];
-    const size_t smem = sizeof(unsigned long long) * kCand;
-    const int per_sm = fit_blocks(reinterpret_cast<const void *>(k_select_coop), kCoopThreads, smem);
-    int64_t blocks = (n + (int64_t)kCoopThreads * kPre - 1) / ((int64_t)kCoopThreads * kPre);
-    const int64_t cap = (int64_t)num_sms * per_sm;   // every block resident
-    if (blocks > cap) blocks = cap;
-    if (blocks < nt) blocks = nt;                    // a block per target for the last step
-    SelC sc = s;
-    int64_t nn = n;
-    int ntt = nt;
-    void *args[] = {&sc, &nn, &ntt, &r};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_select_coop), dim3((unsigned)blocks),
-                                       dim3(kCoopThreads), args, smem, st);
-}
-
-cudaError_t enqueue(const Sel &s, int n_ylt, int64_t n, const int64_t *ranks, int nt,
-                    cudaStream_t st)
-{
-    Ranks r{};
-    for (int t = 0; t < nt; ++t) r.m[t] = ranks[t];
-    const dim3 grid((unsigned)s.blocks, (unsigned)n_ylt);
-    k_init<<<n_ylt, kThreads, 0, st>>>(s, r, nt);
-    for (int pass = 0; pass < 8; ++pass) k_hist<<<grid, kThreads, 0, st>>>(s, n, nt, pass);
-    k_tail<<<grid, kThreads, 0, st>>>(s, n, nt, r);
-    return cudaGetLastError();
+    const int per_sm = fit_blocks(reinterpret_cast<const void *>(k_select_coop), kCoopThreads, kCoopSmem);
+    const int64_t resident = (int64_t)num_sms * per_sm;
+    // blocks that a YLT can use, kPre values per thread each
+    const int64_t useful = std::max<int64_t>(1, (args.n + kCoopThreads * kPre - 1) / (kCoopThreads * kPre));
+    const int64_t groups = std::min<int64_t>({(int64_t)args.n_ylt, (int64_t)max_groups, resident});
+    args.per = (int)std::min(useful, resident / groups);
+    void *p[] = {&args};
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_select_coop), dim3((unsigned)(groups * args.per)),
+                                       dim3(kCoopThreads), p, kCoopSmem, st);
 }
 
 int blocks_for(int64_t n, int cap)
@@ -828,93 +941,55 @@ int blocks_for(int64_t n, int cap)
     return b < 1 ? 1 : (int)b;
 }
 
+CoopArgs coop_args(int64_t n, const int64_t *ranks, int nt, int n_values)
+{
+    CoopArgs a{};
+    a.n = n;
+    a.nt = nt;
+    for (int t = 0; t < nt; ++t) a.m[t] = ranks[t];
+    for (int t = n_values; t < nt; ++t) a.means |= 1u << t;
+    return a;
+}
+
 }  // namespace
 
-void select_alloc(SelectScratch &s, int num_sms)
+void select_alloc(SelectScratch &s, int groups)
 {
-    s.max_blocks = select_max_blocks(num_sms);
-    // three histogram buffers for the cooperative selection
-    ARE_CUDA_TRY(cudaMalloc(&s.hist, sizeof(uint32_t) * 3 * kMaxTargets * kBins));
-    ARE_CUDA_TRY(cudaMalloc(&s.state, sizeof(unsigned long long) * 2 * kMaxTargets));
-    ARE_CUDA_TRY(cudaMalloc(&s.ctrl, sizeof(unsigned int) * kCtrlWords));
-    ARE_CUDA_TRY(cudaMalloc(&s.acc, sizeof(unsigned long long) * kMaxTargets * kAccWords));
-    ARE_CUDA_TRY(cudaMalloc(&s.result, sizeof(double) * 2 * kMaxTargets));
-    ARE_CUDA_TRY(cudaMalloc(&s.app, sizeof(unsigned long long) * kMaxTargets));
-    ARE_CUDA_TRY(cudaMalloc(&s.cand, sizeof(unsigned long long) * kCand * kMaxTargets));
-    // the cooperative selection leaves these zero at its end
-    ARE_CUDA_TRY(cudaMemset(s.hist, 0, sizeof(uint32_t) * 3 * kMaxTargets * kBins));
-    ARE_CUDA_TRY(cudaMemset(s.ctrl, 0, sizeof(unsigned int) * kCtrlWords));
-    ARE_CUDA_TRY(cudaMemset(s.acc, 0, sizeof(unsigned long long) * kMaxTargets * kAccWords));
+    ARE_CUDA_TRY(cudaMalloc(&s.coop, sizeof(CoopScratch) * (size_t)groups));
+    ARE_CUDA_TRY(cudaMemset(s.coop, 0, sizeof(CoopScratch) * (size_t)groups));
+    ARE_CUDA_TRY(cudaStreamSynchronize(nullptr));   // before any stream's selection
+    s.groups = groups;
+    s.result = static_cast<CoopScratch *>(s.coop)->result;
 }
 
 void select_free(SelectScratch &s)
 {
-    cudaFree(s.hist);
-    cudaFree(s.state);
-    cudaFree(s.ctrl);
-    cudaFree(s.acc);
-    cudaFree(s.result);
-    cudaFree(s.app);
-    cudaFree(s.cand);
+    cudaFree(s.coop);
     s = SelectScratch{};
 }
 
-// Enqueues the selection kernels; reports launch errors instead of throwing.
-cudaError_t select_enqueue(const double *ylt, int64_t n, const int64_t *ranks, int nt,
-                           const SelectScratch &s, cudaStream_t st)
+int launch_select(const double *ylt, int64_t n, const int64_t *ranks, int nt, int n_values, double *const *out,
+                  SelectScratch &s, int num_sms, cudaStream_t st)
 {
-    Sel sel{ylt, nullptr, s.hist, s.state, s.ctrl, s.acc, s.result, blocks_for(n, s.max_blocks)};
-    return enqueue(sel, 1, n, ranks, nt, st);
-}
-
-int launch_select(const double *ylt, int64_t n, const int64_t *ranks, int nt, SelectScratch &s,
-                  int num_sms, cudaStream_t st)
-{
-    const SelC sel{ylt, s.hist, s.acc, s.ctrl, s.app, s.cand, s.result};
-    ARE_CUDA_TRY(enqueue_coop(sel, n, ranks, nt, num_sms, st));
+    CoopArgs a = coop_args(n, ranks, nt, n_values);
+    a.single = ylt;
+    a.n_ylt = 1;
+    a.scratch = static_cast<CoopScratch *>(s.coop);
+    for (int t = 0; t < nt && out; ++t) a.out[t] = out[t];
+    ARE_CUDA_TRY(enqueue_coop(a, 1, num_sms, st));
     return 1;
 }
 
-namespace {
-int multi_blocks(int n_ylt, int64_t n, int num_sms)
+int launch_select_multi(const double *const *ylts, int n_ylt, int64_t n, const int64_t *ranks, int nt, int n_values,
+                        double *results, SelectScratch &s, int num_sms, cudaStream_t st)
 {
-    int cap = select_max_blocks(num_sms) / (n_ylt > 0 ? n_ylt : 1);
-    return blocks_for(n, cap < 1 ? 1 : cap);
-}
-size_t align256(size_t x) { return (x + 255) / 256 * 256; }
-}  // namespace
-
-size_t select_multi_bytes(int n_ylt, int64_t n, int num_sms)
-{
-    (void)n;
-    (void)num_sms;
-    return align256(sizeof(uint32_t) * kMaxTargets * kBins * n_ylt) +
-           align256(sizeof(unsigned long long) * 2 * kMaxTargets * n_ylt) +
-           align256(sizeof(unsigned int) * kCtrlWords * n_ylt) +
-           align256(sizeof(unsigned long long) * kMaxTargets * kAccWords * n_ylt) +
-           align256(sizeof(double) * 2 * kMaxTargets * n_ylt);
-}
-
-int launch_select_multi(const double *const *ylts, int n_ylt, int64_t n, const int64_t *ranks,
-                        int nt, void *scratch, int num_sms, cudaStream_t st, double **result)
-{
-    unsigned char *p = static_cast<unsigned char *>(scratch);
-    Sel sel;
-    sel.single = nullptr;
-    sel.many = ylts;
-    sel.blocks = multi_blocks(n_ylt, n, num_sms);
-    sel.hist = reinterpret_cast<uint32_t *>(p);
-    p += align256(sizeof(uint32_t) * kMaxTargets * kBins * n_ylt);
-    sel.state = reinterpret_cast<unsigned long long *>(p);
-    p += align256(sizeof(unsigned long long) * 2 * kMaxTargets * n_ylt);
-    sel.ctrl = reinterpret_cast<unsigned int *>(p);
-    p += align256(sizeof(unsigned int) * kCtrlWords * n_ylt);
-    sel.acc = reinterpret_cast<unsigned long long *>(p);
-    p += align256(sizeof(unsigned long long) * kMaxTargets * kAccWords * n_ylt);
-    sel.result = reinterpret_cast<double *>(p);
-    *result = sel.result;
-    ARE_CUDA_TRY(enqueue(sel, n_ylt, n, ranks, nt, st));
-    return kSelectLaunches;
+    CoopArgs a = coop_args(n, ranks, nt, n_values);
+    a.many = ylts;
+    a.n_ylt = n_ylt;
+    a.scratch = static_cast<CoopScratch *>(s.coop);
+    a.results = results;
+    ARE_CUDA_TRY(enqueue_coop(a, s.groups, num_sms, st));
+    return 1;
 }
 
 }  // namespace are
@@ -1015,18 +1090,24 @@ extern "C" are_status are_risk_measures_static(const double *ylt, int64_t n,
         }
     }
     unsigned char *base = static_cast<unsigned char *>(g_static_addr[dev]);
-    SelectScratch sc;
+    Sel sc;
+    sc.ylt = ylt;
     sc.hist = reinterpret_cast<uint32_t *>(base + kStaticHist);
     sc.state = reinterpret_cast<unsigned long long *>(base + kStaticState);
     sc.ctrl = reinterpret_cast<unsigned int *>(base + kStaticCtrl);
     sc.acc = reinterpret_cast<unsigned long long *>(base + kStaticAcc);
     sc.result = reinterpret_cast<double *>(base + kStaticResult);
-    sc.max_blocks = select_max_blocks(g_static_sms[dev]);
+    sc.blocks = blocks_for(n, g_static_sms[dev] * 4);
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nt = n_rp + n_tv;
     double res[2 * kMaxTargets];
-    cudaError_t e = select_enqueue(ylt, n, ranks, nt, sc, st);
+    Ranks r{};
+    for (int t = 0; t < nt; ++t) r.m[t] = ranks[t];
+    k_init<<<1, kThreads, 0, st>>>(sc, r, nt);
+    for (int pass = 0; pass < 8; ++pass) k_hist<<<sc.blocks, kThreads, 0, st>>>(sc, n, nt, pass);
+    k_tail<<<sc.blocks, kThreads, 0, st>>>(sc, n, nt, r);
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(res, sc.result, sizeof(double) * 2 * nt, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

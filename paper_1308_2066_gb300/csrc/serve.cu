@@ -517,8 +517,8 @@ void scheduler(Server *SP)
                 sl.launched += slice[i];
                 if (sl.launched < sl.req.n_trials) return;
                 launches += launch_select(reinterpret_cast<const double *>(S.d_arena + sl.ylt_off),
-                                          sl.req.n_trials, sl.req.ranks, sl.req.n_rp + sl.req.n_tv, sl.sel,
-                                          S.ctx->num_sms, S.stream);
+                                          sl.req.n_trials, sl.req.ranks, sl.req.n_rp + sl.req.n_tv, sl.req.n_rp,
+                                          nullptr, sl.sel, S.ctx->num_sms, S.stream);
                 ARE_CUDA_TRY(cudaMemcpyAsync(sl.h_res, sl.sel.result, sizeof(double) * 2 * kMaxTargets,
                                              cudaMemcpyDeviceToHost, S.stream));
                 ARE_CUDA_TRY(cudaEventRecord(sl.done_ev, S.stream));
@@ -739,7 +739,7 @@ are_status are_server_start(are_ctx *ctx, int32_t yet, const are_server_cfg *cfg
             S->arena.reset(S->d_arena, cfg->arena_bytes);
             S->slots.resize(cfg->max_inflight);
             for (Slot &sl : S->slots) {
-                select_alloc(sl.sel, ctx->num_sms);
+                select_alloc(sl.sel, 1);
                 ARE_CUDA_TRY(cudaMallocHost(&sl.h_res, sizeof(double) * 2 * kMaxTargets));
                 ARE_CUDA_TRY(cudaEventCreateWithFlags(&sl.done_ev, cudaEventDisableTiming));
             }
