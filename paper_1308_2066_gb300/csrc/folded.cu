@@ -33,7 +33,10 @@
 // and gathers their values, two per round.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "are_internal.cuh"
+#include "elt_tile.cuh"
 #include "fixed.cuh"
 
 namespace are {
@@ -100,6 +103,66 @@ __global__ void k_fold_finish(int32_t catalog, double occ_r, double occ_l, doubl
         best = o > best ? o : best;
     }
     if (lane == 0 && best) atomicMax(hmax, best);
+}
+
+// The same over ELTs in buckets, in one launch: a block per tile of 256 events
+// forms the tile's terms of all ELTs at once, adds them ELT by ELT in shared
+// memory and finishes its events.  (18 launches, each behind the one before,
+// and a 16 MB clear took 97 us at 1M events x 16 ELTs of 20,000 entries.)
+constexpr int kFoldStash = 2 * kEltTile;   // terms kept in shared memory; the rest are formed when added
+
+__global__ void __launch_bounds__(kEltTile)
+    k_fold_tiles(const __grid_constant__ ScatterArgs a, int32_t catalog, double occ_r, double occ_l,
+                 ulonglong2 *__restrict__ F, uint32_t *__restrict__ bits, int32_t words,
+                 unsigned long long *__restrict__ hmax)
+{
+    __shared__ EltTile t;
+    __shared__ double h[kEltTile], stash[kFoldStash];
+    __shared__ uint8_t stash_e[kFoldStash];
+    const int tid = threadIdx.x;
+    const uint32_t e0 = (uint32_t)blockIdx.x * kEltTile;
+    if (tid < 32) t.find(a, (int)blockIdx.x, tid);
+    h[tid] = 0.0;
+    __syncthreads();
+    const uint32_t n = t.start[kMaxElts];
+    for (uint32_t i = tid; i < n && i < kFoldStash; i += kEltTile) {
+        uint32_t e;
+        int j;
+        const int32_t at = t.entry(a, i, e0, e, j);
+        stash[i] = __dmul_rn(a.share[j], net(__dmul_rn(a.fx[j], a.loss[j][at]), a.ded[j], a.lim[j]));
+        stash_e[i] = (uint8_t)e;
+    }
+    for (int j = 0; j < a.n_elts; ++j) {
+        if (t.start[j] == t.start[j + 1]) continue;
+        __syncthreads();
+        for (uint32_t i = t.start[j] + tid; i < t.start[j + 1]; i += kEltTile) {
+            double x;
+            uint32_t e;
+            if (i < kFoldStash) {
+                x = stash[i];
+                e = stash_e[i];
+            } else {
+                int k;
+                const int32_t at = t.entry(a, i, e0, e, k);
+                x = __dmul_rn(a.share[j], net(__dmul_rn(a.fx[j], a.loss[j][at]), a.ded[j], a.lim[j]));
+            }
+            h[e] = __dadd_rn(h[e], x);
+        }
+    }
+    __syncthreads();
+    const bool in = e0 + tid < (uint32_t)catalog;
+    const double o = in ? net(h[tid], occ_r, occ_l) : 0.0;
+    if (in) F[e0 + tid].x = (unsigned long long)__double_as_longlong(o);
+    const uint32_t m = __ballot_sync(kFull, o > 0.0);
+    const uint32_t w = (e0 + tid) >> 5;
+    if ((tid & 31) == 0 && w < (uint32_t)words) bits[w] = m;
+    unsigned long long best = (unsigned long long)__double_as_longlong(o);
+#pragma unroll
+    for (int off = 16; off; off >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(kFull, best, off);
+        best = x > best ? x : best;
+    }
+    if ((tid & 31) == 0 && best > __ldcg(hmax)) atomicMax(hmax, best);
 }
 
 // ---------------------------------------------------------------------------
@@ -277,6 +340,14 @@ int launch_fold(const ScatterArgs &elts, double occ_r, double occ_l, int32_t cat
     const int32_t words = folded_words(catalog);
     double *h = reinterpret_cast<double *>(F);   // h[e] accumulates in the low word of F[e]
     ARE_CUDA_TRY(cudaMemsetAsync(hmax, 0, sizeof *hmax, s));
+    const unsigned fixed_blocks = (unsigned)std::min<int64_t>(((int64_t)catalog + 255) / 256, (int64_t)num_sms * 16);
+    if (elts_bucketed(elts)) {
+        k_fold_tiles<<<(unsigned)(((int64_t)catalog + kEltTile - 1) / kEltTile), kEltTile, 0, s>>>(
+            elts, catalog, occ_r, occ_l, F, bits, words, hmax);
+        k_fold_fixed<<<fixed_blocks, 256, 0, s>>>(catalog, F, hmax);
+        ARE_CUDA_TRY(cudaGetLastError());
+        return 2;
+    }
     ARE_CUDA_TRY(cudaMemsetAsync(F, 0, sizeof(ulonglong2) * (size_t)catalog, s));
     int launches = 0;
     for (int j = 0; j < elts.n_elts; ++j) {

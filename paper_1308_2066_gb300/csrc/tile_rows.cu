@@ -19,7 +19,7 @@
 #include <string>
 
 #include "are_internal.cuh"
-#include "fixed.cuh"
+#include "elt_tile.cuh"
 #include "rows.cuh"
 
 namespace are {
@@ -30,10 +30,7 @@ constexpr int kStash = 2 * kTile;          // entries whose terms are kept betwe
 constexpr unsigned kFull = 0xffffffffu;
 
 // What a block knows of its tile.
-struct Tile {
-    uint32_t start[kMaxElts + 1];          // entries before ELT j's, and all
-    int32_t from[kMaxElts];                // ELT j's first entry of the tile
-    uint32_t base;                         // entries of all ELTs in the tiles before this
+struct Tile : EltTile {
     uint32_t ovf;                          // overflow terms handed out
     uint32_t mask[kTile];                  // per event: the ELTs whose term is not 0
 };
@@ -162,29 +159,8 @@ __global__ void __launch_bounds__(kTile) k_tile_rows(const __grid_constant__ Bui
     const int tid = threadIdx.x, tile = blockIdx.x;
     const uint32_t e0 = (uint32_t)tile * kTile;
     V *const ovf = static_cast<V *>(a.ovf);
-    if (tid < 32) {
-        int32_t from = 0, cnt = 0;
-        if (tid < a.elts.n_elts) {
-            const int32_t tiles = a.elts.tiles[tid];
-            const int32_t *off = a.elts.off[tid];
-            from = tile < tiles ? __ldg(off + tile) : a.elts.n[tid];
-            cnt = tile < tiles ? __ldg(off + tile + 1) - from : 0;
-        }
-        uint32_t incl = (uint32_t)cnt, before = (uint32_t)from;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t o = __shfl_up_sync(kFull, incl, d);
-            if (tid >= d) incl += o;
-            before += __shfl_xor_sync(kFull, before, d);
-        }
-        t.from[tid] = from;
-        t.start[tid] = incl - (uint32_t)cnt;
-        if (tid == 31) {
-            t.start[32] = incl;
-            t.base = before;
-            t.ovf = 0;
-        }
-    }
+    if (tid < 32) t.find(a.elts, tile, tid);
+    if (tid == 0) t.ovf = 0;
     t.mask[tid] = 0;
     {
         uint4 *z = reinterpret_cast<uint4 *>(row);
@@ -195,12 +171,7 @@ __global__ void __launch_bounds__(kTile) k_tile_rows(const __grid_constant__ Bui
     const uint32_t n = t.start[32];
     // entry i of the tile: its event, ELT and term
     auto entry = [&](uint32_t i, uint32_t &e, int &j) -> V {
-        j = 0;
-#pragma unroll
-        for (int s = 16; s; s >>= 1)
-            if (t.start[j + s] <= i) j += s;
-        const int32_t at = t.from[j] + (int32_t)(i - t.start[j]);
-        e = (uint32_t)a.elts.ids[j][at] - e0;
+        const int32_t at = t.entry(a.elts, i, e0, e, j);
         return F::value(fin_term(a.elts.loss[j][at], a.elts.fx[j], a.elts.ded[j], a.elts.lim[j], a.elts.share[j]));
     };
     auto again = [&](uint32_t i, uint32_t &e, int &j) -> V {

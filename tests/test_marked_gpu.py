@@ -132,8 +132,8 @@ def test_rows_built_tile_by_tile(are, orc, J, C, nnz):
     of 256 events around their edges, more entries in a tile than it keeps
     between its passes, every ELT holding an event (overflows), ELTs whose
     last tile comes before the catalog's, an ELT without entries, and ids past
-    the buckets.  FP64 equals the oracle's bit for bit; FP32 terms are rounded
-    once and up to 32 of them added."""
+    the buckets.  FP64 and the folded table equal the oracle's bit for bit; FP32
+    terms are rounded once and up to 32 of them added."""
     import torch
     g = np.random.Generator(np.random.PCG64(J + C))
     top = C if C < 1 << 20 else C - 1
@@ -161,5 +161,7 @@ def test_rows_built_tile_by_tile(are, orc, J, C, nnz):
             else:    # 34 roundings at the scale of the event loss, at most 32 limits
                 bound = 34 * 2.0 ** -24 * sum(e.lim for e in elts if np.isfinite(e.lim))
                 np.testing.assert_allclose(out.cpu().numpy(), ref, rtol=1e-5, atol=bound)
+        are.are_simulate_folded(ctx, layer, y, 0, events.size, out)      # the folded table's tiles
+        np.testing.assert_array_equal(out.cpu().numpy(), ref)
     finally:
         are.are_destroy(ctx)
