@@ -545,13 +545,22 @@ bool uses_marks(are_ctx *ctx, const Layer &L, const Yet &y, are_precision p)
     }
 }
 
-// The rows of a register-rows analysis -- packed, or the dense FP32 table --
-// and, with `marked`, their marks where the layer's analysis uses them.
-void ensure_rows(are_ctx *ctx, Layer &L, const Yet &y, are_precision p, bool marked, cudaStream_t s, bool rebuild)
+// The same for the per-occurrence outputs.  Trials of 20 events take 0.68 of
+// the every-row rate, 60 events 0.97, 200 events 2.2; without terms, at 1000
+// events a trial, the marked form gains 2.7 where 0.27 of the events are
+// marked, 1.4 (FP64 1.5) at 0.55, 1.02 (1.04) at 0.8 and loses (0.77) at 0.96.
+bool occ_uses_marks(are_ctx *ctx, const Layer &L, const Yet &y, bool fp32)
 {
-    const bool fp32 = p != ARE_FP64;
+    if (y.catalog <= 0 || mark_shape(y.catalog).words == 0) return false;
+    if (fp32 && !(L.bound < 1e37)) return false;
+    return (double)y.n_events >= 60.0 * (double)y.n_trials && marked_share(ctx, L, y.catalog) <= 0.8;
+}
+
+// The rows of a register-rows analysis -- packed, or the dense FP32 table --
+// and, with `marked`, their marks.
+void ensure_rows(are_ctx *ctx, Layer &L, const Yet &y, bool fp32, bool marked, cudaStream_t s, bool rebuild)
+{
     const int32_t catalog = y.catalog;
-    marked = marked && uses_marks(ctx, L, y, p);
     if (ensure_packed(ctx, L, catalog, fp32, marked, s, rebuild)) return;
     if (rebuild || !L.t32.d || L.t32.catalog != catalog ||
         (marked && (!L.m32.map.d || L.m32.catalog != catalog)))
@@ -566,7 +575,7 @@ void ensure_direct(are_ctx *ctx, Layer &L, const Yet &y, are_precision p, const 
     const bool fp32 = p != ARE_FP64;
     const int32_t catalog = y.catalog;
     if (te.kernel == 2) {   // a dense table only where the rows are dense
-        ensure_rows(ctx, L, y, p, te.cfg.rows_in_flight == 0, s, rebuild);
+        ensure_rows(ctx, L, y, fp32, te.cfg.rows_in_flight == 0 && uses_marks(ctx, L, y, p), s, rebuild);
         return;
     }
     const Table &t = fp32 ? L.t32 : L.t64;
@@ -1714,8 +1723,10 @@ are_status are_simulate_occurrences(are_ctx *ctx, int32_t layer, int32_t yet, in
         Table &t = fp32 ? L.t32 : L.t64;
         // the rows of the register-rows form (the direct layout, whatever the
         // layer's analysis layout): packed where the layer's row size calls for them
-        const bool packed = ensure_packed(ctx, L, y.catalog, fp32, false, cs.s, false);
-        if (!packed && (!t.d || t.catalog != y.catalog)) build_table(ctx, L, y.catalog, fp32, cs.s);
+        const bool marked = occ_uses_marks(ctx, L, y, fp32);
+        ensure_rows(ctx, L, y, fp32, marked, cs.s, false);
+        const bool packed = row_words(L, y.catalog, fp32) != 0;
+        const MarkMap marks = marked ? (fp32 ? L.m32 : L.m64).map : MarkMap{};
         SimArgs a{};
         a.ids = y.d_ids;
         a.off = y.d_off;
@@ -1742,10 +1753,10 @@ are_status are_simulate_occurrences(are_ctx *ctx, int32_t layer, int32_t yet, in
             const Packed &p = fp32 ? L.p32 : L.p64;
             a.table = p.rows();
             a.table2 = p.ovf();
-            ctx->launches += launch_rows_occ(a, fp32 ? 1 : 0, p.rw, t32, t64, fixed_scale(L), ctx->num_sms,
+            ctx->launches += launch_rows_occ(a, fp32 ? 1 : 0, p.rw, marks, t32, t64, fixed_scale(L), ctx->num_sms,
                                              cs.s);
         } else {         // dense FP32 rows
-            ctx->launches += launch_rows_occ(a, 2, t.jp, t32, t64, fixed_scale(L), ctx->num_sms, cs.s);
+            ctx->launches += launch_rows_occ(a, 2, t.jp, marks, t32, t64, fixed_scale(L), ctx->num_sms, cs.s);
         }
         cs.finish();
     });

@@ -427,9 +427,9 @@ int launch_staged64(const SimArgs &a, int jp, const TermsF64 &t, int num_sms, cu
 // times 2^scale below 2^126).
 // rows_occ.cu: the per-occurrence outputs over the register-rows kernels'
 // rows (form 0 packed FP64, 1 packed FP32, 2 dense FP32; a.table and
-// a.table2 the rows and their overflow).
-int launch_rows_occ(const SimArgs &a, int form, int row_words, const TermsF32 &t32, const TermsF64 &t64, int scale,
-                    int num_sms, cudaStream_t s);
+// a.table2 the rows and their overflow; marks: those of the rows, or d null).
+int launch_rows_occ(const SimArgs &a, int form, int row_words, const MarkMap &marks, const TermsF32 &t32,
+                    const TermsF64 &t64, int scale, int num_sms, cudaStream_t s);
 int launch_rows64(const SimArgs &a, int row_words, const TermsF64 &t, int scale, int num_sms,
                   cudaStream_t s);
 

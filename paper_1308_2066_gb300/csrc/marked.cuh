@@ -45,6 +45,7 @@
 
 #include <cuda_runtime.h>
 
+#include <string>
 #include <type_traits>
 
 #include "are_internal.cuh"
@@ -268,6 +269,37 @@ __device__ __forceinline__ void load_ids(uint32_t (&id)[kSlots], const int32_t *
     }
 }
 
+// Whether quarters of a pass may be read past the last event of the warp's
+// trials (up to t1): where the ids reach that far (to the end of the launch's
+// range, and kIdPad further).
+template <bool FIXED>
+__device__ __forceinline__ bool whole_quarters(const PassArgs &a, int64_t t1)
+{
+    const int64_t end = a.t.trial_begin + a.n_trials, own = a.t.trial_begin + t1;
+    return (FIXED ? (end - own) * (int64_t)a.t.k : __ldg(a.t.off + end) - __ldg(a.t.off + own)) + kIdPad >= 128;
+}
+
+// The marks of the lane's ids in a pass of cnt events, bit u for slot u (the
+// event 32 u + at).
+template <bool FOLD>
+__device__ __forceinline__ uint32_t marks_of(const uint32_t (&id)[kSlots], const uint32_t *marks, uint32_t bits, int cnt,
+                                             int at)
+{
+    uint32_t mask = 0;
+#pragma unroll
+    for (int q = kSlots / 4 - 1; q >= 0; --q)
+        if (q * 128 < cnt) {
+#pragma unroll
+            for (int u = 4 * q + 3; u >= 4 * q; --u) {
+                const uint32_t e = FOLD ? min(id[u], id[u] - bits) : id[u];
+                const uint32_t word = marks[e >> 5];
+                mask = __funnelshift_l(__funnelshift_l(word, word, e), mask, 1);
+            }
+        }
+    const int mine = cnt > at ? (cnt - at + 31) >> 5 : 0;   // the lane's events in the pass
+    return mask & ((1u << mine) - 1u);
+}
+
 // Where a lane's n <= 16 entries start in the warp's list of them all, lane
 // by lane, and their total: from the bits of the counts by ballots (shuffles
 // would take turns with the shared-memory reads).
@@ -400,10 +432,7 @@ __global__ void __launch_bounds__(32 * pass_warps(ACC == ARE_FP32_KAHAN, FIXED),
     const int64_t nw = (int64_t)gridDim.x * kWarps, w = (int64_t)blockIdx.x * kWarps + wib;
     const int64_t t0 = w * a.n_trials / nw, t1 = (w + 1) * a.n_trials / nw;
     if (t0 >= t1) return;
-    // quarters of a pass may be read past the warp's last event where the ids
-    // reach that far (to the end of the range, and kIdPad further)
-    const int64_t r1 = a.t.trial_begin + a.n_trials, w1 = a.t.trial_begin + t1;
-    const bool whole = (FIXED ? (r1 - w1) * (int64_t)a.t.k : __ldg(a.t.off + r1) - __ldg(a.t.off + w1)) + kIdPad >= 128;
+    const bool whole = whole_quarters<FIXED>(a, t1);
     const int at = (lane % R) * RPW + lane / R;   // the lane's event of each group of 32
     double *const ylt = a.t.ylt + t0;
 
@@ -428,21 +457,7 @@ __global__ void __launch_bounds__(32 * pass_warps(ACC == ARE_FP32_KAHAN, FIXED),
         const int cnt = walk.count();
         const int32_t tc = walk.t;
         const bool last = walk.last();
-        // 1. the marks of the lane's ids
-        uint32_t mask = 0;
-#pragma unroll
-        for (int q = kSlots / 4 - 1; q >= 0; --q)
-            if (q * 128 < cnt) {
-#pragma unroll
-                for (int u = 4 * q + 3; u >= 4 * q; --u) {
-                    const uint32_t e = FOLD ? min(id[u], id[u] - a.bits) : id[u];
-                    const uint32_t word = bm[e >> 5];
-                    mask = __funnelshift_l(__funnelshift_l(word, word, e), mask, 1);
-                }
-            }
-        const int mine = cnt > at ? (cnt - at + 31) >> 5 : 0;   // the lane's events in the pass
-        mask &= (1u << mine) - 1u;
-
+        const uint32_t mask = marks_of<FOLD>(id, bm, a.bits, cnt, at);   // 1. the marks of the lane's ids
         if constexpr (KAHAN)
             if (have == 0 && cnt > 0 && !(mask & 1u) && acc.c != 0.f) acc.add(0.f);   // (a later pass's slot 0)
         uint32_t m = mask, before, total;
@@ -544,8 +559,7 @@ void launch_pass_t(const PassArgs &a, const Rows &rows_, int num_sms, cudaStream
     ARE_CUDA_TRY(cudaGetLastError());
 }
 
-template <typename Rows, int ACC>
-void launch_pass(const SimArgs &a, const MarkMap &m, const Rows &rows_, int scale, int num_sms, cudaStream_t s)
+inline PassArgs pass_args(const SimArgs &a, const MarkMap &m, int scale)
 {
     PassArgs p;
     p.t.ids = a.ids;
@@ -560,6 +574,48 @@ void launch_pass(const SimArgs &a, const MarkMap &m, const Rows &rows_, int scal
     p.bits = m.bits;
     p.scale = scale;
     p.n_trials = a.n_trials;
+    return p;
+}
+
+// fn(rows) for the layer's FP32 rows: packed rows of 8 or 16 words with their
+// overflow terms, or dense rows of 8 or 16 terms.
+template <typename F>
+auto with_rows32(const void *table, const void *ovf, bool packed, int row_words, const TermsF32 &tm, F &&fn)
+{
+    auto go = [&](auto r) {
+        r.table = static_cast<const float *>(table);
+        if constexpr (decltype(r)::PACKED) r.ovf = static_cast<const float *>(ovf);
+        r.occ_r = tm.occ_r;
+        r.occ_l = tm.occ_l;
+        return fn(r);
+    };
+    if (packed && row_words == 8) return go(PackedF32<8>{});
+    if (packed && row_words == 16) return go(PackedF32<16>{});
+    if (!packed && row_words == 8) return go(DenseF32<8>{});
+    if (!packed && row_words == 16) return go(DenseF32<16>{});
+    throw Error{ARE_EINVAL, "no marked FP32 rows of " + std::to_string(row_words) + " words"};
+}
+
+// fn(rows) for the layer's packed FP64 rows of 4 or 8 words.
+template <typename F>
+auto with_rows64(const void *table, const void *ovf, int row_words, const TermsF64 &tm, F &&fn)
+{
+    auto go = [&](auto r) {
+        r.table = static_cast<const unsigned long long *>(table);
+        r.ovf = static_cast<const double *>(ovf);
+        r.occ_r = tm.occ_r;
+        r.occ_l = tm.occ_l;
+        return fn(r);
+    };
+    if (row_words == 4) return go(PackedF64<4>{});
+    if (row_words == 8) return go(PackedF64<8>{});
+    throw Error{ARE_EINVAL, "no marked FP64 rows of " + std::to_string(row_words) + " words"};
+}
+
+template <typename Rows, int ACC>
+void launch_pass(const SimArgs &a, const MarkMap &m, const Rows &rows_, int scale, int num_sms, cudaStream_t s)
+{
+    const PassArgs p = pass_args(a, m, scale);
     if (a.off)
         m.fold ? launch_pass_t<Rows, ACC, false, true>(p, rows_, num_sms, s)
                : launch_pass_t<Rows, ACC, false, false>(p, rows_, num_sms, s);
