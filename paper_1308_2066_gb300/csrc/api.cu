@@ -472,14 +472,16 @@ bool ensure_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, bool mark
     return true;
 }
 
-// An upper bound of the layer's occurrence losses: min(OccL, the sum over
-// its ELTs of the largest term), the largest term being the term of the
-// ELT's largest loss (a term is non-decreasing in the loss), with a margin
-// for the rounding of that sum.
-double loss_bound(are_ctx *ctx, const Layer &L)
+}  // namespace
+
+// An upper bound of a layer's occurrence losses: min(OccL, the sum over its
+// ELTs of the largest term), the largest term being the term of the ELT's
+// largest loss (a term is non-decreasing in the loss), with a margin for the
+// rounding of that sum.
+double loss_bound(const are_ctx *ctx, const std::vector<int32_t> &elts, const are_layer_terms &terms)
 {
     double g = 0.0;
-    for (int32_t h : L.elts) {
+    for (int32_t h : elts) {
         const Elt &e = ctx->elts.at(h);
         if (e.n == 0) continue;
         double x = e.terms.fx * e.max_loss - e.terms.deductible;
@@ -487,23 +489,34 @@ double loss_bound(are_ctx *ctx, const Layer &L)
         x = x > e.terms.limit ? e.terms.limit : x;
         g += e.terms.share * x;
     }
-    return std::min(g, L.terms.occ_lim) * (1.0 + 1e-9);
+    return std::min(g, terms.occ_lim) * (1.0 + 1e-9);
+}
+
+// The fixed-point scale of the exact running sums: s = 125 - floor(log2(B))
+// for the upper bound B of the layer's occurrence losses.
+int fixed_scale(double bound)
+{
+    if (!(bound > 0.0)) return 0;
+    int ex = 0;
+    std::frexp(bound, &ex);      // B = f * 2^ex, 0.5 <= f < 1: floor(log2 B) = ex - 1
+    return 125 - (ex - 1);
 }
 
 // An estimate of the share of the catalog's events that have an occurrence
-// loss in the layer: an event with m terms is taken to need one above OccR /
-// m, m the mean number of terms of the events that have any (entries fall on
+// loss in a layer: an event with m terms is taken to need one above OccR / m,
+// m the mean number of terms of the events that have any (entries fall on
 // events independently).  From the ELTs' counts of losses by quarter octave.
-double marked_share(are_ctx *ctx, const Layer &L, int32_t catalog)
+double marked_share(const are_ctx *ctx, const std::vector<int32_t> &elts, const are_layer_terms &terms, int64_t entries,
+                    int32_t catalog)
 {
-    if (L.marked_catalog == catalog) return L.marked;
-    const double per_event = (double)layer_entries(L) / (double)catalog;
+    const double per_event = (double)entries / (double)catalog;
     const double m = per_event > 0.0 ? per_event / -std::expm1(-per_event) : 1.0;
+    const double need = terms.occ_ret / m;         // of a term: share * (fx * x - D), at most share * Lim
     double above = 0.0;
-    for (int32_t h : L.elts) {
+    for (int32_t h : elts) {
         const Elt &e = ctx->elts.at(h);
-        const double need = L.terms.occ_ret / m;   // of a term: share * (fx * x - D), at most share * Lim
-        if (!(e.terms.share * e.terms.limit > 0.0) || e.terms.share * e.terms.limit < need) continue;
+        const double top = e.terms.share * e.terms.limit;
+        if (!(top > 0.0) || top < need) continue;
         const double x = (need / e.terms.share + e.terms.deductible) / e.terms.fx;   // the loss that gives it
         uint64_t bits;
         std::memcpy(&bits, &x, sizeof bits);
@@ -511,13 +524,12 @@ double marked_share(are_ctx *ctx, const Layer &L, int32_t catalog)
         for (size_t i = 0; i < e.bins.size(); ++i)
             above += e.bin_weight * e.bins[i] * std::min(1.0, std::max(0.0, (double)(i + 1) - at));
     }
-    L.marked = -std::expm1(-above / (double)catalog);
-    L.marked_catalog = catalog;
-    return L.marked;
+    return -std::expm1(-above / (double)catalog);
 }
 
-// Whether the register-rows analysis of the layer over a YET looks its
-// occurrences up in marks first (marked.cuh).  It depends on the layer, the
+// Whether a register-rows analysis over a YET looks its occurrences up in
+// marks first (marked.cuh), the layer's losses at most `bound` and `share` of
+// the events marked.  It depends on the layer, the
 // YET and the precision alone, so that every split of the trials, the
 // streamed analysis and the server form a trial's sum alike.
 //  * The marks of the catalog fit a block's shared memory.
@@ -532,17 +544,32 @@ double marked_share(are_ctx *ctx, const Layer &L, int32_t catalog)
 //    at 0.7; the FP32 kernel with FP64 sums gains 2.5, 1.4 and 1.2 there,
 //    1.08 at 0.8 and loses (0.52) at 0.96; FP64 2.3, 1.8, 1.5 and 1.3, and
 //    0.87 at 0.96.
-bool uses_marks(are_ctx *ctx, const Layer &L, const Yet &y, are_precision p)
+bool use_marks(are_precision p, const Yet &y, double bound, double share)
 {
     if (y.catalog <= 0 || mark_shape(y.catalog).words == 0) return false;
-    if (p != ARE_FP64 && !(L.bound < 1e37)) return false;
+    if (p != ARE_FP64 && !(bound < 1e37)) return false;
     const double mean = y.n_trials ? (double)y.n_events / (double)y.n_trials : 0.0;
-    const double share = marked_share(ctx, L, y.catalog);
     switch (p) {
     case ARE_FP32_KAHAN: return mean >= 80.0 && share <= 0.5;
     case ARE_FP32_FP64AGG: return share <= 0.75;
     default: return mean >= 50.0 && share <= 0.85;
     }
+}
+
+namespace {
+
+double layer_share(const are_ctx *ctx, const Layer &L, int32_t catalog)
+{
+    if (L.marked_catalog != catalog) {
+        L.marked = marked_share(ctx, L.elts, L.terms, layer_entries(L), catalog);
+        L.marked_catalog = catalog;
+    }
+    return L.marked;
+}
+
+bool uses_marks(const are_ctx *ctx, const Layer &L, const Yet &y, are_precision p)
+{
+    return y.catalog > 0 && use_marks(p, y, L.bound, layer_share(ctx, L, y.catalog));
 }
 
 // The same for the per-occurrence outputs.  Trials of 20 events take 0.68 of
@@ -553,7 +580,7 @@ bool occ_uses_marks(are_ctx *ctx, const Layer &L, const Yet &y, bool fp32)
 {
     if (y.catalog <= 0 || mark_shape(y.catalog).words == 0) return false;
     if (fp32 && !(L.bound < 1e37)) return false;
-    return (double)y.n_events >= 60.0 * (double)y.n_trials && marked_share(ctx, L, y.catalog) <= 0.8;
+    return (double)y.n_events >= 60.0 * (double)y.n_trials && layer_share(ctx, L, y.catalog) <= 0.8;
 }
 
 // The rows of a register-rows analysis -- packed, or the dense FP32 table --
@@ -670,17 +697,6 @@ ItemWork item_work(const Yet &y, int64_t trial_begin, int64_t n_trials, const It
     return w;
 }
 
-// The fixed-point scale of the exact running sums: s = 125 - floor(log2(B))
-// for the upper bound B of the layer's occurrence losses.
-int fixed_scale(const Layer &L)
-{
-    const double b = L.bound;
-    if (!(b > 0.0)) return 0;
-    int ex = 0;
-    std::frexp(b, &ex);          // b = f * 2^ex, 0.5 <= f < 1: floor(log2 b) = ex - 1
-    return 125 - (ex - 1);
-}
-
 // One layer's analysis stage with a given kernel choice.
 int run_single(are_ctx *ctx, const Layer &L, const Yet &y, int64_t trial_begin, int64_t n_trials,
                are_precision precision, double *d_out, const TuneEntry &te, cudaStream_t s)
@@ -723,7 +739,7 @@ int run_single(are_ctx *ctx, const Layer &L, const Yet &y, int64_t trial_begin, 
         a.table2 = L.p32.ovf();
         a.kernel = 5;
         if (marked)
-            return launch_marked32(a, m.map, precision, true, L.p32.rw, t32, fixed_scale(L), ctx->num_sms, s);
+            return launch_marked32(a, m.map, precision, true, L.p32.rw, t32, fixed_scale(L.bound), ctx->num_sms, s);
         return launch_simulate(a, precision, L.p32.rw, &t32, &t64, ctx->num_sms, s);
     }
     if (compact) {   // the staged kernel, through the row index
@@ -736,8 +752,8 @@ int run_single(are_ctx *ctx, const Layer &L, const Yet &y, int64_t trial_begin, 
         if (te.kernel == 2 && L.p64.d && L.p64.catalog == y.catalog) {   // packed FP64 rows
             a.table = L.p64.rows();
             a.table2 = L.p64.ovf();
-            if (marked) return launch_marked64(a, m.map, L.p64.rw, t64, fixed_scale(L), ctx->num_sms, s);
-            return launch_rows64(a, L.p64.rw, t64, fixed_scale(L), ctx->num_sms, s);
+            if (marked) return launch_marked64(a, m.map, L.p64.rw, t64, fixed_scale(L.bound), ctx->num_sms, s);
+            return launch_rows64(a, L.p64.rw, t64, fixed_scale(L.bound), ctx->num_sms, s);
         }
         if (te.kernel == 3 && L.t32u.d && L.t32u.catalog == y.catalog) {   // the FP32 screen
             a.table2 = L.t32u.d;
@@ -746,7 +762,7 @@ int run_single(are_ctx *ctx, const Layer &L, const Yet &y, int64_t trial_begin, 
         }
         return launch_staged64(a, t.jp, t64, ctx->num_sms, s);   // (or an aux table not built)
     }
-    if (marked) return launch_marked32(a, m.map, precision, false, t.jp, t32, fixed_scale(L), ctx->num_sms, s);
+    if (marked) return launch_marked32(a, m.map, precision, false, t.jp, t32, fixed_scale(L.bound), ctx->num_sms, s);
     return launch_simulate(a, precision, t.jp, &t32, &t64, ctx->num_sms, s);
 }
 
@@ -1246,7 +1262,7 @@ are_status are_define_layer(are_ctx *ctx, const int32_t *elt_handles, int32_t n_
         }
         L.terms = positive_zeros(t);
         for (int32_t h : L.elts) L.entries += ctx->elts[h].n;
-        L.bound = loss_bound(ctx, L);
+        L.bound = loss_bound(ctx, L.elts, L.terms);
         for (int32_t h : L.elts) ctx->elts[h].users++;
         const int32_t h = ctx->next_handle++;
         ctx->layers[h] = L;
@@ -1753,10 +1769,10 @@ are_status are_simulate_occurrences(are_ctx *ctx, int32_t layer, int32_t yet, in
             const Packed &p = fp32 ? L.p32 : L.p64;
             a.table = p.rows();
             a.table2 = p.ovf();
-            ctx->launches += launch_rows_occ(a, fp32 ? 1 : 0, p.rw, marks, t32, t64, fixed_scale(L), ctx->num_sms,
+            ctx->launches += launch_rows_occ(a, fp32 ? 1 : 0, p.rw, marks, t32, t64, fixed_scale(L.bound), ctx->num_sms,
                                              cs.s);
         } else {         // dense FP32 rows
-            ctx->launches += launch_rows_occ(a, 2, t.jp, marks, t32, t64, fixed_scale(L), ctx->num_sms, cs.s);
+            ctx->launches += launch_rows_occ(a, 2, t.jp, marks, t32, t64, fixed_scale(L.bound), ctx->num_sms, cs.s);
         }
         cs.finish();
     });

@@ -393,6 +393,14 @@ int launch_pack64_direct(const ScatterArgs &a, int32_t catalog, int rw, unsigned
 int launch_pack32_direct(const ScatterArgs &a, int32_t catalog, int pw, uint32_t *rows, float *ovf,
                          unsigned long long *ovf_used, cudaStream_t s);
 
+// api.cu: what decides whether an analysis looks occurrences up in marks first
+// (the ELTs by handle, under the context's lock), and the scale of exact sums.
+double loss_bound(const are_ctx *ctx, const std::vector<int32_t> &elts, const are_layer_terms &terms);
+double marked_share(const are_ctx *ctx, const std::vector<int32_t> &elts, const are_layer_terms &terms, int64_t entries,
+                    int32_t catalog);
+bool use_marks(are_precision p, const Yet &y, double bound, double share);
+int fixed_scale(double bound);
+
 // api.cu: how many blocks of `kern` (threads per block, bytes of dynamic
 // shared memory) fit on one SM of the current device.  On the first call for
 // a device it also raises the kernel's dynamic shared-memory limit to `smem`

@@ -11,12 +11,14 @@
 //      (least_work_first) in order of least remaining work less the time
 //      each has already waited (so a long request is not overtaken for
 //      ever by short ones that keep arriving); each takes what it needs,
-//      the last one a partial slice.  The slices of small
-//      requests run in one persistent launch of the multi-layer kernel (one
-//      launch per table width); a request of at least kLargeSlice events
-//      runs its slices on the single-layer register-rows kernel, which is
-//      faster per event.  The kernel is chosen per request, so a request's
-//      result does not depend on the requests around it;
+//      the last one a partial slice.  A request few of whose events have a
+//      loss runs its slices over the marked events (marked.cuh), a launch
+//      each; the slices of the other small requests run in one persistent
+//      launch of the multi-layer kernel (one launch per table width), and a
+//      request of at least kLargeSlice events on the single-layer
+//      register-rows kernel, which is faster per event.  The kernel is chosen
+//      per request, so a request's result does not depend on the requests
+//      around it;
 //   3. selects PML/TVaR for the requests whose last slice was in the launch;
 //   4. waits (bounded) for the previous iteration and posts its results.
 // One iteration is always queued ahead of the one being waited for, so the
@@ -108,6 +110,8 @@ struct Request {
     are_layer_terms terms{};
     int64_t n_trials = 0;
     int64_t entries = 0;            // ELT entries of the request's layer
+    double bound = 0.0;             // upper bound of its occurrence losses
+    bool marked = false;            // its trial passes look occurrences up in marks first
     int n_rp = 0, n_tv = 0;
     int64_t ranks[kMaxTargets] = {};
     Clock::time_point t_submit;
@@ -120,9 +124,11 @@ struct Slot {
     size_t tab_off = 0, tab_bytes = 0, ylt_off = 0, ylt_bytes = 0;
     LayerF32 rec{};
     int64_t launched = 0;           // trials handed to launches so far
-    bool large = false;             // its slices run on the single-layer register-rows kernel
+    bool large = false;             // a request of at least kLargeSlice events
+    bool own = false;               // its slices run on a single-layer kernel, a launch each
     int pw = 0;                     // large: words per packed row (0: the dense rows)
     size_t dense_bytes = 0;         // the dense table (0 for packed rows, which fill the block)
+    MarkMap marks;                  // in the block's end; d null: every row is read
     uint64_t finish_iter = 0;       // iteration whose completion posts the result
     cudaEvent_t done_ev = nullptr;  // recorded after the result's copy: posts it as soon as it fires
     SelectScratch sel;
@@ -221,6 +227,13 @@ float *packed_ovf(Server &S, const Slot &sl)
     return reinterpret_cast<float *>(reinterpret_cast<char *>(packed_used(S, sl)) + 256);
 }
 
+// The rows of a request's table: bytes of its arena block before the marks.
+size_t table_bytes(const Slot &sl, int32_t catalog, int64_t entries)
+{
+    return sl.pw ? up((size_t)catalog * sl.pw * sizeof(float)) + 256 + up(sizeof(float) * (size_t)entries + 8)
+                 : up(sl.dense_bytes);
+}
+
 // Table of an admitted request, built on the server stream in its arena block.
 void build_request_table(Server &S, Slot &sl)
 {
@@ -242,10 +255,12 @@ void build_request_table(Server &S, Slot &sl)
     }
     if (elts_bucketed(a)) {
         const bool packed = sl.pw != 0;
+        TermsF32 t32;
+        t32.occ_r = (float)sl.req.terms.occ_ret;
+        t32.occ_l = (float)sl.req.terms.occ_lim;
         add_launches(S, launch_tile_rows(a, S.y->catalog, true, packed, packed ? sl.pw : sl.jp,
                                          packed ? (void *)packed_rows(S, sl) : (void *)(S.d_arena + sl.tab_off),
-                                         packed ? packed_ovf(S, sl) : nullptr, MarkMap{}, TermsF32{}, TermsF64{},
-                                         S.stream));
+                                         packed ? packed_ovf(S, sl) : nullptr, sl.marks, t32, TermsF64{}, S.stream));
         return;
     }
     if (sl.pw) {   // packed rows straight from the ELT entries
@@ -402,9 +417,18 @@ void scheduler(Server *SP)
                                 : 0;
                     sl.dense_bytes = sl.pw ? 0 : (size_t)S.y->catalog * sl.jp * sizeof(float);
                     sl.tab_bytes = S.cfg.folded ? folded_block_bytes(S.y->catalog)
-                                   : sl.pw ? up((size_t)S.y->catalog * sl.pw * sizeof(float)) + 256 +
-                                                 up(sizeof(float) * (size_t)r.entries + 8)
-                                           : sl.dense_bytes;
+                                                : table_bytes(sl, S.y->catalog, r.entries);
+                    sl.marks = MarkMap{};
+                    // marks for the kernels that take them (rows of up to 16
+                    // words), unless the arena could never hold them too
+                    const MarkMap shape = mark_shape(S.y->catalog);
+                    const size_t mark_bytes = sizeof(uint32_t) * (size_t)shape.words;
+                    const bool marked = r.marked && (sl.pw || sl.jp <= 16) &&
+                                        sl.tab_bytes + mark_bytes + up(sizeof(double) * (size_t)r.n_trials) <=
+                                            S.cfg.arena_bytes;
+                    const size_t marks_at = sl.tab_bytes;
+                    if (marked) sl.tab_bytes += mark_bytes;
+                    sl.own = (sl.large || marked) && !S.cfg.folded;
                     sl.ylt_bytes = sizeof(double) * (size_t)r.n_trials;
                     size_t a = 0, b = 0;
                     if (!S.arena.take(sl.tab_bytes, a)) break;
@@ -414,6 +438,10 @@ void scheduler(Server *SP)
                     }
                     sl.tab_off = a;
                     sl.ylt_off = b;
+                    if (marked) {
+                        sl.marks = shape;
+                        sl.marks.d = reinterpret_cast<uint32_t *>(S.d_arena + a + marks_at);
+                    }
                     sl.req = std::move(r);
                     S.pending.pop_front();
                     sl.busy = true;
@@ -440,7 +468,7 @@ void scheduler(Server *SP)
             const int buf = (int)(S.iter & 1);
             std::vector<int> part[3], big, fold;
             std::vector<int64_t> slice;
-            bool big_first = false;   // the oldest request is a large one: its launch goes first
+            bool big_first = false;   // the oldest request has launches of its own: they go first
             {
                 std::lock_guard<std::mutex> lk(S.mu);
                 std::vector<std::pair<double, int>> order;
@@ -473,10 +501,10 @@ void scheduler(Server *SP)
                     }
                     slice[o.second] = take;
                     left_budget -= (double)take;
-                    if (head) big_first = sl.large && !S.cfg.folded;
+                    if (head) big_first = sl.own;
                     if (S.cfg.folded)
                         fold.push_back(o.second);
-                    else if (sl.large)
+                    else if (sl.own)
                         big.push_back(o.second);
                     else
                         part[sl.jp == 8 ? 0 : sl.jp == 16 ? 1 : 2].push_back(o.second);
@@ -573,7 +601,8 @@ void scheduler(Server *SP)
                 }
             };
             auto launch_large = [&] {
-                // large slices, one single-layer register-rows launch each
+                // one single-layer launch per slice: over the marked events, or
+                // (large requests) over every row
                 for (int i : big) {
                     const Slot &sl = S.slots[i];
                     SimArgs sa;
@@ -597,8 +626,12 @@ void scheduler(Server *SP)
                     TermsF32 tm;
                     tm.occ_r = sl.rec.occ_r;
                     tm.occ_l = sl.rec.occ_l;
-                    launches += launch_simulate(sa, S.cfg.precision, sl.pw ? sl.pw : sl.jp, &tm, nullptr,
-                                                S.ctx->num_sms, S.stream);
+                    if (sl.marks.d)
+                        launches += launch_marked32(sa, sl.marks, S.cfg.precision, sl.pw != 0, sl.pw ? sl.pw : sl.jp, tm,
+                                                    fixed_scale(sl.req.bound), S.ctx->num_sms, S.stream);
+                    else
+                        launches += launch_simulate(sa, S.cfg.precision, sl.pw ? sl.pw : sl.jp, &tm, nullptr,
+                                                    S.ctx->num_sms, S.stream);
                     finish_if_last(i);
                 }
             };
@@ -791,6 +824,10 @@ are_status are_submit(are_ctx *ctx, const are_request *req, int64_t *ticket)
                 r.elts.push_back(req->elt_handles[j]);
                 r.entries += e->second.n;
             }
+            r.terms = positive_zeros(req->terms);
+            r.bound = loss_bound(ctx, r.elts, r.terms);
+            r.marked = use_marks(S->cfg.precision, *S->y, r.bound,
+                                 marked_share(ctx, r.elts, r.terms, r.entries, S->y->catalog));
             for (int32_t i = 0; i < req->n_rp; ++i) {
                 r.ranks[i] = rank_for_return_period(req->n_trials, req->return_periods[i]);
                 ARE_CHECK(r.ranks[i] >= 1, ARE_EINVAL, "return period must be finite and >= 1");
@@ -800,7 +837,6 @@ are_status are_submit(are_ctx *ctx, const are_request *req, int64_t *ticket)
                 ARE_CHECK(r.ranks[req->n_rp + i] >= 1, ARE_EINVAL, "TVaR level must lie in (0, 1)");
             }
         }
-        r.terms = positive_zeros(req->terms);
         r.n_trials = req->n_trials;
         r.n_rp = req->n_rp;
         r.n_tv = req->n_tv;
