@@ -1836,25 +1836,25 @@ are_status are_risk_measures(are_ctx *ctx, const double *ylt, int64_t n,
             tmp = (double *)dalloc(ctx, sizeof(double) * n);
             d_y = tmp;
         }
-        std::vector<double> res(2 * ranks.size());
+        std::vector<double> res(ranks.size());
         try {
             if (tmp) copy_in(tmp, ylt, sizeof(double) * n, s);
             for (size_t b = 0; b < ranks.size(); b += kMaxTargets) {
                 const int nt = (int)std::min<size_t>(kMaxTargets, ranks.size() - b);
                 const int values = std::min(std::max(n_rp - (int32_t)b, 0), nt);
-                ctx->launches += launch_select(d_y, n, ranks.data() + b, nt, values, nullptr, ctx->sel, ctx->num_sms, s);
-                ARE_CUDA_TRY(cudaMemcpyAsync(ctx->h_result, ctx->sel.result, sizeof(double) * 2 * nt,
-                                             cudaMemcpyDeviceToHost, s));
+                double *out[kMaxTargets];   // the kernel writes the pinned results
+                for (int t = 0; t < nt; ++t) out[t] = ctx->h_result + t;
+                ctx->launches += launch_select(d_y, n, ranks.data() + b, nt, values, out, ctx->sel, ctx->num_sms, s);
                 ARE_CUDA_TRY(cudaStreamSynchronize(s));
-                std::memcpy(res.data() + 2 * b, ctx->h_result, sizeof(double) * 2 * nt);
+                std::memcpy(res.data() + b, ctx->h_result, sizeof(double) * nt);
             }
         } catch (...) {
             dfree(ctx, tmp, sizeof(double) * n);
             throw;
         }
         dfree(ctx, tmp, sizeof(double) * n);
-        for (int32_t r = 0; r < n_rp; ++r) pml_out[r] = res[2 * r];
-        for (int32_t r = 0; r < n_tv; ++r) tvar_out[r] = res[2 * (n_rp + r) + 1];
+        for (int32_t r = 0; r < n_rp; ++r) pml_out[r] = res[r];
+        for (int32_t r = 0; r < n_tv; ++r) tvar_out[r] = res[n_rp + r];
     });
 }
 
@@ -1966,7 +1966,7 @@ are_status are_risk_measures_batch(are_ctx *ctx, const double *const *ylts, int3
         CallStream cs(ctx, stream);
         const size_t ptr_bytes = (sizeof(double *) * n_ylt + 255) / 256 * 256;
         if (!ctx->sel_multi.coop) select_alloc(ctx->sel_multi, kMultiGroups);
-        const size_t need = ptr_bytes + sizeof(double) * 2 * kMaxTargets * (size_t)n_ylt;
+        const size_t need = ptr_bytes;
         if (ctx->multi_bytes < need) {
             ARE_CUDA_TRY(cudaStreamSynchronize(cs.s));
             dfree(ctx, ctx->d_multi, ctx->multi_bytes);
@@ -1986,14 +1986,11 @@ are_status are_risk_measures_batch(are_ctx *ctx, const double *const *ylts, int3
         const double *const *d_ptrs = static_cast<const double *const *>(ctx->d_multi);
         ARE_CUDA_TRY(cudaMemcpyAsync(ctx->d_multi, ylts, sizeof(double *) * n_ylt,
                                      cudaMemcpyHostToDevice, cs.s));
-        double *d_res = reinterpret_cast<double *>(static_cast<unsigned char *>(ctx->d_multi) + ptr_bytes);
         for (size_t b = 0; b < ranks.size(); b += kMaxTargets) {
             const int nt = (int)std::min<size_t>(kMaxTargets, ranks.size() - b);
             const int values = std::min(std::max(n_rp - (int32_t)b, 0), nt);
-            ctx->launches += launch_select_multi(d_ptrs, n_ylt, n, ranks.data() + b, nt, values, d_res,
-                                                 ctx->sel_multi, ctx->num_sms, cs.s);
-            ARE_CUDA_TRY(cudaMemcpyAsync(ctx->h_multi, d_res, sizeof(double) * count,
-                                         cudaMemcpyDeviceToHost, cs.s));
+            ctx->launches += launch_select_multi(d_ptrs, n_ylt, n, ranks.data() + b, nt, values, ctx->h_multi,
+                                                 ctx->sel_multi, ctx->num_sms, cs.s);   // (pinned)
             ARE_CUDA_TRY(cudaStreamSynchronize(cs.s));
             for (int32_t y = 0; y < n_ylt; ++y)
                 for (int t = 0; t < nt; ++t) {

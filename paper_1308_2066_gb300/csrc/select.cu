@@ -198,15 +198,17 @@ __device__ __forceinline__ void hist_add(uint32_t *h, bool on, uint32_t bin, int
     else if (on && bin != b0) atomicAdd(h + bin, 1u);
 }
 
-// One warp: find the bucket of h (256 counts) that holds the wanted rank,
+// One warp: find the bucket of h (256 counts in global, or SHARED, memory) that holds the wanted rank,
 // counting down from the top bucket, and extend the target's prefix.
+template <bool SHARED = false>
 __device__ __forceinline__ void pick(const uint32_t *h, unsigned long long *st, int shift, int lane)
 {
     uint32_t c[8];
     unsigned long long lane_sum = 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        c[i] = __ldcg(h + kBins - 1 - (lane * 8 + i));   // lane 0 holds the top buckets
+        const uint32_t *at = h + kBins - 1 - (lane * 8 + i);   // lane 0 holds the top buckets
+        c[i] = SHARED ? *at : __ldcg(at);
         lane_sum += c[i];
     }
     unsigned long long incl = lane_sum;
@@ -432,9 +434,9 @@ __global__ void __launch_bounds__(kThreads) k_tail(Sel s, int64_t n, int nt, Ran
 //
 // Three targets of 1M losses take 43 us (two 8-bit digits and up to 16384
 // kept keys: 83), eight 78 us (302), eight with a run of ties of 2% 79 us
-// (463: it took the radix passes); 1000 losses 26 us (34); 64 YLTs of 100,000
-// at a time 363 us with the copy back (ten launches: 549).  What is left is
-// latency: the launch, three barriers and the chains between them.
+// (463: it took the radix passes); 1000 losses 18 us in one block (34); 64 YLTs
+// of 100,000 at a time 360 us (ten launches: 549).  What is left is latency:
+// the launch, three barriers and the chains between them.
 //
 // The scratch of a group is left ready for the next YLT: histogram A is
 // cleared in C (its readers are past the barrier before), histogram B in A and
@@ -448,6 +450,7 @@ constexpr int kBitsB = 11, kBinsB = 1 << kBitsB;
 constexpr int kShiftA = 64 - kBitsA, kShiftB = kShiftA - kBitsB;
 static_assert(kShiftB == 40, "the radix passes go on with the fourth digit of 8 bits");
 constexpr size_t kCoopSmem = sizeof(uint32_t) * kMaxTargets * kBinsB;
+constexpr int64_t kOneBlock = 8192;     // values that one block selects from by itself: 8 a thread
 static_assert(kCoopSmem >= sizeof(uint32_t) * kBinsA && kCoopSmem >= kCand * 12ull, "what the passes share");
 
 // One group's scratch, zero before its first use.
@@ -573,10 +576,23 @@ __device__ __forceinline__ void for_values(const double *v, int64_t n, int rank,
     }
 }
 
+// ONE: a single YLT of few values by one block, its counts, sums and keys in
+// shared memory and its barriers the block's.
+struct KeptKeys {
+    unsigned long long key[kMaxTargets * kCand];
+    uint32_t times[kMaxTargets * kCand];
+    uint32_t kept[kMaxTargets];
+    unsigned int over;
+};
+
+template <bool ONE>
 __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_constant__ CoopArgs args)
 {
-    cg::grid_group grid = cg::this_grid();
-    extern __shared__ __align__(16) uint32_t h[];        // kCoopSmem
+    extern __shared__ __align__(16) uint32_t h[];        // kCoopSmem (ONE: and KeptKeys)
+    auto barrier = [] {
+        if constexpr (ONE) __syncthreads();
+        else cg::this_grid().sync();
+    };
     __shared__ unsigned long long st[2 * kMaxTargets];   // per target: key prefix, rank left (the same in every block)
     __shared__ unsigned long long acc[kMaxTargets * kAccWords];
     __shared__ uint64_t rep[kMaxTargets];                // per target: the block's first candidate, ~0: none; then its key
@@ -584,14 +600,20 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
     __shared__ uint32_t warp_sum[kCoopThreads / 32];
     __shared__ unsigned int s_mag;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int group = blockIdx.x / args.per, rank = blockIdx.x % args.per, groups = gridDim.x / args.per;
+    const int per = ONE ? 1 : args.per, group = blockIdx.x / per, rank = blockIdx.x % per, groups = gridDim.x / per;
     const int nt = args.nt;
     const int64_t n = args.n;
     CoopScratch &S = args.scratch[group];
-    unsigned int *const over = args.scratch[0].over;
-    auto mine = [&](int i) { return i * args.per + rank; };   // a block's share of the group's clearing
+    KeptKeys &K = *reinterpret_cast<KeptKeys *>(h + kCoopSmem / sizeof(uint32_t));   // ONE
+    unsigned long long *const cand_key = ONE ? K.key : S.key;
+    uint32_t *const cand_times = ONE ? K.times : S.times, *const kept = ONE ? K.kept : S.kept;
+    unsigned int *const over = ONE ? &K.over : args.scratch[0].over;
+    // counts and counters of the scratch: past L1 in global memory
+    auto get = [](const auto *x) { return ONE ? *x : __ldcg(x); };
+    auto mine = [&](int i) { return i * per + rank; };   // a block's share of the group's clearing
+    (void)mine;
     for (int y0 = 0, round = 0; y0 < args.n_ylt; y0 += groups, ++round) {
-        const int y = y0 + group, turn = round & 1;
+        const int y = y0 + group, turn = ONE ? 0 : round & 1;
         const bool on = y < args.n_ylt;
         const bool final_round = y0 + groups >= args.n_ylt;
         const double *__restrict__ v = on ? (args.many ? args.many[y] : args.single) : nullptr;
@@ -602,12 +624,13 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
         }
         if (tid == 0) s_mag = 0;
         for (int i = tid; i < kBinsA; i += kCoopThreads) h[i] = 0;
-        for (int i = mine(tid); i < kMaxTargets * kBinsB; i += args.per * kCoopThreads) S.b[i] = 0;
+        if constexpr (!ONE)
+            for (int i = mine(tid); i < kMaxTargets * kBinsB; i += per * kCoopThreads) S.b[i] = 0;
         if (blockIdx.x == 0 && tid == 0) over[turn] = 0;
         __syncthreads();
         if (on) {
             unsigned int mag = 0;
-            for_values(v, n, rank, args.per, [&](uint64_t k, double x, bool ok) {
+            for_values(v, n, rank, per, [&](uint64_t k, double x, bool ok) {
                 hist_add(h, ok, (uint32_t)(k >> kShiftA), lane);
                 const unsigned int m32 =
                     (unsigned int)(((unsigned long long)__double_as_longlong(x) >> 32) & 0x7fffffffu);
@@ -621,18 +644,21 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
             if (lane == 0 && mag) atomicMax(&s_mag, mag);
         }
         __syncthreads();
-        for (int i = tid; i < kBinsA; i += kCoopThreads)
-            if (h[i]) atomicAdd(&S.a[i], h[i]);
-        if (tid == 0 && s_mag) atomicMax(&S.mag[turn], s_mag);
-        grid.sync();
+        if constexpr (!ONE) {
+            for (int i = tid; i < kBinsA; i += kCoopThreads)
+                if (h[i]) atomicAdd(&S.a[i], h[i]);
+            if (tid == 0 && s_mag) atomicMax(&S.mag[turn], s_mag);
+            barrier();
+        }
         // every block finds every target's bin: thread i holds 8 bins, the
         // top ones first
         {
-            constexpr int per = kBinsA / kCoopThreads;
-            uint32_t c[per], sum = 0;
+            constexpr int bins = kBinsA / kCoopThreads;
+            const uint32_t *const counts = ONE ? h : S.a;
+            uint32_t c[bins], sum = 0;
 #pragma unroll
-            for (int i = 0; i < per; ++i) {
-                c[i] = __ldcg(&S.a[kBinsA - 1 - (tid * per + i)]);
+            for (int i = 0; i < bins; ++i) {
+                c[i] = get(counts + kBinsA - 1 - (tid * bins + i));
                 sum += c[i];
             }
             uint32_t incl = sum;
@@ -661,7 +687,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
                     uint64_t above = excl;
                     int i = 0;
                     while (above + c[i] < r) above += c[i++];
-                    st[2 * t] = (uint64_t)(kBinsA - 1 - (tid * per + i)) << kShiftA;
+                    st[2 * t] = (uint64_t)(kBinsA - 1 - (tid * bins + i)) << kShiftA;
                     st[2 * t + 1] = r - above;
                 }
             }
@@ -670,8 +696,9 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
         // B. the next bits of the targets' bins (a bin shared by targets once)
         for (int i = tid; i < nt * kBinsB; i += kCoopThreads) h[i] = 0;
         if (rank == 0) {
-            for (int i = tid; i < kMaxTargets * kAccWords; i += kCoopThreads) S.acc[i] = 0;
-            if (tid < kMaxTargets) S.kept[tid] = 0;
+            if constexpr (!ONE)
+                for (int i = tid; i < kMaxTargets * kAccWords; i += kCoopThreads) S.acc[i] = 0;
+            if (tid < kMaxTargets) kept[tid] = 0;
         }
         __syncthreads();
         uint32_t PA[kMaxTargets];
@@ -685,7 +712,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
                 if (q < t && PA[q] == PA[t]) first[t] = q;
         }
         if (on)
-            for_values(v, n, rank, args.per, [&](uint64_t k, double, bool ok) {
+            for_values(v, n, rank, per, [&](uint64_t k, double, bool ok) {
                 const uint32_t p = (uint32_t)(k >> kShiftA);
 #pragma unroll
                 for (int t = 0; t < kMaxTargets; ++t)
@@ -693,19 +720,21 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
                         hist_add(h + t * kBinsB, ok && p == PA[t], (uint32_t)(k >> kShiftB) & (kBinsB - 1), lane);
             });
         __syncthreads();
-        for (int i = tid; i < nt * kBinsB; i += kCoopThreads)
-            if (h[i]) atomicAdd(&S.b[i], h[i]);
-        grid.sync();
+        if constexpr (!ONE) {
+            for (int i = tid; i < nt * kBinsB; i += kCoopThreads)
+                if (h[i]) atomicAdd(&S.b[i], h[i]);
+            barrier();
+        }
         if (warp < nt) {   // warp t: lane i holds 64 bins, the top ones first
             int q = 0;
 #pragma unroll
             for (int t = 0; t < kMaxTargets; ++t)
                 if (t == warp) q = first[t];
-            const uint32_t *b = S.b + q * kBinsB;
-            constexpr int per = kBinsB / 32;
+            const uint32_t *b = (ONE ? h : S.b) + q * kBinsB;
+            constexpr int bins = kBinsB / 32;
             uint32_t sum = 0;
-#pragma unroll 16
-            for (int i = 0; i < per; ++i) sum += __ldcg(b + kBinsB - 1 - (lane * per + i));
+#pragma unroll 32
+            for (int i = 0; i < bins; ++i) sum += get(b + kBinsB - 1 - (lane * bins + i));
             uint32_t incl = sum;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
@@ -716,10 +745,10 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
             const uint64_t r = st[2 * warp + 1];
             // the lane whose bins hold the rank, then its bins, two per lane
             const int l = __ffs(__ballot_sync(kFull, excl < r && r <= incl)) - 1;
-            static_assert(per == 64, "two bins per lane");
+            static_assert(bins == 64, "two bins per lane");
             const uint64_t left = r - __shfl_sync(kFull, excl, l);
-            const int i0 = l * per + 2 * lane;
-            const uint32_t c0 = __ldcg(b + kBinsB - 1 - i0), c1 = __ldcg(b + kBinsB - 2 - i0);
+            const int i0 = l * bins + 2 * lane;
+            const uint32_t c0 = get(b + kBinsB - 1 - i0), c1 = get(b + kBinsB - 2 - i0);
             uint32_t run = c0 + c1;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
@@ -740,7 +769,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
         for (int i = tid; i < kMaxTargets * kAccWords; i += kCoopThreads) acc[i] = 0;
         __syncthreads();
         // C. the keys of the targets' bins, and the tail sums above them
-        const int sc = tail_scale(__ldcg(&S.mag[turn]));
+        const int sc = tail_scale(ONE ? s_mag : __ldcg(&S.mag[turn]));
         uint32_t P[kMaxTargets];
 #pragma unroll
         for (int t = 0; t < kMaxTargets; ++t) {
@@ -751,14 +780,14 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
                 if (q < t && P[q] == P[t]) first[t] = q;
         }
         auto keep = [&](int t, uint64_t k, uint32_t times) {
-            const uint32_t at = atomicAdd(&S.kept[t], 1u);
+            const uint32_t at = atomicAdd(&kept[t], 1u);
             if (at < kCand) {
-                S.key[t * kCand + at] = k;
-                S.times[t * kCand + at] = times;
+                cand_key[t * kCand + at] = k;
+                cand_times[t * kCand + at] = times;
             }
         };
         if (on)
-            for_values(v, n, rank, args.per, [&](uint64_t k, double x, bool ok) {
+            for_values(v, n, rank, per, [&](uint64_t k, double x, bool ok) {
                 const uint32_t p = (uint32_t)(k >> kShiftB);
 #pragma unroll
                 for (int t = 0; t < kMaxTargets; ++t) {
@@ -780,21 +809,24 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
                         acc_add(acc + t * kAccWords, ok && p > P[t], x, 1u, sc, lane);
                 }
             });
-        for (int i = mine(tid); i < kBinsA; i += args.per * kCoopThreads) S.a[i] = 0;
-        if (rank == 0 && tid == 0) S.mag[turn ^ 1] = 0;
+        if constexpr (!ONE) {
+            for (int i = mine(tid); i < kBinsA; i += per * kCoopThreads) S.a[i] = 0;
+            if (rank == 0 && tid == 0) S.mag[turn ^ 1] = 0;
+        }
         __syncthreads();
         if (tid < nt && rep_times[tid]) keep(tid, rep[tid], rep_times[tid]);
-        for (int i = tid; i < nt * kAccWords; i += kCoopThreads)
-            if (acc[i]) atomicAdd(&S.acc[i], acc[i]);
+        if constexpr (!ONE)
+            for (int i = tid; i < nt * kAccWords; i += kCoopThreads)
+                if (acc[i]) atomicAdd(&S.acc[i], acc[i]);
         __syncthreads();
-        if (tid < nt && __ldcg(&S.kept[tid]) > kCand) atomicExch(over + turn, 1u);
-        grid.sync();
+        if (tid < nt && get(&kept[tid]) > kCand) atomicExch(over + turn, 1u);
+        barrier();
         double *const res = args.results ? args.results + (size_t)y * 2 * kMaxTargets : S.result;
-        const bool fits = __ldcg(over + turn) == 0;
+        const bool fits = get(over + turn) == 0;
         if (fits && on) {
             // D. block j of the group: targets j, j + per, ..., a warp each where
             // a block has several
-            const bool warps = args.per < nt;
+            const bool warps = ONE || per < nt;
             constexpr int kWarpCand = 512;   // keys that a warp keeps in shared memory
             static_assert(kMaxTargets * kWarpCand * 12 <= kCoopSmem, "each target's keys");
             const int width = warps ? 32 : kCoopThreads, at = warps ? lane : tid;
@@ -803,20 +835,20 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
                 else __syncthreads();
             };
             const int t = warps ? warp : rank;
-            if (t < nt && (!warps || t % args.per == rank)) {
+            if (t < nt && (!warps || t % per == rank)) {
                 int q = 0;
 #pragma unroll
                 for (int i = 0; i < kMaxTargets; ++i)
                     if (i == t) q = first[i];
-                const int c = (int)__ldcg(&S.kept[q]);
-                const unsigned long long *keys = S.key + q * kCand;
-                const uint32_t *times = S.times + q * kCand;
+                const int c = (int)get(&kept[q]);
+                const unsigned long long *keys = cand_key + q * kCand;
+                const uint32_t *times = cand_times + q * kCand;
                 unsigned long long *const sk = reinterpret_cast<unsigned long long *>(h) + (warps ? t * kWarpCand : 0);
                 uint32_t *const sn = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned long long *>(h) +
                                                                   (warps ? kMaxTargets * kWarpCand : kCand)) +
                                      (warps ? t * kWarpCand : 0);
                 unsigned long long *const sum = acc + (warps ? t * kAccWords : 0);
-                if (!warps || c <= kWarpCand) {
+                if (!ONE && (!warps || c <= kWarpCand)) {
                     for (int i = at; i < c; i += width) {
                         sk[i] = __ldcg(keys + i);
                         sn[i] = __ldcg(times + i);
@@ -824,7 +856,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
                     keys = sk;
                     times = sn;
                 }
-                if (at < kAccWords) sum[at] = 0;
+                if (!ONE && at < kAccWords) sum[at] = 0;   // (ONE: on with the sums of C)
                 join();
                 // the key with fewer than r values above it and r or more at or above
                 const uint64_t r = st[2 * t + 1];
@@ -849,7 +881,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
                 join();
                 if (at == 0) {
                     unsigned long long A[kAccWords];
-                    for (int i = 0; i < kAccWords; ++i) A[i] = sum[i] + __ldcg(&S.acc[t * kAccWords + i]);
+                    for (int i = 0; i < kAccWords; ++i) A[i] = sum[i] + (ONE ? 0ull : __ldcg(&S.acc[t * kAccWords + i]));
                     tail_result(A, kt, args.m[t], sc, (args.means >> t) & 1u, res + 2 * t);
                     if (args.out[t]) *args.out[t] = res[2 * t + ((args.means >> t) & 1u)];
                 }
@@ -859,9 +891,9 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
             // the YLT, then the bins' values above the keys
             for (int pass = 3; pass < 8; ++pass) {
                 const int shift = 56 - 8 * pass;
-                uint32_t *gh = S.c + (size_t)(pass % 3) * kMaxTargets * kBins;
+                uint32_t *gh = ONE ? h : S.c + (size_t)(pass % 3) * kMaxTargets * kBins;
                 for (int i = tid; i < nt * kBins; i += kCoopThreads) h[i] = 0;
-                if (rank == 0 && pass >= 5) {   // the buffer of pass - 2, read by every block already
+                if (!ONE && rank == 0 && pass >= 5) {   // the buffer of pass - 2, read by every block already
                     uint32_t *old = S.c + (size_t)((pass - 2) % 3) * kMaxTargets * kBins;
                     for (int i = tid; i < kMaxTargets * kBins; i += kCoopThreads) old[i] = 0;
                 }
@@ -870,7 +902,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
 #pragma unroll
                 for (int t = 0; t < kMaxTargets; ++t) pre[t] = t < nt ? st[2 * t] >> (shift + 8) : 0ull;
                 if (on)
-                    for_values(v, n, rank, args.per, [&](uint64_t k, double, bool ok) {
+                    for_values(v, n, rank, per, [&](uint64_t k, double, bool ok) {
 #pragma unroll
                         for (int t = 0; t < kMaxTargets; ++t) {
                             if (t >= nt) break;
@@ -879,20 +911,22 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
                         }
                     });
                 __syncthreads();
-                for (int i = tid; i < nt * kBins; i += kCoopThreads)
-                    if (h[i]) atomicAdd(&gh[i], h[i]);
-                grid.sync();
-                if (on && warp < nt)
-                    pick(gh + warp * kBins, st + 2 * warp, shift, lane);
+                if constexpr (!ONE) {
+                    for (int i = tid; i < nt * kBins; i += kCoopThreads)
+                        if (h[i]) atomicAdd(&gh[i], h[i]);
+                    barrier();
+                }
+                if (on && warp < nt) pick<ONE>(gh + warp * kBins, st + 2 * warp, shift, lane);
                 __syncthreads();
             }
-            for (int i = tid; i < nt * kAccWords; i += kCoopThreads) acc[i] = 0;
+            if constexpr (!ONE)   // (ONE: on with the sums of C)
+                for (int i = tid; i < nt * kAccWords; i += kCoopThreads) acc[i] = 0;
             __syncthreads();
             uint64_t kt[kMaxTargets];
 #pragma unroll
             for (int t = 0; t < kMaxTargets; ++t) kt[t] = t < nt ? st[2 * t] : ~0ull;
             if (on)
-                for_values(v, n, rank, args.per, [&](uint64_t k, double x, bool ok) {
+                for_values(v, n, rank, per, [&](uint64_t k, double x, bool ok) {
 #pragma unroll
                     for (int t = 0; t < kMaxTargets; ++t) {
                         if (t >= nt) break;
@@ -902,20 +936,23 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
                     }
                 });
             __syncthreads();
-            for (int i = tid; i < nt * kAccWords; i += kCoopThreads)
-                if (acc[i]) atomicAdd(&S.acc[i], acc[i]);
-            grid.sync();
+            if constexpr (!ONE) {
+                for (int i = tid; i < nt * kAccWords; i += kCoopThreads)
+                    if (acc[i]) atomicAdd(&S.acc[i], acc[i]);
+                barrier();
+            }
             if (on && rank == 0) {
                 if (tid < nt) {
                     unsigned long long A[kAccWords];
-                    for (int i = 0; i < kAccWords; ++i) A[i] = __ldcg(&S.acc[tid * kAccWords + i]);
+                    for (int i = 0; i < kAccWords; ++i) A[i] = ONE ? acc[tid * kAccWords + i] : __ldcg(&S.acc[tid * kAccWords + i]);
                     tail_result(A, st[2 * tid], args.m[tid], sc, (args.means >> tid) & 1u, res + 2 * tid);
                     if (args.out[tid]) *args.out[tid] = res[2 * tid + ((args.means >> tid) & 1u)];
                 }
-                for (int i = tid; i < 3 * kMaxTargets * kBins; i += kCoopThreads) S.c[i] = 0;
+                if constexpr (!ONE)
+                    for (int i = tid; i < 3 * kMaxTargets * kBins; i += kCoopThreads) S.c[i] = 0;
             }
         }
-        if (final_round && rank == 0 && tid == 0) S.mag[0] = S.mag[1] = 0;
+        if (!ONE && final_round && rank == 0 && tid == 0) S.mag[0] = S.mag[1] = 0;
         __syncthreads();
     }
 }
@@ -923,14 +960,21 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
 // One launch over n_ylt YLTs: `args` but for the groups.
 cudaError_t enqueue_coop(CoopArgs args, int max_groups, int num_sms, cudaStream_t st)
 {
-    const int per_sm = fit_blocks(reinterpret_cast<const void *>(k_select_coop), kCoopThreads, kCoopSmem);
+    if (args.n_ylt == 1 && args.n <= kOneBlock) {
+        constexpr size_t smem = kCoopSmem + sizeof(KeptKeys);
+        args.per = 1;
+        fit_blocks(reinterpret_cast<const void *>(k_select_coop<true>), kCoopThreads, smem);
+        k_select_coop<true><<<1, kCoopThreads, smem, st>>>(args);
+        return cudaGetLastError();
+    }
+    const int per_sm = fit_blocks(reinterpret_cast<const void *>(k_select_coop<false>), kCoopThreads, kCoopSmem);
     const int64_t resident = (int64_t)num_sms * per_sm;
     // blocks that a YLT can use, kPre values per thread each
     const int64_t useful = std::max<int64_t>(1, (args.n + kCoopThreads * kPre - 1) / (kCoopThreads * kPre));
     const int64_t groups = std::min<int64_t>({(int64_t)args.n_ylt, (int64_t)max_groups, resident});
     args.per = (int)std::min(useful, resident / groups);
     void *p[] = {&args};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_select_coop), dim3((unsigned)(groups * args.per)),
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_select_coop<false>), dim3((unsigned)(groups * args.per)),
                                        dim3(kCoopThreads), p, kCoopSmem, st);
 }
 

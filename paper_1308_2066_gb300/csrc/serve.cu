@@ -132,7 +132,7 @@ struct Slot {
     uint64_t finish_iter = 0;       // iteration whose completion posts the result
     cudaEvent_t done_ev = nullptr;  // recorded after the result's copy: posts it as soon as it fires
     SelectScratch sel;
-    double *h_res = nullptr;        // pinned, 2 * kMaxTargets
+    double *h_res = nullptr;        // pinned, kMaxTargets
     Clock::time_point t_admit;
 };
 
@@ -189,8 +189,8 @@ void post(Server &S, const Request &r, are_status st, const double *res, Clock::
     p.res.n_tv = r.n_tv;
     p.res.n_trials = r.n_trials;
     if (res) {
-        for (int i = 0; i < r.n_rp; ++i) p.res.pml[i] = res[2 * i];
-        for (int i = 0; i < r.n_tv; ++i) p.res.tvar[i] = res[2 * (r.n_rp + i) + 1];
+        for (int i = 0; i < r.n_rp; ++i) p.res.pml[i] = res[i];
+        for (int i = 0; i < r.n_tv; ++i) p.res.tvar[i] = res[r.n_rp + i];
     }
     const Clock::time_point now = Clock::now();
     p.res.total_us = us_between(r.t_submit, now);
@@ -536,7 +536,7 @@ void scheduler(Server *SP)
                 ARE_CUDA_TRY(cudaMemcpyAsync(d, h, off, cudaMemcpyHostToDevice, S.stream));
             int launches = 0;
             // A request whose last slice is in this launch has its risk
-            // measures selected and copied right after its own kernels, then
+            // measures selected right after its own kernels, then
             // its own completion event: its result is posted when that
             // fires, not when the whole iteration has.
             auto finish_if_last = [&](int i) {
@@ -544,11 +544,11 @@ void scheduler(Server *SP)
                 Slot &sl = S.slots[i];
                 sl.launched += slice[i];
                 if (sl.launched < sl.req.n_trials) return;
+                double *out[kMaxTargets];   // the kernel writes the pinned results
+                for (int t = 0; t < kMaxTargets; ++t) out[t] = sl.h_res + t;
                 launches += launch_select(reinterpret_cast<const double *>(S.d_arena + sl.ylt_off),
                                           sl.req.n_trials, sl.req.ranks, sl.req.n_rp + sl.req.n_tv, sl.req.n_rp,
-                                          nullptr, sl.sel, S.ctx->num_sms, S.stream);
-                ARE_CUDA_TRY(cudaMemcpyAsync(sl.h_res, sl.sel.result, sizeof(double) * 2 * kMaxTargets,
-                                             cudaMemcpyDeviceToHost, S.stream));
+                                          out, sl.sel, S.ctx->num_sms, S.stream);
                 ARE_CUDA_TRY(cudaEventRecord(sl.done_ev, S.stream));
                 sl.finishing = true;
                 sl.finish_iter = S.iter;
@@ -773,7 +773,7 @@ are_status are_server_start(are_ctx *ctx, int32_t yet, const are_server_cfg *cfg
             S->slots.resize(cfg->max_inflight);
             for (Slot &sl : S->slots) {
                 select_alloc(sl.sel, 1);
-                ARE_CUDA_TRY(cudaMallocHost(&sl.h_res, sizeof(double) * 2 * kMaxTargets));
+                ARE_CUDA_TRY(cudaMallocHost(&sl.h_res, sizeof(double) * kMaxTargets));
                 ARE_CUDA_TRY(cudaEventCreateWithFlags(&sl.done_ev, cudaEventDisableTiming));
             }
             S->work_bytes = 3 * up(sizeof(LayerF32) * cfg->max_inflight) + 3 * sizeof(unsigned long long);
