@@ -1552,10 +1552,9 @@ static void simulate_streamed(are_ctx *ctx, int32_t layer, int32_t catalog_size,
             v.d_off = d_off;
             for (int i = 0; i < 2; ++i) buf[i] = (int32_t *)dalloc(ctx, buf_bytes);
             if (id_bits)
-                for (int i = 0; i < 2; ++i) {
-                    wbuf[i] = (uint32_t *)dalloc(ctx, wbuf_bytes);
-                    ARE_CUDA_TRY(cudaMemsetAsync(wbuf[i], 0, wbuf_bytes, s));
-                }
+                // (not cleared, 340 MB at the default chunk: the unpacking masks
+                // out the bits past a chunk's ids)
+                for (int i = 0; i < 2; ++i) wbuf[i] = (uint32_t *)dalloc(ctx, wbuf_bytes);
             d_out = dev_out ? ylt : (double *)dalloc(ctx, sizeof(double) * n_trials);
             for (cudaEvent_t *e : {&start, &ready[0], &ready[1], &done[0], &done[1]})
                 ARE_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
