@@ -132,12 +132,12 @@ struct Compact {
 // Packed table of one layer: catalog rows of 32 or 64 bytes holding each
 // event's non-zero terms in column order behind the mask of their columns,
 // a counter and the overflow terms, in one allocation laid out [rows |
-// counter (256 B) | overflow].  FP64 (built from the ELT entries by
-// launch_pack64_direct):
+// counter (256 B) | overflow].  Built from the ELT entries by
+// launch_tile_rows (ELTs in buckets), or launch_pack32/64_direct (catalogs
+// of more than kMaxBucketedId events).  FP64:
 // rw = 4 or 8 64-bit words per row, the mask and the overflow offset in word
 // 0, up to rw - 1 terms inline and every term of a longer row in the
-// overflow.  FP32 (built from the ELT entries by launch_pack32_direct):
-// rw = 8 or 16 32-bit words, the mask in word 0, up to rw - 1 terms inline;
+// overflow.  FP32: rw = 8 or 16 32-bit words, the mask in word 0, up to rw - 1 terms inline;
 // a longer row keeps rw - 2 inline and the offset of the rest in its last
 // word.  The row size follows the layer's entries per catalog event
 // (packed_row_words).
@@ -229,8 +229,8 @@ struct SimArgs {
     int kernel;              // 1 staged, 2 register rows, 3 (FP64) staged screen
     int epl;                 // staged FP32 kernel: events per lane per batch (1 or 2);
                              // register-rows kernel: groups of 32 events per batch (1 or 2);
-                             // 0: the kernel's default (one event per lane; one group over
-                             // 32-byte FP32 rows, two over wider rows and FP64 rows)
+                             // 0: the kernel's default (one event per lane; one group, two
+                             // over 32-byte FP64 rows)
     double *marg;            // per-occurrence marginals, or null
     double *occ_max;         // largest occurrence loss per trial, or null
     int64_t marg_base;       // event index of marg[0]

@@ -16,6 +16,10 @@
 // trial, so it is formed once per ELT entry here instead of once per
 // occurrence; every occurrence still reads its event's whole row.  An event
 // the ELT does not hold has x = 0 and stores f_j(0) = 0.
+//
+// The tables are built here where the ELTs' entries are not in buckets of 256
+// events (ids past kMaxBucketedId) and for the staged kernels' dense FP64 and
+// screen tables; tile_rows.cu builds the others in one launch.
 #include <cuda_runtime.h>
 
 #include "are_internal.cuh"
@@ -154,7 +158,8 @@ __global__ void k_pack32_over(const ScatterArgs a, const uint32_t *__restrict__ 
 
 }  // namespace
 
-// Packed FP32 rows (pw words) straight from the layer's ELT entries: rows
+// Packed FP32 rows (pw words) straight from the layer's ELT entries (ids past
+// kMaxBucketedId; tile_rows.cu otherwise): rows
 // catalog x pw words, ovf room for every entry, ovf_used a device counter.
 // Three launches, no dense table.
 int launch_pack32_direct(const ScatterArgs &a, int32_t catalog, int pw, uint32_t *rows, float *ovf,
@@ -195,7 +200,8 @@ int packed_row_words(int n_elts, double terms_per_event, bool fp32)
     return terms_per_event <= 0.5 ? 4 : 8;
 }
 
-// Packed FP64 rows (rw words) straight from the layer's ELT entries: rows
+// Packed FP64 rows (rw words) straight from the layer's ELT entries (ids past
+// kMaxBucketedId; tile_rows.cu otherwise): rows
 // catalog x rw words, ovf room for every entry, ovf_used a device counter.
 // Three launches, no dense table.
 int launch_pack64_direct(const ScatterArgs &a, int32_t catalog, int rw, unsigned long long *rows, double *ovf,

@@ -280,7 +280,7 @@ struct BodyF32 {
     }
 };
 
-// Packed FP32 table (repack.cu, launch_pack32_direct): row e is PW = 8 or
+// Packed FP32 table (tile_rows.cu or repack.cu): row e is PW = 8 or
 // 16 words (32 or 64 bytes) -- word 0 the mask of the ELT columns whose term
 // is not 0, then up to PW - 1 of those terms in column order.  A row of more terms
 // keeps the first PW - 2 inline and in word PW - 1 the offset of the rest
@@ -379,7 +379,7 @@ __device__ __forceinline__ W4 load4w(const unsigned long long *p)
     return r;
 }
 
-// FP64 path over the packed FP64 table (repack.cu, launch_pack64_direct):
+// FP64 path over the packed FP64 table (tile_rows.cu or repack.cu):
 // row e is RW = 4 or 8 words (32 or 64 bytes) -- word 0 holds the mask of
 // the ELT columns whose term is not 0 (low 32 bits) and an overflow offset
 // (high 32 bits), words 1 .. RW - 1 the non-zero terms in column order.  A

@@ -73,7 +73,12 @@ void launch_t(const SimArgs &a, const TermsF64 &tm, int scale, int num_sms, cuda
 template <int RW>
 void go(const SimArgs &a, const TermsF64 &tm, int scale, int num_sms, cudaStream_t s)
 {
-    const bool two = a.epl != 1;
+    // Unless the caller asks for one: two groups of 32 events over 32-byte rows
+    // (12M occurrences, 120 events a trial: 72 us, one group 79), one over
+    // 64-byte rows, whose second group costs a block per SM (48M occurrences,
+    // 1M events: 1000 events a trial 459 us, two 502; 120 events 512 and 544).
+    // Five blocks of one group over 64-byte rows spill: 545.
+    const bool two = a.epl == 0 ? RW == 4 : a.epl != 1;
     if (a.off)
         two ? launch_t<RW, 2, false>(a, tm, scale, num_sms, s) : launch_t<RW, 1, false>(a, tm, scale, num_sms, s);
     else

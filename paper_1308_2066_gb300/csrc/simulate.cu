@@ -437,10 +437,19 @@ void launch_packed_t(const SimArgs &a, const TermsF32 &tm, int num_sms, cudaStre
     ARE_CUDA_TRY(cudaGetLastError());
 }
 
+// Groups of 32 events per batch, unless the caller asks for one: one.  Two put
+// twice the loads in flight per warp, but the second group's registers cost
+// the fifth block per SM and a trial's last batch is emptier.  Ragged trials,
+// 48M occurrences, one group against two, us: 64-byte packed rows, Kahan, 1M
+// events 244 / 330 (trials of 1000 events), 297 / 396 (120); 20,000 events 258
+// / 311 and 299 / 369; 2M events, past L2, 415 / 532; FP64 sums 265 / 377;
+// dense 64-byte rows, 1M events 218 / 250.  (Six blocks of one group spill: 314
+// and 238.)  32-byte rows, 12M occurrences: 60 / 58 at 120 events, 115 / 134 at
+// 20.  Both add a trial's events in the same order.
 template <int PW, int ACC>
 void launch_packed(const SimArgs &a, const TermsF32 &tm, int num_sms, cudaStream_t s)
 {
-    const bool two = a.epl == 0 ? PW > 8 : a.epl != 1;
+    const bool two = a.epl != 0 && a.epl != 1;
     if (a.off)
         two ? launch_packed_t<PW, 2, ACC, false>(a, tm, num_sms, s)
             : launch_packed_t<PW, 1, ACC, false>(a, tm, num_sms, s);
@@ -452,7 +461,7 @@ void launch_packed(const SimArgs &a, const TermsF32 &tm, int num_sms, cudaStream
 template <int JP, int ACC>
 void launch_rows(const SimArgs &a, const TermsF32 &tm, int num_sms, cudaStream_t s)
 {
-    const bool two = a.epl == 0 ? JP > 8 : a.epl != 1;
+    const bool two = a.epl == 0 ? JP > 16 : a.epl != 1;
     if (a.off)
         two ? launch_rows_t<JP, 2, ACC, false>(a, tm, num_sms, s)
             : launch_rows_t<JP, 1, ACC, false>(a, tm, num_sms, s);
