@@ -29,8 +29,10 @@ import hashlib
 import json
 import math
 import os
+import re
 import subprocess
 import sys
+import tempfile
 import threading
 import time
 
@@ -102,6 +104,7 @@ KERNEL_SOURCES = {
     "k_sim_items": ["sim_items.cu", "rows.cuh", "are_internal.cuh"],
     "k_simulate": ["simulate.cu", "are_internal.cuh"],
     "k_folded": ["folded.cu", "fixed.cuh", "are_internal.cuh"],
+    "k_marked": ["marked.cuh", "marked32.cu", "marked64.cu", "rows.cuh", "fixed.cuh", "are_internal.cuh"],
 }
 
 
@@ -219,6 +222,9 @@ def kernel_key(prec: int, J: int, tuned=None, rows=None, ragged=False) -> str:
     rb, packed = rows if rows else (None, False)
     u = t.get("rows_in_flight") or (1 if prec != 0 and (rb == 32 or (rb is None and J <= 8)) else 2)
     cur = "ragged" if ragged else "fixed"
+    if t.get("kernel") == 2 and t.get("rows_in_flight") == 0:   # the marked events' rows
+        form = "PackedF64" if prec == 0 else "PackedF32" if packed else "DenseF32"
+        return f"k_marked<{form}<{(rb or 32) // (8 if prec == 0 else 4)}>,{prec},{cur}>"
     if prec == 0:
         jp = math.ceil(J / 4) * 4
         kind = t.get("kernel", 2)
@@ -242,6 +248,50 @@ def layer_rows(are, ctx, layer, yet, prec, tuned=None):
     """(row_bytes, packed) of the rows the analysis of this layer reads per
     occurrence under the tuned kernel choice (the library's answer)."""
     return are.are_layer_rows(ctx, layer, yet, prec, (tuned or {}).get("kernel", -1))
+
+
+def read_every_row(are, ctx, prec, tuned, on=True, only=True):
+    """The register-rows choices of this precision over marked events (the
+    library's default form) set to read every occurrence's row, with the
+    default groups of 32 events, for one layer alone too where the choice is
+    a portfolio's; on=False: back to the default form.  only=False: all the
+    precision's choices made register rows.  Returns the tuned choice as it
+    then is (not timed in that form)."""
+    groups = (2 if prec == 0 else 1) if on else 0
+    with tempfile.TemporaryDirectory() as d:
+        path = os.path.join(d, "tune.jsonl")
+        are.are_tune_save(ctx, path)
+        with open(path) as f:
+            entries = [json.loads(ln) for ln in f]
+        for e in [e for e in entries if e["key"].endswith("_multi")]:
+            for jp in (range(4, 33, 4) if prec == 0 else (8, 16, 32)):
+                key = re.sub(r"_jp\d+_(ev\d+)_multi", rf"_jp{jp}_\1_single", e["key"])
+                if not any(x["key"] == key for x in entries):
+                    entries.append(dict(e, key=key, kernel=2, rows_in_flight=0))
+        with open(path, "w") as f:
+            for e in entries:
+                if e["key"].startswith(f"p{prec}_") and (e["kernel"] == 2 or not only) and \
+                        (not on or not only or e["rows_in_flight"] == 0):
+                    e["kernel"], e["rows_in_flight"] = 2, groups
+                f.write(json.dumps(e) + "\n")
+        are.are_tune_load(ctx, path)
+    return dict(tuned, rows_in_flight=groups, ms=None)
+
+
+def untuned_rows(are, ctx, layers, yet, prec, stream):
+    """Without tuning: the default register rows, every occurrence's row read."""
+    choice = are.are_autotune(ctx, layers, yet, prec, stream)   # makes the entries
+    read_every_row(are, ctx, prec, choice, only=False)
+
+
+def marked_choice(tuned) -> bool:
+    """Whether the tuner picked the form over the marked events."""
+    return bool(tuned) and tuned["kernel"] == 2 and tuned["rows_in_flight"] == 0
+
+
+MARKED_WHAT = ("the library's default: one bit per catalog event, built with the table in every step, "
+               "tells which occurrences can add a loss, and only their rows are read (the same results "
+               "bit for bit); not the headline, which reads the row of every occurrence")
 
 
 class Resident:
@@ -429,15 +479,17 @@ def roofline(n_events, n_trials, J, prec, sim_ms, tuned=None, ceiling=None, rows
                           "shapes_timed": len(shapes)}}
 
 
-def folded_roofline(n_events, n_trials, sim_ms):
-    """The folded table's trial pass: HBM traffic is the id stream and the
-    YLT; the values of the few events with h > 0 come from L2."""
+def folded_roofline(n_events, n_trials, sim_ms, key=None):
+    """The folded table's trial pass, or the pass over marked events (key):
+    HBM traffic is the id stream and the YLT; the values or rows of the few
+    events with a loss come from L2."""
     peak, src = hbm_peak()
+    key = key or kernel_key("folded", 0)
     bytes_ = 4 * n_events + 8 * n_trials
     achieved = bytes_ / (sim_ms * 1e-3) / 1e9
     return {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
-            "frac": round(achieved / peak, 4), "traffic": ncu_traffic(kernel_key("folded", 0)),
-            "kernel": kernel_key("folded", 0), "algorithmic_bytes_per_launch": bytes_,
+            "frac": round(achieved / peak, 4), "traffic": ncu_traffic(key),
+            "kernel": key, "algorithmic_bytes_per_launch": bytes_,
             "peak_source": f"{src} HBM copy bandwidth",
             "note": "algorithmic bytes = 4 B id per event + 8 B per trial"}
 
@@ -608,7 +660,8 @@ def next_record(are, torch, res, steps, warmup):
             "hbm_frac": round(hbm_bytes / (ms * 1e-3) / 1e9 / hbm, 4),
             "ylt_rel_diff_max_vs_analysis": diff,
             "what": "are_simulate_occurrences: every occurrence's marginal (8 B), each trial's "
-                    "largest occurrence loss and the YLT"}
+                    "largest occurrence loss and the YLT; rows of the marked events only, the value "
+                    "counts events x J"}
     del marg
     torch.cuda.empty_cache()
     are.are_prepare(ctx, res.layer, res.yet, 1, stream)
@@ -671,7 +724,13 @@ def portfolio_record(are, torch, prec, steps, warmup, tune=True, variants=True, 
         n = y.n_trials
         stream = torch.cuda.Stream()
         outs = [torch.empty(n, dtype=torch.float64, device="cuda") for _ in layers]
+        if not tune:
+            untuned_rows(are, ctx, layers, yet, prec, stream)
         tuned = are.are_autotune(ctx, layers, yet, prec, stream) if tune else None
+        marked = tuned if marked_choice(tuned) else None   # timed on its own below
+        if tune:
+            every = read_every_row(are, ctx, prec, tuned)
+            tuned = every if marked else tuned
         lookups = sum(y.n_events * len(L.elts) for L in all_layers)   # the whole portfolio
 
         def batched():
@@ -729,6 +788,15 @@ def portfolio_record(are, torch, prec, steps, warmup, tune=True, variants=True, 
                       "value_unit": "G event-ELT lookups/s equivalent", "gpu_launches": launches_f,
                       "what": ("per layer: FP64 folded table (one lookup per occurrence) and one "
                                "exact trial pass; batched PML/TVaR")}
+        marked_events = None
+        if marked:
+            read_every_row(are, ctx, prec, marked, on=False)
+            ms_m, launches_m, _ = timed(batched, max(1, steps // 2))
+            ms_mp, _, _ = timed(plain, max(1, steps // 2))
+            marked_events = {"ms_per_step": round(ms_m, 4), "gpu_launches": launches_m, "tuned": marked,
+                             "plain_ms_per_step": round(ms_mp, 4), "speedup_vs_plain": round(ms_mp / ms_m, 3),
+                             "value": round(lookups / (ms_m * 1e-3) / 1e9, 3),
+                             "value_unit": "G event-ELT lookups/s equivalent", "what": MARKED_WHAT}
         pml, tv = batched()
         per_layer = {i: ([float(x) for x in pml[k]], [float(x) for x in tv[k]])
                      for k, i in enumerate(mine)}
@@ -772,7 +840,8 @@ def portfolio_record(are, torch, prec, steps, warmup, tune=True, variants=True, 
                       "gpu_launches": launches_p,
                       "how": "64 x (repack + are_simulate + are_risk_measures)"},
             "speedup_vs_plain": round(ms_p / ms_b, 3),
-            "folded_variant": folded, "tuned": tuned, "kernel": portfolio_kernel_name(tuned, prec),
+            "folded_variant": folded, "marked_events": marked_events, "tuned": tuned,
+            "kernel": portfolio_kernel_name(tuned, prec),
             "gpu_launches": launches, "clocks": clocks,
             "pml_layer0": per_layer[0][0], "tvar_layer0": per_layer[0][1]}
     finally:
@@ -841,7 +910,13 @@ def precision_record(are, torch, steps, warmup, tune=True, compact=True, n_trial
             return float(np.mean([a.elapsed_time(b) for a, b in evs[warmup:]]))
 
         for p in (0, 2, 1):
+            if not tune:
+                untuned_rows(are, ctx, [layer], yet, p, stream)
             tuned = are.are_autotune(ctx, [layer], yet, p, stream) if tune else None
+            ms_marked = None
+            if marked_choice(tuned):
+                ms_marked = timed(p)
+                tuned = read_every_row(are, ctx, p, tuned)
             ms = timed(p)
             got = out.cpu().numpy()
             if p == 1:
@@ -858,6 +933,7 @@ def precision_record(are, torch, steps, warmup, tune=True, compact=True, n_trial
             rp, rt = oracle.risk_measures(full, RPS, LEVELS)
             rows[PRECISION_NAMES[p]] = {
                 "sim_ms": round(ms, 4), "tuned": tuned,
+                "marked_events_sim_ms": round(ms_marked, 4) if ms_marked else None,
                 "kernel": kernel_key(p, len(L.elts), tuned, layer_rows(are, ctx, layer, yet, p, tuned),
                                      ragged=True),
                 "value": round(y.n_events * len(L.elts) / (ms * 1e-3) / 1e9, 3),
@@ -994,7 +1070,9 @@ def serving_record(are, torch, prec, rates, seconds_per_rate, min_requests=200,
             rows[str(int(rate))] = row
         return {"workload": wl.name, "request_trials": "log-uniform 1e4..1e6 (YET prefix)",
                 "request_elts": "1..16 of the pool", "measures": "PML 100/250, TVaR 99",
-                "precision": PRECISION_NAMES[prec], "rates": rows}
+                "precision": PRECISION_NAMES[prec], "rates": rows,
+                "rows_read": "the marked events' where a layer's marks pay, else every occurrence's; "
+                             "g_lookups_s counts events x J"}
     finally:
         are.are_destroy(ctx)
 
@@ -1078,12 +1156,27 @@ def main():
     if not args.no_tune:
         for p in paths:
             tuned[PRECISION_NAMES[p]] = are.are_autotune(ctx, [res.layer], res.yet, p, stream)
-    results = {}
+    else:
+        for p in paths:
+            untuned_rows(are, ctx, [res.layer], res.yet, p, stream)
+    # the headline and its variants read every occurrence's row; the form over
+    # the marked events is timed on its own
+    marked = {p: tuned[PRECISION_NAMES[p]] for p in paths if marked_choice(tuned.get(PRECISION_NAMES[p]))}
+    for p in marked:
+        tuned[PRECISION_NAMES[p]] = read_every_row(are, ctx, p, marked[p])
+    results, marked_results = {}, {}
     for p in paths:
         r = time_path(are, torch, res, p, args.steps, args.warmup, stream, ylt, gather, world)
         r["ms"] = max_over_ranks(r["ms"], world, torch)
         r["sim_ms"] = max_over_ranks(r["sim_ms"], world, torch)
         results[p] = r
+    for p in marked:
+        read_every_row(are, ctx, p, marked[p], on=False)
+        r = time_path(are, torch, res, p, args.steps, args.warmup, stream, ylt, gather, world)
+        r["ms"] = max_over_ranks(r["ms"], world, torch)
+        r["sim_ms"] = max_over_ranks(r["sim_ms"], world, torch)
+        marked_results[p] = r
+        read_every_row(are, ctx, p, marked[p])
     folded = None
     if not args.no_variants:
         folded = time_folded(are, torch, res, args.steps, args.warmup, stream, ylt, gather, world)
@@ -1138,6 +1231,18 @@ def main():
                                                   rows[p]),
                              "pml": r["pml"], "tvar": r["tvar"], "clocks": r["clocks"]}
         for p, r in results.items() if p != prec}
+    if marked_results:
+        line["marked_events"] = {"what": MARKED_WHAT}
+        for p, r in marked_results.items():
+            ms_m = r["ms"] / args.steps
+            line["marked_events"][PRECISION_NAMES[p]] = {
+                "ms_per_step": round(ms_m, 4), "sim_ms": round(r["sim_ms"], 4),
+                "value": round(lookups / (ms_m * 1e-3) / 1e9, 3),
+                "value_unit": "G event-ELT lookups/s equivalent (events x J / step time)",
+                "roofline": folded_roofline(y.n_events, y.n_trials, r["sim_ms"],
+                                            kernel_key(p, J, marked[p], rows[p])),
+                "tuned": marked[p], "pml": r["pml"], "tvar": r["tvar"], "clocks": r["clocks"],
+                "gpu_launches": r["launches"]}
     if folded is not None:
         ms_f = folded["ms"] / args.steps
         line["variants"]["fp64_folded"] = {
