@@ -340,13 +340,44 @@ void fill_terms(const Layer &L, TermsF32 &t32, TermsF64 &t64)
     t32.occ_l = (float)L.terms.occ_lim;
 }
 
-// The layer's marks beside its FP32 or FP64 rows, sized for `catalog`.
-MarkMap &size_marks(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32)
+int64_t layer_entries(const Layer &L)
+{
+    ARE_CHECK(L.entries < (1LL << 32), ARE_EINVAL, "a layer's ELTs hold 2^32 or more entries");
+    return L.entries;
+}
+
+// Words per packed row of the layer over a catalog of `catalog` events (0:
+// the dense FP32 row), from its ELT entries per catalog event.
+int row_words(const Layer &L, int32_t catalog, bool fp32)
+{
+    const double tpe = catalog > 0 ? (double)layer_entries(L) / (double)catalog : 0.0;
+    return packed_row_words((int)L.elts.size(), tpe, fp32);
+}
+
+// Whether some call may look the layer's occurrences up in marks: what
+// use_marks and occ_uses_marks ask of the layer and the catalog alone (the
+// largest share that either takes), whatever the YET's trials.
+constexpr double kMostMarked32 = 0.8, kMostMarked64 = 0.85;
+double layer_share(const are_ctx *ctx, const Layer &L, int32_t catalog);
+bool may_use_marks(const are_ctx *ctx, const Layer &L, int32_t catalog, bool fp32)
+{
+    if (mark_shape(catalog).words == 0 || (fp32 && !(L.bound < 1e37))) return false;
+    return layer_share(ctx, L, catalog) <= (fp32 ? kMostMarked32 : kMostMarked64);
+}
+
+// The layer's marks beside its FP32 or FP64 register rows, sized for
+// `catalog`; none where no call uses them.  They are made with the rows, also
+// for a call that reads every row (a YET of short trials, say): rows that are
+// there are only read from then on, so that a later call that wants marks
+// writes nothing that another stream may be reading.  They cost the build 0 to
+// 3 us over 1M events and 8 over 2M, where they fold, and at most 166 KB.
+MarkMap size_marks(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, const ScatterArgs &a)
 {
     Marks &m = fp32 ? L.m32 : L.m64;
-    if (m.map.d && m.catalog != catalog) free_marks(ctx, m);
-    if (!m.map.d) {
-        const MarkMap shape = mark_shape(catalog);
+    const MarkMap shape =
+        elts_bucketed(a) && may_use_marks(ctx, L, catalog, fp32) ? mark_shape(catalog) : MarkMap{};
+    if (m.map.d && (m.catalog != catalog || !shape.words)) free_marks(ctx, m);
+    if (!m.map.d && shape.words) {
         uint32_t *d = (uint32_t *)dalloc(ctx, sizeof(uint32_t) * (size_t)shape.words);
         ++L.generation;
         m.map = shape;
@@ -356,9 +387,9 @@ MarkMap &size_marks(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32)
     return m.map;
 }
 
-// Build (or rebuild) the layer's table for `catalog` in fp32 or fp64; with
-// `marked` (fp32) its marks too.
-Table &build_table(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, cudaStream_t s, bool marked = false)
+// Build (or rebuild) the layer's table for `catalog` in fp32 or fp64, and the
+// marks where its rows are register rows (dense FP32).
+Table &build_table(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, cudaStream_t s)
 {
     Table &t = fp32 ? L.t32 : L.t64;
     const int jp = table_jp((int)L.elts.size(), fp32);
@@ -367,7 +398,7 @@ Table &build_table(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, cudaStrea
     TermsF32 t32;
     TermsF64 t64;
     fill_terms(L, t32, t64);
-    const MarkMap m = marked ? size_marks(ctx, L, catalog, true) : MarkMap{};
+    const MarkMap m = fp32 && !row_words(L, catalog, true) ? size_marks(ctx, L, catalog, true, a) : MarkMap{};
     if (fp32 && elts_bucketed(a)) {
         ctx->launches += launch_tile_rows(a, catalog, true, false, jp, t.d, nullptr, m, t32, t64, s);
         return t;
@@ -410,23 +441,9 @@ void size_packed(are_ctx *ctx, Layer &L, Packed &p, int32_t catalog, int rw, siz
     }
 }
 
-int64_t layer_entries(const Layer &L)
-{
-    ARE_CHECK(L.entries < (1LL << 32), ARE_EINVAL, "a layer's ELTs hold 2^32 or more entries");
-    return L.entries;
-}
-
-// Words per packed row of the layer over a catalog of `catalog` events (0:
-// the dense FP32 row), from its ELT entries per catalog event.
-int row_words(const Layer &L, int32_t catalog, bool fp32)
-{
-    const double tpe = catalog > 0 ? (double)layer_entries(L) / (double)catalog : 0.0;
-    return packed_row_words((int)L.elts.size(), tpe, fp32);
-}
-
-// The packed rows of the layer (and, with `marked`, their marks), built from
-// its ELT entries with no dense table: what the register-rows kernels read.
-void build_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, int words, bool marked, cudaStream_t s)
+// The packed rows of the layer and their marks, built from its ELT entries
+// with no dense table: what the register-rows kernels read.
+void build_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, int words, cudaStream_t s)
 {
     Packed &p = fp32 ? L.p32 : L.p64;
     const size_t elem = fp32 ? sizeof(float) : sizeof(double);
@@ -435,7 +452,7 @@ void build_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, int words,
     TermsF32 t32;
     TermsF64 t64;
     fill_terms(L, t32, t64);
-    const MarkMap m = marked ? size_marks(ctx, L, catalog, fp32) : MarkMap{};
+    const MarkMap m = size_marks(ctx, L, catalog, fp32, a);
     if (elts_bucketed(a)) {
         ctx->launches += launch_tile_rows(a, catalog, fp32, true, words, p.rows(), p.ovf(), m, t32, t64, s);
         return;
@@ -459,16 +476,14 @@ void ensure_aux(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, int kernel, 
 }
 
 // The packed rows a register-rows analysis (kernel 2) of the layer reads,
-// built if missing (or always, with rebuild, or where `marked` asks for marks
-// that are missing); false where it reads the dense FP32 table instead.
-bool ensure_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, bool marked, cudaStream_t s, bool rebuild)
+// built if missing (or always, with rebuild); false where it reads the dense
+// FP32 table instead.
+bool ensure_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, cudaStream_t s, bool rebuild)
 {
     const int w = row_words(L, catalog, fp32);
     if (!w) return false;
     const Packed &p = fp32 ? L.p32 : L.p64;
-    const Marks &m = fp32 ? L.m32 : L.m64;
-    if (rebuild || !p.d || p.catalog != catalog || p.rw != w || (marked && (!m.map.d || m.catalog != catalog)))
-        build_packed(ctx, L, catalog, fp32, w, marked, s);
+    if (rebuild || !p.d || p.catalog != catalog || p.rw != w) build_packed(ctx, L, catalog, fp32, w, s);
     return true;
 }
 
@@ -552,7 +567,7 @@ bool use_marks(are_precision p, const Yet &y, double bound, double share)
     switch (p) {
     case ARE_FP32_KAHAN: return mean >= 80.0 && share <= 0.5;
     case ARE_FP32_FP64AGG: return share <= 0.75;
-    default: return mean >= 50.0 && share <= 0.85;
+    default: return mean >= 50.0 && share <= kMostMarked64;
     }
 }
 
@@ -580,18 +595,23 @@ bool occ_uses_marks(are_ctx *ctx, const Layer &L, const Yet &y, bool fp32)
 {
     if (y.catalog <= 0 || mark_shape(y.catalog).words == 0) return false;
     if (fp32 && !(L.bound < 1e37)) return false;
-    return (double)y.n_events >= 60.0 * (double)y.n_trials && layer_share(ctx, L, y.catalog) <= 0.8;
+    return (double)y.n_events >= 60.0 * (double)y.n_trials && layer_share(ctx, L, y.catalog) <= kMostMarked32;
 }
 
 // The rows of a register-rows analysis -- packed, or the dense FP32 table --
-// and, with `marked`, their marks.
-void ensure_rows(are_ctx *ctx, Layer &L, const Yet &y, bool fp32, bool marked, cudaStream_t s, bool rebuild)
+// and their marks.
+void ensure_rows(are_ctx *ctx, Layer &L, const Yet &y, bool fp32, cudaStream_t s, bool rebuild)
 {
     const int32_t catalog = y.catalog;
-    if (ensure_packed(ctx, L, catalog, fp32, marked, s, rebuild)) return;
-    if (rebuild || !L.t32.d || L.t32.catalog != catalog ||
-        (marked && (!L.m32.map.d || L.m32.catalog != catalog)))
-        build_table(ctx, L, catalog, true, s, marked);
+    if (ensure_packed(ctx, L, catalog, fp32, s, rebuild)) return;
+    if (rebuild || !L.t32.d || L.t32.catalog != catalog) build_table(ctx, L, catalog, true, s);
+}
+
+// The marks of the layer's register rows over `catalog`; d null: none.
+MarkMap marks_of(const Layer &L, int32_t catalog, bool fp32)
+{
+    const Marks &m = fp32 ? L.m32 : L.m64;
+    return m.catalog == catalog ? m.map : MarkMap{};
 }
 
 // The tables that a kernel choice reads for a layer in the direct layout,
@@ -602,7 +622,7 @@ void ensure_direct(are_ctx *ctx, Layer &L, const Yet &y, are_precision p, const 
     const bool fp32 = p != ARE_FP64;
     const int32_t catalog = y.catalog;
     if (te.kernel == 2) {   // a dense table only where the rows are dense
-        ensure_rows(ctx, L, y, fp32, te.cfg.rows_in_flight == 0 && uses_marks(ctx, L, y, p), s, rebuild);
+        ensure_rows(ctx, L, y, fp32, s, rebuild);
         return;
     }
     const Table &t = fp32 ? L.t32 : L.t64;
@@ -730,16 +750,16 @@ int run_single(are_ctx *ctx, const Layer &L, const Yet &y, int64_t trial_begin, 
     TermsF64 t64;
     fill_terms(L, t32, t64);
     a.n_elts = (int32_t)L.elts.size();
-    const Marks &m = fp32 ? L.m32 : L.m64;   // built where this choice uses them (ensure_rows)
-    const bool marked = !compact && te.kernel == 2 && te.cfg.rows_in_flight == 0 && m.map.d &&
-                        m.catalog == y.catalog && uses_marks(ctx, L, y, precision);
+    const MarkMap marks = marks_of(L, y.catalog, fp32);
+    const bool marked = !compact && te.kernel == 2 && te.cfg.rows_in_flight == 0 && marks.d &&
+                        uses_marks(ctx, L, y, precision);
     if (fp32 && !compact && te.kernel == 2 && L.p32.d && L.p32.catalog == y.catalog &&
         L.p32.rw == row_words(L, y.catalog, true)) {
         a.table = L.p32.rows();   // register rows over the packed FP32 rows
         a.table2 = L.p32.ovf();
         a.kernel = 5;
         if (marked)
-            return launch_marked32(a, m.map, precision, true, L.p32.rw, t32, fixed_scale(L.bound), ctx->num_sms, s);
+            return launch_marked32(a, marks, precision, true, L.p32.rw, t32, fixed_scale(L.bound), ctx->num_sms, s);
         return launch_simulate(a, precision, L.p32.rw, &t32, &t64, ctx->num_sms, s);
     }
     if (compact) {   // the staged kernel, through the row index
@@ -752,7 +772,7 @@ int run_single(are_ctx *ctx, const Layer &L, const Yet &y, int64_t trial_begin, 
         if (te.kernel == 2 && L.p64.d && L.p64.catalog == y.catalog) {   // packed FP64 rows
             a.table = L.p64.rows();
             a.table2 = L.p64.ovf();
-            if (marked) return launch_marked64(a, m.map, L.p64.rw, t64, fixed_scale(L.bound), ctx->num_sms, s);
+            if (marked) return launch_marked64(a, marks, L.p64.rw, t64, fixed_scale(L.bound), ctx->num_sms, s);
             return launch_rows64(a, L.p64.rw, t64, fixed_scale(L.bound), ctx->num_sms, s);
         }
         if (te.kernel == 3 && L.t32u.d && L.t32u.catalog == y.catalog) {   // the FP32 screen
@@ -762,7 +782,7 @@ int run_single(are_ctx *ctx, const Layer &L, const Yet &y, int64_t trial_begin, 
         }
         return launch_staged64(a, t.jp, t64, ctx->num_sms, s);   // (or an aux table not built)
     }
-    if (marked) return launch_marked32(a, m.map, precision, false, t.jp, t32, fixed_scale(L.bound), ctx->num_sms, s);
+    if (marked) return launch_marked32(a, marks, precision, false, t.jp, t32, fixed_scale(L.bound), ctx->num_sms, s);
     return launch_simulate(a, precision, t.jp, &t32, &t64, ctx->num_sms, s);
 }
 
@@ -1738,10 +1758,9 @@ are_status are_simulate_occurrences(are_ctx *ctx, int32_t layer, int32_t yet, in
         Table &t = fp32 ? L.t32 : L.t64;
         // the rows of the register-rows form (the direct layout, whatever the
         // layer's analysis layout): packed where the layer's row size calls for them
-        const bool marked = occ_uses_marks(ctx, L, y, fp32);
-        ensure_rows(ctx, L, y, fp32, marked, cs.s, false);
+        ensure_rows(ctx, L, y, fp32, cs.s, false);
         const bool packed = row_words(L, y.catalog, fp32) != 0;
-        const MarkMap marks = marked ? (fp32 ? L.m32 : L.m64).map : MarkMap{};
+        const MarkMap marks = occ_uses_marks(ctx, L, y, fp32) ? marks_of(L, y.catalog, fp32) : MarkMap{};
         SimArgs a{};
         a.ids = y.d_ids;
         a.off = y.d_off;

@@ -1,0 +1,74 @@
+"""A layer's tables over a context's life: what a call builds, leaves alone,
+and does without where memory is short."""
+import math
+
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+INF = math.inf
+CATALOG = 30_000
+
+
+@pytest.fixture(scope="module")
+def are():
+    import torch
+    assert torch.cuda.is_available()
+    import paper_1308_2066_gb300 as are
+    are.lib()
+    return are
+
+
+def elts_of(J, nnz=400, seed=0):
+    g = np.random.Generator(np.random.PCG64(900 + J + seed))
+    return [W.ELT(g.permutation(CATALOG)[:nnz].astype(np.int32), g.lognormal(11, 1.5, nnz)) for _ in range(J)]
+
+
+def load_elts(are, ctx, elts):
+    return [are.are_load_elt(ctx, e.ids, e.losses) for e in elts]
+
+
+def yet_of(are, ctx, n, k, seed):
+    ids = np.random.Generator(np.random.PCG64(seed)).integers(0, CATALOG, n * k).astype(np.int32)
+    return are.are_load_yet(ctx, CATALOG, n, None, k, ids)
+
+
+def simulate(are, ctx, layer, y, n, p):
+    import torch
+    out = torch.full((n,), -1.0, dtype=torch.float64, device="cuda")
+    are.are_simulate(ctx, layer, y, 0, n, p, out)
+    return out.cpu().numpy()
+
+
+# dense 32-byte rows and packed rows; FP32 with either sum reads the same rows
+@pytest.mark.parametrize("J", [6, 12])
+def test_a_table_that_is_there_is_only_read(are, J):
+    """Once a layer's table is built, no analysis writes it again, whatever
+    precision, trial length or call comes next: each is one kernel."""
+    import torch
+    n, k = 300, 200
+    ctx, fresh = are.are_create(0), are.are_create(0)
+    try:
+        elts = elts_of(J)
+        layer = are.are_define_layer(ctx, load_elts(are, ctx, elts), 3e4, 2e6, 0.0, INF)
+        short, long_ = yet_of(are, ctx, n, 20, 1), yet_of(are, ctx, n, k, 2)
+        other = are.are_define_layer(fresh, load_elts(are, fresh, elts), 3e4, 2e6, 0.0, INF)
+        other_long = yet_of(are, fresh, n, k, 2)
+        marg = torch.zeros(n * k, dtype=torch.float64, device="cuda")
+        for first, later in ((1, (1, 2)), (0, (0,))):
+            are.are_prepare(ctx, layer, short, first)
+            simulate(are, ctx, layer, short, n, first)
+            for p in later:
+                for call in (lambda: simulate(are, ctx, layer, short, n, p),
+                             lambda: simulate(are, ctx, layer, long_, n, p),
+                             lambda: are.are_simulate_occurrences(ctx, layer, long_, 0, n, p, marg)):
+                    before = are.are_launch_count(ctx)
+                    call()
+                    assert are.are_launch_count(ctx) == before + 1
+                np.testing.assert_array_equal(simulate(are, ctx, layer, long_, n, p),
+                                              simulate(are, fresh, other, other_long, n, p))
+    finally:
+        are.are_destroy(ctx)
+        are.are_destroy(fresh)
