@@ -366,11 +366,12 @@ bool may_use_marks(const are_ctx *ctx, const Layer &L, int32_t catalog, bool fp3
 }
 
 // The layer's marks beside its FP32 or FP64 register rows, sized for
-// `catalog`; none where no call uses them.  They are made with the rows, also
-// for a call that reads every row (a YET of short trials, say): rows that are
-// there are only read from then on, so that a later call that wants marks
-// writes nothing that another stream may be reading.  They cost the build 0 to
-// 3 us over 1M events and 8 over 2M, where they fold, and at most 166 KB.
+// `catalog`; none where no call uses them, or no memory is left for them (then
+// every row is read).  They are made with the rows, also for a call that reads
+// every row (a YET of short trials, say): rows that are there are only read
+// from then on, so that a later call that wants marks writes nothing that
+// another stream may be reading.  They cost the build 0 to 3 us over 1M events
+// and 8 over 2M, where they fold, and at most 166 KB.
 MarkMap size_marks(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, const ScatterArgs &a)
 {
     Marks &m = fp32 ? L.m32 : L.m64;
@@ -378,7 +379,13 @@ MarkMap size_marks(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, const Sca
         elts_bucketed(a) && may_use_marks(ctx, L, catalog, fp32) ? mark_shape(catalog) : MarkMap{};
     if (m.map.d && (m.catalog != catalog || !shape.words)) free_marks(ctx, m);
     if (!m.map.d && shape.words) {
-        uint32_t *d = (uint32_t *)dalloc(ctx, sizeof(uint32_t) * (size_t)shape.words);
+        uint32_t *d;
+        try {
+            d = (uint32_t *)dalloc(ctx, sizeof(uint32_t) * (size_t)shape.words);
+        } catch (const Error &e) {
+            if (e.code != ARE_ENOMEM) throw;
+            return m.map;
+        }
         ++L.generation;
         m.map = shape;
         m.map.d = d;
@@ -394,17 +401,24 @@ Table &build_table(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, cudaStrea
     Table &t = fp32 ? L.t32 : L.t64;
     const int jp = table_jp((int)L.elts.size(), fp32);
     const ScatterArgs a = scatter_args(ctx, L, catalog, jp);
+    const bool rows = fp32 && !row_words(L, catalog, true);   // register rows
     size_table(ctx, L, t, catalog, jp, fp32 ? 4 : 8);
-    TermsF32 t32;
-    TermsF64 t64;
-    fill_terms(L, t32, t64);
-    const MarkMap m = fp32 && !row_words(L, catalog, true) ? size_marks(ctx, L, catalog, true, a) : MarkMap{};
-    if (fp32 && elts_bucketed(a)) {
-        ctx->launches += launch_tile_rows(a, catalog, true, false, jp, t.d, nullptr, m, t32, t64, s);
-        return t;
+    try {
+        TermsF32 t32;
+        TermsF64 t64;
+        fill_terms(L, t32, t64);
+        const MarkMap m = rows ? size_marks(ctx, L, catalog, true, a) : MarkMap{};
+        if (fp32 && elts_bucketed(a)) {
+            ctx->launches += launch_tile_rows(a, catalog, true, false, jp, t.d, nullptr, m, t32, t64, s);
+        } else {
+            ARE_CUDA_TRY(cudaMemsetAsync(t.d, 0, t.bytes, s));
+            ctx->launches += launch_scatter_table(t.d, fp32, a, s);
+        }
+    } catch (...) {   // what is kept is built
+        free_table(ctx, t);
+        if (rows) free_marks(ctx, L.m32);
+        throw;
     }
-    ARE_CUDA_TRY(cudaMemsetAsync(t.d, 0, t.bytes, s));
-    ctx->launches += launch_scatter_table(t.d, fp32, a, s);
     return t;
 }
 
@@ -449,21 +463,24 @@ void build_packed(are_ctx *ctx, Layer &L, int32_t catalog, bool fp32, int words,
     const size_t elem = fp32 ? sizeof(float) : sizeof(double);
     const ScatterArgs a = scatter_args(ctx, L, catalog, table_jp((int)L.elts.size(), fp32));
     size_packed(ctx, L, p, catalog, words, words * elem, elem * (size_t)layer_entries(L));
-    TermsF32 t32;
-    TermsF64 t64;
-    fill_terms(L, t32, t64);
-    const MarkMap m = size_marks(ctx, L, catalog, fp32, a);
-    if (elts_bucketed(a)) {
-        ctx->launches += launch_tile_rows(a, catalog, fp32, true, words, p.rows(), p.ovf(), m, t32, t64, s);
-        return;
+    try {
+        TermsF32 t32;
+        TermsF64 t64;
+        fill_terms(L, t32, t64);
+        const MarkMap m = size_marks(ctx, L, catalog, fp32, a);
+        if (elts_bucketed(a))
+            ctx->launches += launch_tile_rows(a, catalog, fp32, true, words, p.rows(), p.ovf(), m, t32, t64, s);
+        else if (fp32)   // ids past the buckets' range (and past any marks)
+            ctx->launches += launch_pack32_direct(a, catalog, words, static_cast<uint32_t *>(p.rows()),
+                                                  static_cast<float *>(p.ovf()), p.used(), s);
+        else
+            ctx->launches += launch_pack64_direct(a, catalog, words, static_cast<unsigned long long *>(p.rows()),
+                                                  static_cast<double *>(p.ovf()), p.used(), s);
+    } catch (...) {   // what is kept is built
+        free_packed(ctx, p);
+        free_marks(ctx, fp32 ? L.m32 : L.m64);
+        throw;
     }
-    // ids past the buckets' range (and past any marks)
-    if (fp32)
-        ctx->launches += launch_pack32_direct(a, catalog, words, static_cast<uint32_t *>(p.rows()),
-                                              static_cast<float *>(p.ovf()), p.used(), s);
-    else
-        ctx->launches += launch_pack64_direct(a, catalog, words, static_cast<unsigned long long *>(p.rows()),
-                                              static_cast<double *>(p.ovf()), p.used(), s);
 }
 
 // The table beside a layer's dense FP64 table that a kernel choice reads:

@@ -72,3 +72,34 @@ def test_a_table_that_is_there_is_only_read(are, J):
     finally:
         are.are_destroy(ctx)
         are.are_destroy(fresh)
+
+
+@pytest.mark.parametrize("J,p", [(6, 1), (12, 2), (12, 0)])
+def test_rows_without_room_for_their_marks(are, J, p):
+    """A memory budget that holds a layer's rows but not their marks: the
+    analysis reads every row instead, and the losses are the same."""
+    n, k = 200, 150
+    elts = elts_of(J)
+
+    def run(room):
+        ctx = are.are_create(0, room)
+        try:
+            y = yet_of(are, ctx, n, k, 3)
+            layer = are.are_define_layer(ctx, load_elts(are, ctx, elts), 3e4, 2e6, 0.0, INF)
+            loaded = are.are_memory_used(ctx)
+            got = simulate(are, ctx, layer, y, n, p)
+            np.testing.assert_array_equal(simulate(are, ctx, layer, y, n, p), got)
+            return got, loaded, are.are_memory_used(ctx)
+        finally:
+            are.are_destroy(ctx)
+
+    want, loaded, used = run(0)
+    assert (want > 0).mean() > 0.2
+    marks = (CATALOG + 127) // 128 * 16
+    assert used - loaded >= CATALOG * 32 + marks
+    got, _, held = run(used - marks // 2)
+    assert held == used - marks
+    if p == 2:      # the sums over every row round each addition
+        np.testing.assert_allclose(got, want, rtol=k * 2.0 ** -52, atol=0)
+    else:
+        np.testing.assert_array_equal(got, want)
