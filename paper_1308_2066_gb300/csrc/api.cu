@@ -1905,13 +1905,13 @@ are_status are_simulate_portfolio(are_ctx *ctx, const int32_t *layers, int32_t n
         check_multi_args(ctx, layers, n_layers, y, trial_begin, n_trials, ylts);
         CallStream cs(ctx, stream);
         const bool fp32 = precision != ARE_FP64;
-        ensure_tables(ctx, layers, n_layers, y, precision, cs.s,
-                      tuned(ctx, precision, y, max_width(ctx, layers, n_layers, fp32), n_layers > 1));
+        // one choice for the tables, the plan and its launches, also of a single layer
+        const TuneEntry te = tuned(ctx, precision, y, max_width(ctx, layers, n_layers, fp32), true);
+        ensure_tables(ctx, layers, n_layers, y, precision, cs.s, te);
         const std::vector<int32_t> lv(layers, layers + n_layers);
         const std::vector<double *> yv(ylts, ylts + n_layers);
         std::vector<uint64_t> gens;
         for (int32_t h : lv) gens.push_back(ctx->layers.at(h).generation);
-        const TuneEntry te = tuned(ctx, precision, y, max_width(ctx, layers, n_layers, fp32), true);
 
         Plan *plan = nullptr;
         for (Plan &p : ctx->plans)

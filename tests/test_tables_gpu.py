@@ -1,5 +1,6 @@
 """A layer's tables over a context's life: what a call builds, leaves alone,
 and does without where memory is short."""
+import json
 import math
 
 import numpy as np
@@ -103,3 +104,34 @@ def test_rows_without_room_for_their_marks(are, J, p):
         np.testing.assert_allclose(got, want, rtol=k * 2.0 ** -52, atol=0)
     else:
         np.testing.assert_array_equal(got, want)
+
+
+@pytest.mark.parametrize("p,kernel", [(1, 0), (1, 1), (2, 0), (2, 2), (0, 1), (0, 3)])
+def test_a_portfolio_of_one_layer_under_a_tuned_choice(are, tmp_path, p, kernel):
+    """A tuning entry for several layers also decides for a portfolio of one:
+    its tables are the ones that the kernel reads, and the losses are those of
+    are_simulate under the same choice."""
+    import torch
+    n, k, J = 200, 150, 12
+    elts = elts_of(J)
+    got = {}
+    for kind in ("multi", "single"):
+        ctx = are.are_create(0)
+        try:
+            y = yet_of(are, ctx, n, k, 4)
+            layer = are.are_define_layer(ctx, load_elts(are, ctx, elts), 3e4, 2e6, 0.0, INF)
+            path = tmp_path / "tune.jsonl"
+            path.write_text("".join(json.dumps(
+                {"key": f"p{p}_fixed_jp{jp}_ev256_{kind}", "kernel": kernel, "rows_in_flight": 1,
+                 "trials_per_item": 8, "blocks_per_sm": 0, "ms": 1.0}) + "\n" for jp in (12, 16)))
+            are.are_tune_load(ctx, str(path))
+            if kind == "single":
+                got[kind] = simulate(are, ctx, layer, y, n, p)
+            else:
+                out = torch.full((n,), -1.0, dtype=torch.float64, device="cuda")
+                are.are_simulate_portfolio(ctx, [layer], y, 0, n, p, [out])
+                got[kind] = out.cpu().numpy()
+        finally:
+            are.are_destroy(ctx)
+    assert (got["multi"] > 0).mean() > 0.2
+    np.testing.assert_array_equal(got["multi"], got["single"])
