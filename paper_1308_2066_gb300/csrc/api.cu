@@ -654,12 +654,13 @@ void ensure_tables(are_ctx *ctx, Layer &L, const Yet &y, are_precision precision
 {
     const bool fp32 = precision != ARE_FP64;
     const int32_t catalog = y.catalog;
-    if (fp32 && L.layout == ARE_LAYOUT_COMPACT) {
+    const TuneEntry te = tuned(ctx, precision, y, table_jp((int)L.elts.size(), fp32), false);
+    // (the persistent kernel reads the dense table in either layout)
+    if (fp32 && L.layout == ARE_LAYOUT_COMPACT && te.kernel != 0) {
         if (rebuild || !L.comp.d || L.comp.catalog != catalog) build_compact(ctx, L, catalog, s);
         return;
     }
-    const int jp = table_jp((int)L.elts.size(), fp32);
-    ensure_direct(ctx, L, y, precision, tuned(ctx, precision, y, jp, false), s, rebuild);
+    ensure_direct(ctx, L, y, precision, te, s, rebuild);
 }
 
 Layer &layer_of(are_ctx *ctx, int32_t h)

@@ -135,3 +135,28 @@ def test_a_portfolio_of_one_layer_under_a_tuned_choice(are, tmp_path, p, kernel)
             are.are_destroy(ctx)
     assert (got["multi"] > 0).mean() > 0.2
     np.testing.assert_array_equal(got["multi"], got["single"])
+
+
+@pytest.mark.parametrize("p", [1, 2])
+def test_a_compact_layer_under_the_tuned_persistent_kernel(are, tmp_path, p):
+    """The persistent kernel reads the dense table, which is then built for a
+    layer of the compact layout too, and again for another catalog."""
+    n, k, J = 200, 150, 12
+    ctx = are.are_create(0)
+    try:
+        layer = are.are_define_layer(ctx, load_elts(are, ctx, elts_of(J)), 3e4, 2e6, 0.0, INF)
+        path = tmp_path / "tune.jsonl"
+        path.write_text(json.dumps({"key": f"p{p}_fixed_jp16_ev256_single", "kernel": 0, "rows_in_flight": 1,
+                                    "trials_per_item": 8, "blocks_per_sm": 0, "ms": 1.0}) + "\n")
+        are.are_tune_load(ctx, str(path))
+        for catalog in (CATALOG, CATALOG + 5000):
+            ids = np.random.Generator(np.random.PCG64(5)).integers(0, catalog, n * k).astype(np.int32)
+            y = are.are_load_yet(ctx, catalog, n, None, k, ids)
+            out = {}
+            for layout in (are.ARE_LAYOUT_COMPACT, are.ARE_LAYOUT_DIRECT):
+                are.are_set_table_layout(ctx, layer, layout)
+                out[layout] = simulate(are, ctx, layer, y, n, p)
+            assert (out[are.ARE_LAYOUT_DIRECT] > 0).mean() > 0.2
+            np.testing.assert_array_equal(out[are.ARE_LAYOUT_COMPACT], out[are.ARE_LAYOUT_DIRECT])
+    finally:
+        are.are_destroy(ctx)
