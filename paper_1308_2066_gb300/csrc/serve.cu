@@ -419,17 +419,17 @@ void scheduler(Server *SP)
                     sl.tab_bytes = S.cfg.folded ? folded_block_bytes(S.y->catalog)
                                                 : table_bytes(sl, S.y->catalog, r.entries);
                     sl.marks = MarkMap{};
+                    sl.ylt_bytes = sizeof(double) * (size_t)r.n_trials;
                     // marks for the kernels that take them (rows of up to 16
-                    // words), unless the arena could never hold them too
+                    // words), unless the arena, empty, could not hold the two
+                    // blocks as it rounds them
                     const MarkMap shape = mark_shape(S.y->catalog);
                     const size_t mark_bytes = sizeof(uint32_t) * (size_t)shape.words;
-                    const bool marked = r.marked && (sl.pw || sl.jp <= 16) &&
-                                        sl.tab_bytes + mark_bytes + up(sizeof(double) * (size_t)r.n_trials) <=
-                                            S.cfg.arena_bytes;
+                    const bool marked = r.marked && !S.cfg.folded && (sl.pw || sl.jp <= 16) &&
+                                        up(sl.tab_bytes + mark_bytes) + up(sl.ylt_bytes) <= S.cfg.arena_bytes;
                     const size_t marks_at = sl.tab_bytes;
                     if (marked) sl.tab_bytes += mark_bytes;
                     sl.own = (sl.large || marked) && !S.cfg.folded;
-                    sl.ylt_bytes = sizeof(double) * (size_t)r.n_trials;
                     size_t a = 0, b = 0;
                     if (!S.arena.take(sl.tab_bytes, a)) break;
                     if (!S.arena.take(sl.ylt_bytes, b)) {
