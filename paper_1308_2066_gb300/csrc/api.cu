@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <tuple>
 #include <unordered_map>
 
@@ -159,7 +160,7 @@ void dfree(are_ctx *ctx, void *p, size_t bytes)
 
 // The context's pinned host scratch for the length of a call (under the
 // context's lock), kept between calls up to kHostScratchKept.
-constexpr size_t kHostScratchKept = 64u << 20;
+constexpr size_t kHostScratchFirst = 1u << 20, kHostScratchKept = 64u << 20;
 constexpr size_t kIdsSeenKept = (8u << 20) / sizeof(uint64_t);
 class HostScratch {
   public:
@@ -170,12 +171,17 @@ class HostScratch {
     }
     HostScratch(const HostScratch &) = delete;
     HostScratch &operator=(const HostScratch &) = delete;
+    // nullptr: not to be had
     void *get(size_t bytes)
     {
         if (bytes > ctx->h_scratch_bytes) {
             const size_t size = std::max(bytes, std::min(2 * ctx->h_scratch_bytes, kHostScratchKept));
             release();
-            ARE_CUDA_TRY(cudaMallocHost(&ctx->h_scratch, size));
+            if (cudaMallocHost(&ctx->h_scratch, size) != cudaSuccess) {
+                cudaGetLastError();
+                ctx->h_scratch = nullptr;
+                return nullptr;
+            }
             ctx->h_scratch_bytes = size;
         }
         return ctx->h_scratch;
@@ -1008,6 +1014,7 @@ are_status are_create(are_ctx **out, int device, size_t mem_budget_bytes)
         ARE_CUDA_TRY(cudaMalloc(&ctx->d_flag, sizeof(int)));
         ARE_CUDA_TRY(cudaMallocHost(&ctx->h_flag, sizeof(int)));
         ARE_CUDA_TRY(cudaMallocHost(&ctx->h_result, sizeof(double) * 2 * kMaxTargets));
+        HostScratch(ctx).get(kHostScratchFirst);   // (here, not in the first load)
         select_alloc(ctx->sel, 1);
     });
     if (st != ARE_OK) {
@@ -1176,102 +1183,130 @@ are_status are_load_elt(are_ctx *ctx, int32_t n_entries, const int32_t *event_id
         fence_device_inputs({event_ids, losses});
         cudaStream_t s = ctx->stream;
         const size_t n = (size_t)n_entries;
+        // The entries in pinned memory, where the host checks them and the
+        // device reads them unless they are in its own.  (A device copy of host
+        // entries to bucket them from took the budget twice, and releasing it
+        // waited for every stream.)
         HostScratch hs(ctx);
+        const bool device = n && (is_device_ptr(event_ids) || is_device_ptr(losses));
+        double *const pin_loss =
+            n ? static_cast<double *>(hs.get(n * (sizeof(double) + sizeof(int32_t)))) : nullptr;
+        int32_t *const pin_ids = pin_loss ? reinterpret_cast<int32_t *>(pin_loss + n) : nullptr;
         const int32_t *ids = event_ids;   // on the host
         const double *loss = losses;
-        if (n && (is_device_ptr(event_ids) || is_device_ptr(losses))) {
-            double *in_loss = static_cast<double *>(hs.get(n * (sizeof(double) + sizeof(int32_t))));
-            int32_t *in_ids = reinterpret_cast<int32_t *>(in_loss + n);
-            ARE_CUDA_TRY(cudaMemcpyAsync(in_loss, losses, n * sizeof(double), cudaMemcpyDefault, s));
-            ARE_CUDA_TRY(cudaMemcpyAsync(in_ids, event_ids, n * sizeof(int32_t), cudaMemcpyDefault, s));
+        if (device) {
+            ARE_CHECK(pin_loss, ARE_ENOMEM, "no pinned memory for the ELT's entries");
+            ARE_CUDA_TRY(cudaMemcpyAsync(pin_ids, event_ids, n * sizeof(int32_t), cudaMemcpyDefault, s));
+            ARE_CUDA_TRY(cudaMemcpyAsync(pin_loss, losses, n * sizeof(double), cudaMemcpyDefault, s));
             ARE_CUDA_TRY(cudaStreamSynchronize(s));
-            ids = in_ids;
-            loss = in_loss;
+            ids = pin_ids;
+            loss = pin_loss;
         }
-        constexpr uint64_t kSign = 1ull << 63, kInf = 0x7ffull << 52;
+        const bool copy = !device && pin_loss;
         int32_t max_id = -1;
-        uint64_t most = 0, least = ~0ull;   // of the losses' bit patterns (-0.0 as 0)
-        bool bad_id = false, bad_loss = false;
-        auto bits_of = [&](size_t i) {
-            uint64_t x;
-            std::memcpy(&x, loss + i, sizeof x);
-            return x == kSign ? 0 : x;
-        };
+        bool bad_id = false;
         for (size_t i = 0; i < n; ++i) {
-            bad_id |= ids[i] < 0;
-            max_id = std::max(max_id, ids[i]);
-        }
-        for (size_t i = 0; i < n; ++i) {
-            const uint64_t x = bits_of(i);
-            bad_loss |= x >= kInf;          // negative, infinite or NaN
-            most = std::max(most, x);
-            least = std::min(least, x);
+            const int32_t id = ids[i];
+            if (copy) pin_ids[i] = id;
+            bad_id |= id < 0;
+            max_id = std::max(max_id, id);
         }
         ARE_CHECK(!bad_id, ARE_EINVAL, "negative event id in ELT");
-        ARE_CHECK(!bad_loss, ARE_EINVAL, "ELT losses must be finite and >= 0");
         Elt e;
-        std::memcpy(&e.max_loss, &most, sizeof most);
-        ARE_CHECK(std::isfinite(f.fx * e.max_loss), ARE_EINVAL, "fx * loss overflows");
-        bool dup = false;
-        if (n == 0) {
-        } else if (max_id < (1 << 28)) {   // bitmap of the ids seen
-            std::vector<uint64_t> &seen = ctx->ids_seen;
-            seen.assign((size_t)max_id / 64 + 1, 0);
-            for (size_t i = 0; i < n; ++i) {
-                uint64_t &w = seen[(size_t)ids[i] >> 6];
-                const uint64_t b = 1ull << (ids[i] & 63);
-                dup |= (w & b) != 0;
-                w |= b;
-            }
-            if (seen.size() > kIdsSeenKept) std::vector<uint64_t>().swap(seen);
-        } else {
-            std::vector<int32_t> sorted(ids, ids + n);
-            std::sort(sorted.begin(), sorted.end());
-            dup = std::adjacent_find(sorted.begin(), sorted.end()) != sorted.end();
-        }
-        ARE_CHECK(!dup, ARE_EINVAL, "duplicate event id within one ELT");
         e.n = n_entries;
         e.max_id = max_id;
         e.terms = f;
-        if (n) {   // the losses by quarter octave, of up to about 4096 of them
-            e.bin0 = (int32_t)(least >> 50);
-            e.bins.assign((size_t)((int32_t)(most >> 50) - e.bin0 + 1), 0u);
-            const size_t step = n / 4096 + 1;
-            for (size_t i = 0; i < n; i += step) ++e.bins[(size_t)((int32_t)(bits_of(i) >> 50) - e.bin0)];
-            e.bin_weight = (double)n / (double)((n + step - 1) / step);
-        }
-        if (n && max_id < kMaxBucketedId) e.tiles = max_id / kEltTile + 1;
-        e.ids_bytes = sizeof(int32_t) * (n + (e.tiles ? 2 * ((size_t)e.tiles + 1) : 0));   // ids, offsets, scratch
-        char *tmp = nullptr;
-        const size_t tmp_bytes = n * (sizeof(double) + sizeof(int32_t));
-        try {
+        const int32_t tiles = pin_loss && max_id < kMaxBucketedId ? max_id / kEltTile + 1 : 0;
+        auto take = [&](int32_t t) {
+            e.tiles = t;
+            e.ids_bytes = sizeof(int32_t) * (n + (t ? (size_t)t + 1 : 0));   // ids, offsets
             e.d_ids = (int32_t *)dalloc(ctx, e.ids_bytes);
-            e.d_loss = (double *)dalloc(ctx, sizeof(double) * n);
-            if (!e.tiles) {
+            try {
+                e.d_loss = (double *)dalloc(ctx, sizeof(double) * n);
+            } catch (...) {
+                dfree(ctx, e.d_ids, e.ids_bytes);
+                e.d_ids = nullptr;
+                throw;
+            }
+            if (t) e.d_off = e.d_ids + n;
+        };
+        // Room for the entries, without that of their buckets where it is
+        // short; what is wrong with the entries is said first.
+        std::exception_ptr no_room;
+        bool dup = n > (size_t)(max_id + 1LL);
+        if (!dup) try {
+                try {
+                    take(tiles);
+                } catch (const Error &x) {
+                    if (!tiles || x.code != ARE_ENOMEM) throw;
+                    take(0);
+                }
+            } catch (...) {
+                no_room = std::current_exception();
+            }
+        const bool buckets = e.d_ids && e.tiles;   // filled by the device while the host checks the rest
+        const bool there = device && readable_here(ctx, event_ids, sizeof(int32_t)) &&
+                           readable_here(ctx, losses, sizeof(double));
+        const int32_t *const src_ids = there ? event_ids : pin_ids;
+        try {
+            if (buckets) ctx->launches += launch_bucket_offsets(src_ids, n_entries, e.tiles, e.d_off, s);
+            constexpr uint64_t kSign = 1ull << 63, kInf = 0x7ffull << 52;
+            uint64_t most = 0, least = ~0ull;   // of the losses' bit patterns (-0.0 as 0)
+            bool bad_loss = false;
+            auto bits_of = [&](size_t i) {
+                uint64_t x;
+                std::memcpy(&x, loss + i, sizeof x);
+                return x == kSign ? 0 : x;
+            };
+            for (size_t i = 0; i < n; ++i) {
+                const uint64_t x = bits_of(i);
+                if (copy) std::memcpy(pin_loss + i, loss + i, sizeof(double));
+                bad_loss |= x >= kInf;          // negative, infinite or NaN
+                most = std::max(most, x);
+                least = std::min(least, x);
+            }
+            ARE_CHECK(!bad_loss, ARE_EINVAL, "ELT losses must be finite and >= 0");
+            std::memcpy(&e.max_loss, &most, sizeof most);
+            ARE_CHECK(std::isfinite(f.fx * e.max_loss), ARE_EINVAL, "fx * loss overflows");
+            if (buckets)
+                ctx->launches += launch_bucket_fill(src_ids, there ? losses : pin_loss, n_entries, e.tiles, e.d_ids,
+                                                    e.d_loss, e.d_off, s);
+            if (n == 0 || dup) {
+            } else if (max_id < (1 << 28)) {   // bitmap of the ids seen
+                std::vector<uint64_t> &seen = ctx->ids_seen;
+                seen.assign((size_t)max_id / 64 + 1, 0);
+                for (size_t i = 0; i < n; ++i) {
+                    uint64_t &w = seen[(size_t)ids[i] >> 6];
+                    const uint64_t b = 1ull << (ids[i] & 63);
+                    dup |= (w & b) != 0;
+                    w |= b;
+                }
+                if (seen.size() > kIdsSeenKept) std::vector<uint64_t>().swap(seen);
+            } else {
+                std::vector<int32_t> sorted(ids, ids + n);
+                std::sort(sorted.begin(), sorted.end());
+                dup = std::adjacent_find(sorted.begin(), sorted.end()) != sorted.end();
+            }
+            ARE_CHECK(!dup, ARE_EINVAL, "duplicate event id within one ELT");
+            if (n) {   // the losses by quarter octave, of up to about 4096 of them
+                e.bin0 = (int32_t)(least >> 50);
+                e.bins.assign((size_t)((int32_t)(most >> 50) - e.bin0 + 1), 0u);
+                const size_t step = n / 4096 + 1;
+                for (size_t i = 0; i < n; i += step) ++e.bins[(size_t)((int32_t)(bits_of(i) >> 50) - e.bin0)];
+                e.bin_weight = (double)n / (double)((n + step - 1) / step);
+            }
+            if (no_room) std::rethrow_exception(no_room);
+            if (!buckets) {
                 copy_in(e.d_ids, event_ids, sizeof(int32_t) * n, s);
                 copy_in(e.d_loss, losses, sizeof(double) * n, s);
-            } else {   // bucketed on the device, from where the entries are if they can be read there
-                e.d_off = e.d_ids + n;
-                const int32_t *src_ids = event_ids;
-                const double *src_loss = losses;
-                if (!readable_here(ctx, event_ids, sizeof(int32_t)) || !readable_here(ctx, losses, sizeof(double))) {
-                    tmp = (char *)dalloc(ctx, tmp_bytes);
-                    copy_in(tmp, losses, sizeof(double) * n, s);
-                    copy_in(tmp + sizeof(double) * n, event_ids, sizeof(int32_t) * n, s);
-                    src_loss = reinterpret_cast<const double *>(tmp);
-                    src_ids = reinterpret_cast<const int32_t *>(src_loss + n);
-                }
-                ctx->launches += launch_bucket(src_ids, src_loss, n_entries, e.tiles, e.d_ids, e.d_loss, e.d_off,
-                                               e.d_off + e.tiles + 1, s);
             }
             ARE_CUDA_TRY(cudaStreamSynchronize(s));
         } catch (...) {
-            dfree(ctx, tmp, tmp_bytes);
+            cudaStreamSynchronize(s);   // (the device may be reading the pinned entries)
             dfree(ctx, e.d_ids, e.ids_bytes);
             dfree(ctx, e.d_loss, sizeof(double) * n);
             throw;
         }
-        dfree(ctx, tmp, tmp_bytes);
         const int32_t h = ctx->next_handle++;
         ctx->elts[h] = std::move(e);
         *elt_handle = h;

@@ -66,7 +66,7 @@ constexpr int64_t kIdPad = 64;     // zero ids after the last event (vector over
 // An ELT's entries lie in buckets, one per tile of kEltTile catalog events in
 // event order (within a bucket in any order), with the buckets' offsets,
 // where the ids stay below kMaxBucketedId (a block's shared memory counts the
-// buckets); else in the order given.
+// buckets) and the budget holds the offsets; else in the order given.
 constexpr int32_t kEltTile = 256;
 constexpr int32_t kMaxBucketedId = 48 * 1024 * kEltTile;
 struct Elt {
@@ -171,7 +171,7 @@ struct Marks {
 };
 // The shape of a catalog's marks; words 0 where more than two events would
 // share a bit.
-static_assert(2LL * 32 * kMaxMarkWords <= kMaxBucketedId, "a marked catalog's ELTs lie in buckets");
+static_assert(2LL * 32 * kMaxMarkWords <= kMaxBucketedId, "a marked catalog's ids have buckets");
 inline MarkMap mark_shape(int32_t catalog)
 {
     MarkMap m;
@@ -363,8 +363,9 @@ inline bool elts_bucketed(const ScatterArgs &a)
     return true;
 }
 // tile_rows.cu
-int launch_bucket(const int32_t *ids, const double *loss, int32_t n, int32_t tiles, int32_t *out_ids, double *out_loss,
-                  int32_t *off, int32_t *next, cudaStream_t s);
+int launch_bucket_offsets(const int32_t *ids, int32_t n, int32_t tiles, int32_t *off, cudaStream_t s);
+int launch_bucket_fill(const int32_t *ids, const double *loss, int32_t n, int32_t tiles, int32_t *out_ids,
+                       double *out_loss, int32_t *off, cudaStream_t s);
 int launch_tile_rows(const ScatterArgs &elts, int32_t catalog, bool fp32, bool packed, int words, void *rows, void *ovf,
                      const MarkMap &marks, const TermsF32 &o32, const TermsF64 &o64, cudaStream_t s);
 int launch_screen64(const SimArgs &a, int jp32, const TermsF64 &t, int num_sms, cudaStream_t s);

@@ -814,6 +814,7 @@ are_status are_submit(are_ctx *ctx, const are_request *req, int64_t *ticket)
                           t.agg_ret >= 0 && !std::isnan(t.occ_lim) && t.occ_lim >= 0 &&
                           !std::isnan(t.agg_lim) && t.agg_lim >= 0,
                       ARE_EINVAL, "bad layer terms");
+            bool bucketed = true;   // what marks are built from
             for (int32_t j = 0; j < req->n_elts; ++j) {
                 auto e = ctx->elts.find(req->elt_handles[j]);
                 ARE_CHECK(e != ctx->elts.end(), ARE_ENOTFOUND,
@@ -823,11 +824,12 @@ are_status are_submit(are_ctx *ctx, const are_request *req, int64_t *ticket)
                           ARE_EINVAL, "ELT appears twice in the request");
                 r.elts.push_back(req->elt_handles[j]);
                 r.entries += e->second.n;
+                bucketed &= e->second.n == 0 || e->second.d_off;
             }
             r.terms = positive_zeros(req->terms);
             r.bound = loss_bound(ctx, r.elts, r.terms);
-            r.marked = use_marks(S->cfg.precision, *S->y, r.bound,
-                                 marked_share(ctx, r.elts, r.terms, r.entries, S->y->catalog));
+            r.marked = bucketed && use_marks(S->cfg.precision, *S->y, r.bound,
+                                             marked_share(ctx, r.elts, r.terms, r.entries, S->y->catalog));
             for (int32_t i = 0; i < req->n_rp; ++i) {
                 r.ranks[i] = rank_for_return_period(req->n_trials, req->return_periods[i]);
                 ARE_CHECK(r.ranks[i] >= 1, ARE_EINVAL, "return period must be finite and >= 1");

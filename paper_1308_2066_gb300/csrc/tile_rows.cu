@@ -236,11 +236,14 @@ __global__ void __launch_bounds__(kTile) k_tile_rows(const __grid_constant__ Bui
 
 // An ELT's entries into buckets, one per tile of events.
 // 1. One block counts the buckets and scans the counts in its shared memory,
-//    kRead entries per thread in flight.
+//    kRead entries per thread in flight.  off[i + 1] receives where bucket i
+//    starts; with FILL (few entries) where it ends, and the block fills the
+//    buckets too.
 constexpr int kBucketThreads = 1024;
+template <bool FILL>
 __global__ void __launch_bounds__(kBucketThreads)
-    k_bucket_offsets(const int32_t *__restrict__ ids, int32_t n, int32_t tiles, int32_t *__restrict__ off,
-                     int32_t *__restrict__ next)
+    k_bucket_offsets(const int32_t *__restrict__ ids, const double *__restrict__ loss, int32_t n, int32_t tiles,
+                     int32_t *__restrict__ off, int32_t *__restrict__ out_ids, double *__restrict__ out_loss)
 {
     extern __shared__ int32_t count[];
     __shared__ int32_t sums[kBucketThreads / 32];
@@ -286,19 +289,27 @@ __global__ void __launch_bounds__(kBucketThreads)
         run += c;
     }
     __syncthreads();
-    for (int i = tid; i < tiles; i += kBucketThreads) off[i] = next[i] = count[i];
-    if (tid == 0) off[tiles] = n;
+    if constexpr (FILL) {
+        for (int32_t i = tid; i < n; i += kBucketThreads) {
+            const int32_t id = ids[i], at = atomicAdd(count + id / kEltTile, 1);
+            out_ids[at] = id;
+            out_loss[at] = loss[i];
+        }
+        __syncthreads();
+    }
+    for (int i = tid; i < tiles; i += kBucketThreads) off[i + 1] = count[i];
+    if (tid == 0) off[0] = 0;
 }
 
-// 2. The entries to their buckets.  (One block doing this too took 64 us for
-//    50,000 entries: a store of 32 scattered words occupies the SM for 32
-//    cycles.)
+// 2. The entries to their buckets, off[i + 1] counted up to where bucket i ends
+//    and the next starts.  (One block doing this too took 64 us for 50,000
+//    entries: a store of 32 scattered words occupies the SM for 32 cycles.)
 __global__ void k_bucket_fill(const int32_t *__restrict__ ids, const double *__restrict__ loss, int32_t n,
-                              int32_t *__restrict__ next, int32_t *__restrict__ out_ids, double *__restrict__ out_loss)
+                              int32_t *__restrict__ off, int32_t *__restrict__ out_ids, double *__restrict__ out_loss)
 {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const int32_t id = ids[i], at = atomicAdd(next + id / kEltTile, 1);
+    const int32_t id = ids[i], at = atomicAdd(off + 1 + id / kEltTile, 1);
     out_ids[at] = id;
     out_loss[at] = loss[i];
 }
@@ -312,17 +323,43 @@ void launch_t(const BuildArgs &a, cudaStream_t s)
 
 }  // namespace
 
-// off: tiles + 1 offsets; next: scratch for as many.
-int launch_bucket(const int32_t *ids, const double *loss, int32_t n, int32_t tiles, int32_t *out_ids, double *out_loss,
-                  int32_t *off, int32_t *next, cudaStream_t s)
+// The entries of an ELT into buckets: the offsets (off, tiles + 1 of them) once
+// the ids are at hand, then the rest; up to kFewEntries of them are both one
+// launch, the second (2000 entries in host memory load in 38 us, in two
+// launches 40; 100 entries 32 and 35).  ids and loss: device memory, or pinned
+// host memory.
+constexpr int32_t kFewEntries = 2048;
+namespace {
+template <bool FILL>
+void launch_offsets(const int32_t *ids, const double *loss, int32_t n, int32_t tiles, int32_t *off, int32_t *out_ids,
+                    double *out_loss, cudaStream_t s)
 {
     constexpr size_t most = sizeof(int32_t) * (kMaxBucketedId / kEltTile);
     static_assert(most <= 200 * 1024, "the bucket counts fit a block");
-    fit_blocks(reinterpret_cast<const void *>(k_bucket_offsets), kBucketThreads, most);   // raises the shared-memory limit
-    k_bucket_offsets<<<1, kBucketThreads, sizeof(int32_t) * (size_t)tiles, s>>>(ids, n, tiles, off, next);
-    k_bucket_fill<<<(unsigned)(((int64_t)n + 255) / 256), 256, 0, s>>>(ids, loss, n, next, out_ids, out_loss);
+    fit_blocks(reinterpret_cast<const void *>(k_bucket_offsets<FILL>), kBucketThreads, most);   // raises the limit
+    k_bucket_offsets<FILL><<<1, kBucketThreads, sizeof(int32_t) * (size_t)tiles, s>>>(ids, loss, n, tiles, off, out_ids,
+                                                                                      out_loss);
     ARE_CUDA_TRY(cudaGetLastError());
-    return 2;
+}
+}  // namespace
+
+int launch_bucket_offsets(const int32_t *ids, int32_t n, int32_t tiles, int32_t *off, cudaStream_t s)
+{
+    if (n <= kFewEntries) return 0;
+    launch_offsets<false>(ids, nullptr, n, tiles, off, nullptr, nullptr, s);
+    return 1;
+}
+
+int launch_bucket_fill(const int32_t *ids, const double *loss, int32_t n, int32_t tiles, int32_t *out_ids,
+                       double *out_loss, int32_t *off, cudaStream_t s)
+{
+    if (n <= kFewEntries) {
+        launch_offsets<true>(ids, loss, n, tiles, off, out_ids, out_loss, s);
+    } else {
+        k_bucket_fill<<<(unsigned)(((int64_t)n + 255) / 256), 256, 0, s>>>(ids, loss, n, off, out_ids, out_loss);
+        ARE_CUDA_TRY(cudaGetLastError());
+    }
+    return 1;
 }
 
 // The rows of a layer (and its marks, where marks.d is set), every ELT's
