@@ -109,9 +109,19 @@ void release_cache(are_ctx *ctx)
     ctx->cached = 0;
 }
 
+// Gives the batched selections' scratch back (they wait for their streams, so
+// none is using it between calls).
+void dfree(are_ctx *ctx, void *p, size_t bytes);
+void release_batch_scratch(are_ctx *ctx)
+{
+    dfree(ctx, ctx->sel_multi.coop, select_bytes(ctx->sel_multi.groups));
+    ctx->sel_multi = SelectScratch{};
+}
+
 void *dalloc(are_ctx *ctx, size_t bytes)
 {
     if (bytes == 0) bytes = 16;
+    if (ctx->budget && ctx->used + bytes > ctx->budget) release_batch_scratch(ctx);
     ARE_CHECK(ctx->budget == 0 || ctx->used + bytes <= ctx->budget, ARE_ENOMEM,
               "memory budget exceeded: need " + std::to_string(bytes) + " bytes, " +
                   std::to_string(ctx->budget - ctx->used) + " left");
@@ -956,6 +966,28 @@ void ensure_tables(are_ctx *ctx, const int32_t *layers, int32_t n_layers, const 
     for (int32_t i = 0; i < n_layers; ++i) ensure_direct(ctx, layer_of(ctx, layers[i]), y, p, te, s, false);
 }
 
+// The scratch of a batched selection on stream s, for up to `groups` YLTs at a
+// time: as many as the budget has room for, or else the single selection's,
+// once nothing on the device can be using that.
+SelectScratch &batch_scratch(are_ctx *ctx, int groups, cudaStream_t s)
+{
+    SelectScratch &m = ctx->sel_multi;
+    for (int g = groups; g > m.groups; g /= 2) {
+        void *d;
+        try {
+            d = dalloc(ctx, select_bytes(g));
+        } catch (const Error &e) {
+            if (e.code != ARE_ENOMEM) throw;
+            continue;
+        }
+        release_batch_scratch(ctx);
+        select_use(m, d, g, s);
+    }
+    if (m.groups) return m;
+    ARE_CUDA_TRY(cudaDeviceSynchronize());
+    return ctx->sel;
+}
+
 int max_width(are_ctx *ctx, const int32_t *layers, int32_t n_layers, bool fp32)
 {
     int jp = 0;
@@ -1058,7 +1090,7 @@ are_status are_destroy(are_ctx *ctx)
         if (ctx->h_multi) cudaFreeHost(ctx->h_multi);
         if (ctx->capture) cudaStreamDestroy(ctx->capture);
         select_free(ctx->sel);
-        select_free(ctx->sel_multi);
+        release_batch_scratch(ctx);
         if (ctx->d_flag) cudaFree(ctx->d_flag);
         if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
         if (ctx->h_result) cudaFreeHost(ctx->h_result);
@@ -2035,9 +2067,7 @@ are_status are_risk_measures_batch(are_ctx *ctx, const double *const *ylts, int3
         for (int32_t r = 0; r < n_tv; ++r) ranks.push_back(rank_level(n, tvar_levels[r]));
         if (ranks.empty()) return;
         CallStream cs(ctx, stream);
-        const size_t ptr_bytes = (sizeof(double *) * n_ylt + 255) / 256 * 256;
-        if (!ctx->sel_multi.coop) select_alloc(ctx->sel_multi, kMultiGroups);
-        const size_t need = ptr_bytes;
+        const size_t need = (sizeof(double *) * n_ylt + 255) / 256 * 256;
         if (ctx->multi_bytes < need) {
             ARE_CUDA_TRY(cudaStreamSynchronize(cs.s));
             dfree(ctx, ctx->d_multi, ctx->multi_bytes);
@@ -2054,6 +2084,7 @@ are_status are_risk_measures_batch(are_ctx *ctx, const double *const *ylts, int3
             ARE_CUDA_TRY(cudaMallocHost(&ctx->h_multi, sizeof(double) * count));
             ctx->h_multi_count = count;
         }
+        SelectScratch &scratch = batch_scratch(ctx, std::min(n_ylt, kMultiGroups), cs.s);
         const double *const *d_ptrs = static_cast<const double *const *>(ctx->d_multi);
         ARE_CUDA_TRY(cudaMemcpyAsync(ctx->d_multi, ylts, sizeof(double *) * n_ylt,
                                      cudaMemcpyHostToDevice, cs.s));
@@ -2061,7 +2092,7 @@ are_status are_risk_measures_batch(are_ctx *ctx, const double *const *ylts, int3
             const int nt = (int)std::min<size_t>(kMaxTargets, ranks.size() - b);
             const int values = std::min(std::max(n_rp - (int32_t)b, 0), nt);
             ctx->launches += launch_select_multi(d_ptrs, n_ylt, n, ranks.data() + b, nt, values, ctx->h_multi,
-                                                 ctx->sel_multi, ctx->num_sms, cs.s);   // (pinned)
+                                                 scratch, ctx->num_sms, cs.s);   // (pinned)
             ARE_CUDA_TRY(cudaStreamSynchronize(cs.s));
             for (int32_t y = 0; y < n_ylt; ++y)
                 for (int t = 0; t < nt; ++t) {

@@ -459,8 +459,10 @@ struct SelectScratch {
     int groups = 0;                 // YLTs selected at a time
     double *result = nullptr;       // single YLT, per target: value, tail mean
 };
-void select_alloc(SelectScratch &s, int groups);
-constexpr int kMultiGroups = 16;    // of the batched selection (3.5 MB)
+void select_alloc(SelectScratch &s, int groups);   // outside the budget
+size_t select_bytes(int groups);
+void select_use(SelectScratch &s, void *d, int groups, cudaStream_t st);
+constexpr int kMultiGroups = 16;    // of the batched selection (3.5 MB of the budget)
 // Ranks of the risk measures (definitions in include/are.h); -1 when the
 // return period or level is out of range.
 int64_t rank_for_return_period(int64_t n, double rp);

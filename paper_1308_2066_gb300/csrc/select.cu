@@ -997,6 +997,17 @@ CoopArgs coop_args(int64_t n, const int64_t *ranks, int nt, int n_values)
 
 }  // namespace
 
+size_t select_bytes(int groups) { return sizeof(CoopScratch) * (size_t)groups; }
+
+// s over select_bytes(groups) of device memory at d, for selections on `st`.
+void select_use(SelectScratch &s, void *d, int groups, cudaStream_t st)
+{
+    s.coop = d;
+    s.groups = groups;
+    s.result = static_cast<CoopScratch *>(d)->result;
+    ARE_CUDA_TRY(cudaMemsetAsync(d, 0, select_bytes(groups), st));
+}
+
 void select_alloc(SelectScratch &s, int groups)
 {
     ARE_CUDA_TRY(cudaMalloc(&s.coop, sizeof(CoopScratch) * (size_t)groups));

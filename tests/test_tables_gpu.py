@@ -160,3 +160,32 @@ def test_a_compact_layer_under_the_tuned_persistent_kernel(are, tmp_path, p):
             np.testing.assert_array_equal(out[are.ARE_LAYOUT_COMPACT], out[are.ARE_LAYOUT_DIRECT])
     finally:
         are.are_destroy(ctx)
+
+
+def test_the_batched_selection_within_a_budget(are):
+    """Its scratch is charged to the budget, given back to whoever needs the
+    room, and done without where there is none: the measures are the same."""
+    import torch
+    g = np.random.Generator(np.random.PCG64(8))
+    ylts = [torch.from_numpy(g.lognormal(14, 2.0, 20_000)).cuda() for _ in range(5)]
+    args = (ylts, 20_000, (100.0, 20.0), (0.99,))
+    ctx = are.are_create(0)
+    try:
+        want = are.are_risk_measures_batch(ctx, *args)
+        held = are.are_memory_used(ctx)
+        assert held > 100_000
+    finally:
+        are.are_destroy(ctx)
+    for room in (held, held // 2, 256):
+        ctx = are.are_create(0, room)
+        try:
+            for _ in range(2):
+                for a, b in zip(are.are_risk_measures_batch(ctx, *args), want):
+                    np.testing.assert_array_equal(a, b)
+                assert are.are_memory_used(ctx) <= room
+            if room > 256:     # what the scratch holds is to be had
+                are.are_load_yet(ctx, 10, 1, None, (room - 256) // 4 - 64, np.zeros((room - 256) // 4 - 64, np.int32))
+                for a, b in zip(are.are_risk_measures_batch(ctx, *args), want):
+                    np.testing.assert_array_equal(a, b)
+        finally:
+            are.are_destroy(ctx)
