@@ -507,8 +507,12 @@ __global__ void __launch_bounds__(32 * pass_warps(ACC == ARE_FP32_KAHAN, FIXED),
                 // event adds a 0, which leaves s - c as it is but may round s
                 // again (once: a second 0 changes nothing, and none does while
                 // c is 0), and so do the slots past the trial of its last
-                // batch of R groups.  Bits 0 .. 15: the pass that waited.
-                const int slots = kSlots + (cnt + 32 * R - 1) / (32 * R) * R;
+                // group of 32.  (That is the register-rows kernels' default,
+                // one group per batch.  Two pad an odd number of groups with
+                // one more 0: the same sum in another pair, whose merge may
+                // round its last bits otherwise.)  Bits 0 .. 15: the pass that
+                // waited.
+                const int slots = kSlots + ((cnt + 31) >> 5);
                 const uint32_t all = mask << kSlots | held;
                 const uint32_t skip = first - held_at - __popc(held);
                 uint32_t i = held_at;
