@@ -703,6 +703,7 @@ Folded &build_folded(are_ctx *ctx, Layer &L, int32_t catalog, cudaStream_t s)
 {
     Folded &f = L.fold;
     const int32_t words = folded_words(catalog);
+    const ScatterArgs a = scatter_args(ctx, L, catalog, 0);   // (or an id outside the catalog)
     if (f.d && f.catalog != catalog) free_folded(ctx, f);
     if (!f.d) {
         f.words = words;
@@ -710,9 +711,13 @@ Folded &build_folded(are_ctx *ctx, Layer &L, int32_t catalog, cudaStream_t s)
         f.d = dalloc(ctx, f.bytes);
         f.catalog = catalog;
     }
-    const ScatterArgs a = scatter_args(ctx, L, catalog, 0);
-    ctx->launches += launch_fold(a, L.terms.occ_ret, L.terms.occ_lim, catalog, f.F(), f.bits(),
-                                 f.hmax(), ctx->num_sms, s);
+    try {
+        ctx->launches += launch_fold(a, L.terms.occ_ret, L.terms.occ_lim, catalog, f.F(), f.bits(),
+                                     f.hmax(), ctx->num_sms, s);
+    } catch (...) {   // what is kept is built
+        free_folded(ctx, f);
+        throw;
+    }
     return f;
 }
 

@@ -189,3 +189,27 @@ def test_the_batched_selection_within_a_budget(are):
                     np.testing.assert_array_equal(a, b)
         finally:
             are.are_destroy(ctx)
+
+
+def test_a_refused_table_is_not_kept(are):
+    """A layer whose ELT holds an id outside the YET's catalog is refused each
+    time, in every form, and keeps no table."""
+    import torch
+    ctx = are.are_create(0)
+    try:
+        ids = np.array([3, 700], np.int32)
+        layer = are.are_define_layer(ctx, [are.are_load_elt(ctx, ids, np.array([5.0, 7.0]))])
+        y = are.are_load_yet(ctx, 700, 4, None, 8, np.full(32, 3, np.int32))
+        out = torch.zeros(4, dtype=torch.float64, device="cuda")
+        held = are.are_memory_used(ctx)
+        for call in (lambda: are.are_prepare_folded(ctx, layer, y),
+                     lambda: are.are_simulate_folded(ctx, layer, y, 0, 4, out),
+                     lambda: are.are_prepare(ctx, layer, y, 0), lambda: are.are_prepare(ctx, layer, y, 1),
+                     lambda: are.are_simulate(ctx, layer, y, 0, 4, 0, out),
+                     lambda: are.are_simulate(ctx, layer, y, 0, 4, 1, out)):
+            with pytest.raises(are.AreError) as e:
+                call()
+            assert e.value.status == are.ARE_EINVAL
+            assert are.are_memory_used(ctx) == held
+    finally:
+        are.are_destroy(ctx)
