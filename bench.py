@@ -212,10 +212,12 @@ def items_bytes(wl) -> int:
 
 def kernel_key(prec: int, J: int, tuned=None, rows=None, ragged=False) -> str:
     """Name of the kernel that runs the analysis stage for this precision
-    under the tuned choice (untuned: the register-rows kernels with their
-    default batch: one group of 32 events over 32-byte FP32 rows, two
-    otherwise).  rows: (row_bytes, packed) from are_layer_rows, which names
-    the packed-row instances; ragged: the YET has trials of varying length."""
+    under the tuned choice (None: register rows, every row read, with one
+    group of 32 events per batch over 32-byte FP32 rows and two otherwise;
+    the library's own default over 64-byte rows is one, so a record of an
+    untuned run names its choice: every_row_choice).  rows: (row_bytes,
+    packed) from are_layer_rows, which names the packed-row instances;
+    ragged: the YET has trials of varying length."""
     if prec == "folded":
         return "k_folded<fixed,smem_bits>"
     t = tuned or {}
@@ -250,14 +252,20 @@ def layer_rows(are, ctx, layer, yet, prec, tuned=None):
     return are.are_layer_rows(ctx, layer, yet, prec, (tuned or {}).get("kernel", -1))
 
 
+def every_row_choice(prec) -> dict:
+    """Register rows that read every occurrence's row: one group of 32 events
+    per batch, FP64 two (the library's defaults over 32-byte rows)."""
+    return {"kernel": 2, "rows_in_flight": 2 if prec == 0 else 1}
+
+
 def read_every_row(are, ctx, prec, tuned, on=True, only=True):
     """The register-rows choices of this precision over marked events (the
-    library's default form) set to read every occurrence's row, with the
-    default groups of 32 events, for one layer alone too where the choice is
-    a portfolio's; on=False: back to the default form.  only=False: all the
+    library's default form) set to read every occurrence's row
+    (every_row_choice), for one layer alone too where the choice is a
+    portfolio's; on=False: back to the default form.  only=False: all the
     precision's choices made register rows.  Returns the tuned choice as it
     then is (not timed in that form)."""
-    groups = (2 if prec == 0 else 1) if on else 0
+    groups = every_row_choice(prec)["rows_in_flight"] if on else 0
     with tempfile.TemporaryDirectory() as d:
         path = os.path.join(d, "tune.jsonl")
         are.are_tune_save(ctx, path)
@@ -279,7 +287,7 @@ def read_every_row(are, ctx, prec, tuned, on=True, only=True):
 
 
 def untuned_rows(are, ctx, layers, yet, prec, stream):
-    """Without tuning: the default register rows, every occurrence's row read."""
+    """Without tuning: register rows, every occurrence's row read."""
     choice = are.are_autotune(ctx, layers, yet, prec, stream)   # makes the entries
     read_every_row(are, ctx, prec, choice, only=False)
 
@@ -290,8 +298,9 @@ def marked_choice(tuned) -> bool:
 
 
 MARKED_WHAT = ("the library's default: one bit per catalog event, built with the table in every step, "
-               "tells which occurrences can add a loss, and only their rows are read (the same results "
-               "bit for bit); not the headline, which reads the row of every occurrence")
+               "tells which occurrences can add a loss, and only their rows are read (the same trial "
+               "losses bit for bit, but for FP32 with FP64 sums, which are exact here and round each "
+               "addition there); not the headline, which reads the row of every occurrence")
 
 
 class Resident:
@@ -456,7 +465,7 @@ def roofline(n_events, n_trials, J, prec, sim_ms, tuned=None, ceiling=None, rows
     dense_bytes = algorithmic_bytes(n_events, n_trials, J, 8 if prec == 0 else 4)
     secs = sim_ms * 1e-3
     achieved = bytes_ / secs / 1e9
-    key = kernel_key(prec, J, tuned, rows)
+    key = kernel_key(prec, J, tuned or every_row_choice(prec), rows)
     traffic = ncu_traffic(key)
     best, shapes = ceiling
     rate = n_events / secs
@@ -934,8 +943,8 @@ def precision_record(are, torch, steps, warmup, tune=True, compact=True, n_trial
             rows[PRECISION_NAMES[p]] = {
                 "sim_ms": round(ms, 4), "tuned": tuned,
                 "marked_events_sim_ms": round(ms_marked, 4) if ms_marked else None,
-                "kernel": kernel_key(p, len(L.elts), tuned, layer_rows(are, ctx, layer, yet, p, tuned),
-                                     ragged=True),
+                "kernel": kernel_key(p, len(L.elts), tuned or every_row_choice(p),
+                                     layer_rows(are, ctx, layer, yet, p, tuned), ragged=True),
                 "value": round(y.n_events * len(L.elts) / (ms * 1e-3) / 1e9, 3),
                 "ylt_rel_err_max": float(rel.max()), "ylt_rel_err_median": float(np.median(rel)),
                 "pml": [float(x) for x in pml], "pml_oracle": [float(x) for x in rp],
