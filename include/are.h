@@ -275,9 +275,9 @@ typedef struct {
  * table row, mean events per trial and one layer vs several.  Later
  * are_simulate and are_simulate_portfolio calls of that kind use it.
  * Untuned work runs the register-rows kernel in its default form: over the
- * marked events where the layer's share of them is small, else over every
- * row, with one group of 32 events per batch over 32-byte FP32 rows and two
- * over wider rows and FP64 rows.
+ * marked events where the layer's share of them is small (catalogs of up to
+ * 2,662,400 events), else over every row, with one group of 32 events per
+ * batch, or two over 32-byte FP64 rows.
  * *best (may be NULL) receives the winner.  Runs on `stream` and waits. */
 ARE_API are_status are_autotune(are_ctx *ctx, const int32_t *layers, int32_t n_layers,
                                 int32_t yet, are_precision precision, void *stream,

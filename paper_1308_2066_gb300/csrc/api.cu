@@ -577,9 +577,9 @@ double marked_share(const are_ctx *ctx, const std::vector<int32_t> &elts, const 
 
 // Whether a register-rows analysis over a YET looks its occurrences up in
 // marks first (marked.cuh), the layer's losses at most `bound` and `share` of
-// the events marked.  It depends on the layer, the
-// YET and the precision alone, so that every split of the trials, the
-// streamed analysis and the server form a trial's sum alike.
+// the events marked.  It depends on the layer, the YET and the precision
+// alone, so that every split of the trials, the streamed analysis and the
+// server form a trial's sum alike (where memory is left for the marks).
 //  * The marks of the catalog fit a block's shared memory.
 //  * FP32: losses far below the type's largest value (the exact sums hold no
 //    infinity).

@@ -610,8 +610,7 @@ __global__ void __launch_bounds__(kCoopThreads) k_select_coop(const __grid_const
     unsigned int *const over = ONE ? &K.over : args.scratch[0].over;
     // counts and counters of the scratch: past L1 in global memory
     auto get = [](const auto *x) { return ONE ? *x : __ldcg(x); };
-    auto mine = [&](int i) { return i * per + rank; };   // a block's share of the group's clearing
-    (void)mine;
+    [[maybe_unused]] auto mine = [&](int i) { return i * per + rank; };   // a block's share of the group's clearing
     for (int y0 = 0, round = 0; y0 < args.n_ylt; y0 += groups, ++round) {
         const int y = y0 + group, turn = ONE ? 0 : round & 1;
         const bool on = y < args.n_ylt;
