@@ -1240,15 +1240,17 @@ are_status are_load_elt(are_ctx *ctx, int32_t n_entries, const int32_t *event_id
             loss = pin_loss;
         }
         const bool copy = !device && pin_loss;
-        int32_t max_id = -1;
-        bool bad_id = false;
-        for (size_t i = 0; i < n; ++i) {
-            const int32_t id = ids[i];
-            if (copy) pin_ids[i] = id;
-            bad_id |= id < 0;
-            max_id = std::max(max_id, id);
+        // (copied, then looked through: one loop of both is not vectorised)
+        if (copy) {
+            for (size_t i = 0; i < n; ++i) pin_ids[i] = ids[i];
+            ids = pin_ids;
         }
-        ARE_CHECK(!bad_id, ARE_EINVAL, "negative event id in ELT");
+        int32_t max_id = -1, min_id = 0;
+        for (size_t i = 0; i < n; ++i) {
+            max_id = std::max(max_id, ids[i]);
+            min_id = std::min(min_id, ids[i]);
+        }
+        ARE_CHECK(min_id >= 0, ARE_EINVAL, "negative event id in ELT");
         Elt e;
         e.n = n_entries;
         e.max_id = max_id;

@@ -122,3 +122,25 @@ def test_elts_without_buckets(are):
     assert (out[True][0] > 0).mean() > 0.2
     for a, b in zip(out[True], out[False]):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("where", ["host", "device"])
+@pytest.mark.parametrize("nnz", [1, 1023, 1025, 2047, 2048, 2049, 3000])
+def test_every_entry_is_found(are, where, nnz):
+    """One-event trials over the catalog give the losses back, whatever the
+    order of the ids: sizes around a block's threads and its entries."""
+    import torch
+    ids, losses = elt(20 + nnz, nnz)
+    want = np.zeros(CATALOG)
+    want[ids] = losses
+    if where == "device":
+        ids, losses = torch.from_numpy(ids).cuda(), torch.from_numpy(losses).cuda()
+    ctx = are.are_create(0)
+    try:
+        layer = are.are_define_layer(ctx, [are.are_load_elt(ctx, ids, losses)])
+        y = are.are_load_yet(ctx, CATALOG, CATALOG, None, 1, np.arange(CATALOG, dtype=np.int32))
+        out = torch.full((CATALOG,), -1.0, dtype=torch.float64, device="cuda")
+        are.are_simulate(ctx, layer, y, 0, CATALOG, 0, out)
+        np.testing.assert_array_equal(out.cpu().numpy(), want)
+    finally:
+        are.are_destroy(ctx)
