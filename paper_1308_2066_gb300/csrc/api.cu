@@ -1752,16 +1752,47 @@ are_status are_pack_ids(are_ctx *ctx, const int32_t *ids, int64_t n, int32_t id_
         ARE_CHECK(id_bits >= 1 && id_bits <= 32, ARE_EINVAL, "id_bits must lie in 1 .. 32");
         ARE_CHECK(n >= 0 && (n == 0 || (ids && out)), ARE_EINVAL, "NULL array");
         ARE_CHECK(!is_device_ptr(ids) && !is_device_ptr(out), ARE_EINVAL, "ids and out must be host memory");
-        const uint64_t lim = id_bits == 32 ? (1ull << 32) : (1ull << id_bits);
+        // bits that no id may have (the sign among them)
+        const uint32_t bad = id_bits >= 31 ? 0x80000000u : ~((1u << id_bits) - 1u);
+        auto check = [&](int64_t i0, int64_t i1) {
+            for (int64_t i = i0; i < i1; ++i)
+                ARE_CHECK(!((uint32_t)ids[i] & bad), ARE_EINVAL,
+                          "id " + std::to_string(ids[i]) + " does not fit in " + std::to_string(id_bits) + " bits");
+        };
         const int64_t words = (n * id_bits + 31) / 32;
-        uint64_t acc = 0;   // bits not yet written, the lowest first
+        // 128 ids at a time: 32 ids fill id_bits whole words, so four runs of 32
+        // go side by side.  (One id after another, each checked, 200M ids of 20
+        // bits took 160 to 186 ms, as the compiler laid the loop out.)
+        int64_t i = 0;
+        for (; i + 128 <= n; i += 128) {
+            const int32_t *const v = ids + i;
+            uint32_t *o = out + i / 32 * id_bits, any = 0;
+            uint64_t acc[4] = {0, 0, 0, 0};   // bits not yet written, the lowest first
+            int have = 0;
+            for (int j = 0; j < 32; ++j) {
+                for (int g = 0; g < 4; ++g) {
+                    const uint32_t x = (uint32_t)v[32 * g + j];
+                    any |= x;
+                    acc[g] |= (uint64_t)x << have;
+                }
+                have += id_bits;
+                if (have >= 32) {
+                    for (int g = 0; g < 4; ++g) {
+                        o[g * id_bits] = (uint32_t)acc[g];
+                        acc[g] >>= 32;
+                    }
+                    ++o;
+                    have -= 32;
+                }
+            }
+            if (any & bad) check(i, i + 128);
+        }
+        check(i, n);
+        uint64_t acc = 0;
         int have = 0;
-        int64_t w = 0;
-        for (int64_t i = 0; i < n; ++i) {
-            const int32_t v = ids[i];
-            ARE_CHECK(v >= 0 && (uint64_t)v < lim, ARE_EINVAL,
-                      "id " + std::to_string(v) + " does not fit in " + std::to_string(id_bits) + " bits");
-            acc |= (uint64_t)(uint32_t)v << have;
+        int64_t w = i / 32 * id_bits;
+        for (; i < n; ++i) {
+            acc |= (uint64_t)(uint32_t)ids[i] << have;
             have += id_bits;
             if (have >= 32) {
                 out[w++] = (uint32_t)acc;
