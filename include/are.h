@@ -271,7 +271,8 @@ typedef struct {
  * (one layer: the single-layer kernels and persistent-kernel settings;
  * several: back-to-back single-layer launches, or the persistent kernel with
  * its rows in flight and trials per work item)
- * and keep the fastest for this kind of work: precision, YET layout, widest
+ * and keep the fastest (several layers: the persistent kernel where it is
+ * within 5% of it) for this kind of work: precision, YET layout, widest
  * table row, mean events per trial and one layer vs several.  Later
  * are_simulate and are_simulate_portfolio calls of that kind use it.
  * Untuned work runs the register-rows kernel in its default form: over the

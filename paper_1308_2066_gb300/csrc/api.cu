@@ -2200,7 +2200,7 @@ are_status are_autotune(are_ctx *ctx, const int32_t *layers, int32_t n_layers, i
         size_t work_bytes = 0;
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         TuneEntry win;
-        win.ms = 1e300;
+        double win_score = 1e300;
         try {
             ARE_CUDA_TRY(cudaEventCreate(&e0));
             ARE_CUDA_TRY(cudaEventCreate(&e1));
@@ -2246,7 +2246,15 @@ are_status are_autotune(are_ctx *ctx, const int32_t *layers, int32_t n_layers, i
                     best_ms = std::min(best_ms, (double)ms);
                 }
                 c.ms = best_ms;
-                if (best_ms < win.ms) win = c;
+                // A launch per layer is timed at the rate at which this host
+                // launches, which differs by some percent from run to run (12
+                // layers of 4000 trials: 99 to 102 us where the persistent
+                // launches take 97 to 99): it has to win by more than that.
+                const double score = best_ms * (multi && c.kernel != 0 ? 1.05 : 1.0);
+                if (score < win_score) {
+                    win = c;
+                    win_score = score;
+                }
             }
         } catch (...) {
             cudaStreamSynchronize(cs.s);
